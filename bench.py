@@ -457,9 +457,9 @@ def run_ours(args):
                                                        2: "tcgen05 3xtf32 coefficients"}
                        .get(stats["proj_variant"], "untuned"),
                        "fused_transform_planes_autotuned": stats["fused_planes"],
-                       "projection_gemm_tile_autotuned": {0: "64 rows", 1: "80 rows",
-                                                          2: "80 rows, half split-K",
-                                                          3: "80 rows, twice split-K"}
+                       "projection_gemm_tile_autotuned": {0: "default split-K",
+                                                          1: "half split-K", 2: "twice split-K",
+                                                          3: "four times split-K"}
                        .get(stats["gemm_shape"], "untuned"),
                        "n_deflate": int(ctx_deflate)},
             "eigenpairs_per_s": round(eigpairs, 4),

@@ -201,9 +201,8 @@ typedef struct {
   long long graph_launches;     /* CG-loop graphs launched */
   int fused_planes;             /* x-planes per group of the fused FP32 transform the
                                    autotuner chose (-1: untuned or not used) */
-  int gemm_shape;               /* tile shape of the FP64 / double-float projection GEMMs the
-                                   autotuner chose: 0 64-row tiles, 1 80-row, 2 80-row with
-                                   half the default split-K, 3 80-row with twice (-1 untuned) */
+  int gemm_shape;               /* split-K of the FP64 projection GEMMs the autotuner chose: 0 the
+                                   default, 1 half of it, 2 twice, 3 four times (-1 untuned) */
 } pdep_stats;
 
 /* Fill *opt with the defaults (FP64, cg_tol 1e-10, dav_tol 1e-8, ...). */

@@ -499,9 +499,8 @@ bool tune_done(const pdep_ctx* c, const std::string& key) {
   return it != c->tunes.end() && it->second.best >= 0;
 }
 
-// GEMM tile candidates of the projection GEMMs: tile height 64 or 80 rows,
-// split-K at the default, half or twice the default
-const GemmShape kGemmShapes[4] = {{4, 8}, {5, 8}, {5, 4}, {5, 16}};
+// split-K candidates of the FP64 projection GEMMs, in eighths of the default
+const int kGemmSplits[4] = {8, 4, 16, 32};
 std::string shape_key(const char* what, const SysData& s) {
   return std::string(what) + ":" + std::to_string(s.n_ext) + ":" + std::to_string(s.n_pw);
 }
@@ -651,15 +650,14 @@ int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list,
     R* S;
     // shift of the occupied and the deflated empty states: state w moves to
     // eps_{n_ext} - eps_v, the bottom of the spectrum the CG still sees
-    // (double-float transforms take double-float GEMMs too: FP64 matrices,
-    // arithmetic on the FP32 pipe)
+    // (after double-float transforms too; df names their profile class)
     using G = typename std::conditional<std::is_same<C, df>::value, df, R>::type;
     RET(ws(c, sizeof(R) == 8 ? "pv_64" : "pv_32", (size_t)s.n_ext * std::max(m, 1), &S));
     const R* P = psi_of(s, (R*)nullptr);
-    // tile shapes of the pair, autotuned per problem shape
-    RET(tuned_call(c, shape_key(std::is_same<G, df>::value ? "pv_df" : "pv_64", s), 4, 1, m, st,
+    // split-K of the pair, autotuned per problem shape
+    RET(tuned_call(c, shape_key(std::is_same<G, df>::value ? "pv_df" : "pv_64", s), 4, 0, m, st,
                    [&](int k) -> int {
-                     const GemmShape sh = kGemmShapes[k];
+                     const int sh = kGemmSplits[k];
                      CK(gemm<G>(true, s.n_ext, m, s.n_pw, 1.0, P, s.ld, X, s.ld, 0.0, S,
                                 s.n_ext, st, d_list, nullptr, d_count, sh));
                      CK(scale_rows<R>(S, s.n_ext, s.n_ext, m, sigma_of(s, (R*)nullptr), st));
@@ -674,14 +672,14 @@ int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list,
 // RHS split for deflation: S = Psi_ext^T B; the deflated states' part of the
 // solution is Xd = sum_c psi_c S_c,i / (eps_c - eps_v(i)) (exact, H psi_c =
 // eps_c psi_c); then B <- B - Psi_ext S leaves the part the CG solves.
-// (G: FP64, or double-float arithmetic on the FP64 matrices in the mixed modes)
+// (G: FP64, or df for the mixed modes' profile class)
 template <typename G>
 int split_rhs_t(pdep_ctx* c, SysData& s, double* B, int n, double* Xd, cudaStream_t st) {
   double* S;
   RET(ws(c, "pc_64", (size_t)s.n_ext * n, &S));
-  RET(tuned_call(c, shape_key(std::is_same<G, df>::value ? "split_df" : "split_64", s), 4, 1, n, st,
+  RET(tuned_call(c, shape_key(std::is_same<G, df>::value ? "split_df" : "split_64", s), 4, 0, n, st,
                  [&](int k) -> int {
-                   const GemmShape sh = kGemmShapes[k];
+                   const int sh = kGemmSplits[k];
                    CK(gemm<G>(true, s.n_ext, n, s.n_pw, 1.0, s.d_psi, s.ld, B, s.ld, 0.0, S,
                               s.n_ext, st, nullptr, nullptr, nullptr, sh));
                    CK(gemm<G>(false, s.n_pw, n, s.n_ext, -1.0, s.d_psi, s.ld, S, s.n_ext, 1.0, B,

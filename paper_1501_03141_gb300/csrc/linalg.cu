@@ -78,23 +78,21 @@ __device__ __forceinline__ double2 block_sum2_r(R a, R b) {
 }
 
 // ---------------------------------------------------------------------------
-// GEMM (SIMT, register-tiled 64x64x16)
+// FP32 GEMM (SIMT, register-tiled 64x64x16); FP64 is in fx_gemm.cu
 // ---------------------------------------------------------------------------
 // C tile of (16 TM) x 64 per CTA of 256 threads (16 x 16, each thread TM x 4
 // outputs), K tiles of 16 staged in shared memory.  TM = 5 gives 80-row tiles
 // for the 80-state projection coefficients (n_occ + n_deflate on the 48^3
 // workload), which 64-row tiles would cover with 37% padding.
-// R: arithmetic type (float, double, or df: double-float on FP64 matrices);
-// matrices are stored in Io<R>::T.
-template <typename R, bool TA, int TM>
-__global__ void __launch_bounds__(256) k_gemm(int m, int n, int k, R alpha,
-                                              const typename Io<R>::T* __restrict__ A,
-                                              long long lda, const typename Io<R>::T* __restrict__ B,
-                                              long long ldb, R beta, typename Io<R>::T* __restrict__ C,
-                                              long long ldc, int kchunk,
-                                              int atomic, const int* __restrict__ bmap,
+template <bool TA, int TM>
+__global__ void __launch_bounds__(256) k_gemm(int m, int n, int k, float alpha,
+                                              const float* __restrict__ A, long long lda,
+                                              const float* __restrict__ B, long long ldb,
+                                              float beta, float* __restrict__ C, long long ldc,
+                                              int kchunk, int atomic, const int* __restrict__ bmap,
                                               const int* __restrict__ cmap,
                                               const int* __restrict__ ndev, int has_beta) {
+  using R = float;
   constexpr int BM = 16 * TM, BN = 64, BK = 16;
   __shared__ R As[BK][BM + 1];
   __shared__ R Bs[BK][BN + 1];
@@ -119,11 +117,11 @@ __global__ void __launch_bounds__(256) k_gemm(int m, int n, int k, R alpha,
         // A is k x m: consecutive threads read consecutive k of one row
         const int i = e >> 4, kk = e & 15;
         const int gi = row0 + i, gk = kb + kk;
-        As[kk][i] = (gi < m && gk < kend) ? R(A[gk + (long long)gi * lda]) : R(0);
+        As[kk][i] = (gi < m && gk < kend) ? A[gk + (long long)gi * lda] : R(0);
       } else {
         const int i = e % BM, kk = e / BM;
         const int gi = row0 + i, gk = kb + kk;
-        As[kk][i] = (gi < m && gk < kend) ? R(A[gi + (long long)gk * lda]) : R(0);
+        As[kk][i] = (gi < m && gk < kend) ? A[gi + (long long)gk * lda] : R(0);
       }
     }
     {
@@ -133,7 +131,7 @@ __global__ void __launch_bounds__(256) k_gemm(int m, int n, int k, R alpha,
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int gk = kb + kk0 + q;
-        Bs[kk0 + q][j] = (gj < n && gk < kend) ? R(B[gk + bc]) : R(0);
+        Bs[kk0 + q][j] = (gj < n && gk < kend) ? B[gk + bc] : R(0);
       }
     }
     __syncthreads();
@@ -147,7 +145,7 @@ __global__ void __launch_bounds__(256) k_gemm(int m, int n, int k, R alpha,
 #pragma unroll
       for (int a = 0; a < TM; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = mad(av[a], bv[b], acc[a][b]);
+        for (int b = 0; b < 4; ++b) acc[a][b] += av[a] * bv[b];
     }
     __syncthreads();
   }
@@ -159,13 +157,13 @@ __global__ void __launch_bounds__(256) k_gemm(int m, int n, int k, R alpha,
     for (int b = 0; b < 4; ++b) {
       const int gj = col0 + ty + 16 * b;
       if (gj >= n) continue;
-      typename Io<R>::T* c = C + gi + (long long)(cmap ? cmap[gj] : gj) * ldc;
+      R* c = C + gi + (long long)(cmap ? cmap[gj] : gj) * ldc;
       if (atomic) {
-        atomicAdd(c, io_of<R>(alpha * acc[a][b]));
+        atomicAdd(c, alpha * acc[a][b]);
       } else {
         R v = alpha * acc[a][b];
-        if (has_beta) v += beta * R(*c);
-        *c = io_of<R>(v);
+        if (has_beta) v += beta * *c;
+        *c = v;
       }
     }
   }
@@ -184,75 +182,66 @@ __global__ void k_scale_mat(R* C, long long ldc, int m, int n, R beta, const int
   }
 }
 
+// FP64 matrices; R = df marks the mixed modes' products in the profile
 template <typename R>
 cudaError_t gemm(bool transA, int m, int n, int k, double alpha, const typename Io<R>::T* A,
                  long long lda, const typename Io<R>::T* B, long long ldb, double beta,
                  typename Io<R>::T* C, long long ldc, cudaStream_t st, const int* bmap,
-                 const int* cmap, const int* ndev, GemmShape shape) {
-  using T = typename Io<R>::T;
+                 const int* cmap, const int* ndev, int split_x8) {
   if (m <= 0 || n <= 0) return cudaSuccess;
-  // 80-row tiles when they pad m less than 64-row tiles do (or as tuned)
-  const bool t80 = shape.tm ? shape.tm == 5 : ((m + 79) / 80) * 80 < ((m + 63) / 64) * 64;
-  const int bm = t80 ? 80 : 64;
-  const int tm = (m + bm - 1) / bm, tn = (n + 63) / 64;
-  int splits = 1;
-  const long long tiles = (long long)tm * tn;
-  if (tiles < 2LL * num_sms() && k > 256) {
-    splits = (int)((2LL * num_sms() + tiles - 1) / tiles);
-    splits = std::min(splits, (k + 255) / 256);
-    splits = std::max(splits, 1);
-  }
-  if (shape.split_x8 > 0 && k > 256)
-    splits = std::max(1, std::min((k + 127) / 128, (splits * shape.split_x8 + 7) / 8));
-  int kchunk = (k + splits - 1) / splits;
-  kchunk = ((kchunk + 15) / 16) * 16;
-  if (kchunk == 0) kchunk = 16;
-  splits = std::max(1, (k + kchunk - 1) / kchunk);
-  if (k <= 0) splits = 1;
-  int atomic = 0;
-  if (splits > 1 || k <= 0) {
-    const long long tot = (long long)m * n;
-    const int blocks = (int)std::min<long long>((tot + 255) / 256, 4096);
-    count_launch();
-    k_scale_mat<T><<<blocks, 256, 0, st>>>(C, ldc, m, n, (T)beta, cmap, ndev);
-    if (k <= 0) return cudaGetLastError();
-    atomic = 1;
-  }
-  dim3 grid(tm, tn, splits);
-  ProfScope ps(std::is_same<R, df>::value ? PC_GEMM_DF : sizeof(R) == 8 ? PC_GEMM_F64 : PC_GEMM_F32,
-               st, 2.0 * m * n * (double)k,
-               ((double)m * k + (double)k * n + (beta != 0.0 ? 2.0 : 1.0) * m * n) * sizeof(T),
-               ndev, n);
-  count_launch();
-  const R al = R(alpha), be = R(beta);
-  const int hb = beta != 0.0 ? 1 : 0;
-  if (transA) {
-    if (t80)
-      k_gemm<R, true, 5><<<grid, 256, 0, st>>>(m, n, k, al, A, lda, B, ldb, be, C, ldc, kchunk,
-                                               atomic, bmap, cmap, ndev, hb);
-    else
-      k_gemm<R, true, 4><<<grid, 256, 0, st>>>(m, n, k, al, A, lda, B, ldb, be, C, ldc, kchunk,
-                                               atomic, bmap, cmap, ndev, hb);
+  if constexpr (sizeof(typename Io<R>::T) == 8) {
+    return gemm_fx(transA, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, num_sms(), st, bmap, cmap,
+                   ndev, split_x8, std::is_same<R, df>::value);
   } else {
-    if (t80)
-      k_gemm<R, false, 5><<<grid, 256, 0, st>>>(m, n, k, al, A, lda, B, ldb, be, C, ldc, kchunk,
-                                                atomic, bmap, cmap, ndev, hb);
-    else
-      k_gemm<R, false, 4><<<grid, 256, 0, st>>>(m, n, k, al, A, lda, B, ldb, be, C, ldc, kchunk,
-                                                atomic, bmap, cmap, ndev, hb);
+    // 80-row tiles when they pad m less than 64-row tiles do
+    const bool t80 = ((m + 79) / 80) * 80 < ((m + 63) / 64) * 64;
+    const int bm = t80 ? 80 : 64;
+    const int tm = (m + bm - 1) / bm, tn = (n + 63) / 64;
+    int splits = 1;
+    const long long tiles = (long long)tm * tn;
+    if (tiles < 2LL * num_sms() && k > 256) {
+      splits = (int)((2LL * num_sms() + tiles - 1) / tiles);
+      splits = std::min(splits, (k + 255) / 256);
+      splits = std::max(splits, 1);
+    }
+    int kchunk = (k + splits - 1) / splits;
+    kchunk = ((kchunk + 15) / 16) * 16;
+    if (kchunk == 0) kchunk = 16;
+    splits = std::max(1, (k + kchunk - 1) / kchunk);
+    if (k <= 0) splits = 1;
+    int atomic = 0;
+    if (splits > 1 || k <= 0) {
+      const long long tot = (long long)m * n;
+      const int blocks = (int)std::min<long long>((tot + 255) / 256, 4096);
+      count_launch();
+      k_scale_mat<float><<<blocks, 256, 0, st>>>(C, ldc, m, n, (float)beta, cmap, ndev);
+      if (k <= 0) return cudaGetLastError();
+      atomic = 1;
+    }
+    dim3 grid(tm, tn, splits);
+    ProfScope ps(PC_GEMM_F32, st, 2.0 * m * n * (double)k,
+                 ((double)m * k + (double)k * n + (beta != 0.0 ? 2.0 : 1.0) * m * n) * sizeof(float),
+                 ndev, n);
+    count_launch();
+    const float al = (float)alpha, be = (float)beta;
+    const int hb = beta != 0.0 ? 1 : 0;
+    auto kern = transA ? (t80 ? k_gemm<true, 5> : k_gemm<true, 4>)
+                       : (t80 ? k_gemm<false, 5> : k_gemm<false, 4>);
+    kern<<<grid, 256, 0, st>>>(m, n, k, al, A, lda, B, ldb, be, C, ldc, kchunk, atomic, bmap, cmap,
+                               ndev, hb);
+    return cudaGetLastError();
   }
-  return cudaGetLastError();
 }
 
 template cudaError_t gemm<double>(bool, int, int, int, double, const double*, long long,
                                   const double*, long long, double, double*, long long,
-                                  cudaStream_t, const int*, const int*, const int*, GemmShape);
+                                  cudaStream_t, const int*, const int*, const int*, int);
 template cudaError_t gemm<df>(bool, int, int, int, double, const double*, long long,
                               const double*, long long, double, double*, long long, cudaStream_t,
-                              const int*, const int*, const int*, GemmShape);
+                              const int*, const int*, const int*, int);
 template cudaError_t gemm<float>(bool, int, int, int, double, const float*, long long,
                                  const float*, long long, double, float*, long long, cudaStream_t,
-                                 const int*, const int*, const int*, GemmShape);
+                                 const int*, const int*, const int*, int);
 
 // ---------------------------------------------------------------------------
 // one-sided Jacobi eigensolver

@@ -15,21 +15,20 @@ namespace pdep {
 // Split over k (atomic accumulation) when the tile count is small.  Optional
 // column maps: column j of B is B[:, bmap[j]] and column j of C is C[:, cmap[j]].
 // ndev (optional): device count of the mapped columns (<= n); the launch is
-// sized for n and columns from *ndev on are left untouched.  R is the
-// arithmetic type: float, double, or df (double-float arithmetic on the FP32
-// pipe; the matrices are FP64).
-// shape (optional): tile height (tm 4: 64 rows, 5: 80 rows; 0 = the one that
-// pads m less) and split-K multiplier of the default split (split_x8 / 8,
-// 0 = default); the autotuner picks it per GEMM shape.
-struct GemmShape {
-  int tm = 0;
-  int split_x8 = 0;
-};
+// sized for n and columns from *ndev on are left untouched.  R: float, or
+// double / df on FP64 matrices, both by exact integer products on the FP16
+// tensor cores (fx_gemm.cu; df only names another profile class).
+// split_x8 (FP64; optional): split-K multiplier of the default split
+// (split_x8 / 8, 0 = default); the autotuner picks it per GEMM shape.
 template <typename R>
 cudaError_t gemm(bool transA, int m, int n, int k, double alpha, const typename Io<R>::T* A,
                  long long lda, const typename Io<R>::T* B, long long ldb, double beta,
                  typename Io<R>::T* C, long long ldc, cudaStream_t st, const int* bmap = nullptr,
-                 const int* cmap = nullptr, const int* ndev = nullptr, GemmShape shape = {});
+                 const int* cmap = nullptr, const int* ndev = nullptr, int split_x8 = 0);
+cudaError_t gemm_fx(bool transA, int m, int n, int k, double alpha, const double* A, long long lda,
+                    const double* B, long long ldb, double beta, double* C, long long ldc, int sms,
+                    cudaStream_t st, const int* bmap, const int* cmap, const int* ndev,
+                    int split_x8, bool df_class);
 
 // Symmetric eigendecomposition of the n x n matrix M (lda), FP64:
 // one-sided (Hestenes) Jacobi on M - sigma I (sigma = twice the Gershgorin

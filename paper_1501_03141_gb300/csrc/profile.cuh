@@ -22,7 +22,7 @@ enum ProfClass : int {
   PC_COLS_DF = 13,       // double-float transforms (mixed-precision refinement)
   PC_SLAB_DF = 14,
   PC_HPSI_FUSED = 15,    // FP32 H x in one launch (column scratch in shared memory)
-  PC_GEMM_DF = 16,       // double-float GEMMs (mixed-precision projections)
+  PC_GEMM_DF = 16,       // FP64 GEMMs of the mixed modes' refinement
 };
 
 // counts one kernel launch (always cheap); while this thread captures a
