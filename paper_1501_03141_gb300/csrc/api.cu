@@ -78,13 +78,11 @@ struct SysData {
   UCol* d_ucol = nullptr;
   int2* d_slot = nullptr;
   double* d_g2 = nullptr;
-  cpx<double>* d_tw64[3] = {nullptr, nullptr, nullptr};
   cpx<float>* d_tw32[3] = {nullptr, nullptr, nullptr};
-  cpx<df>* d_twdf[3] = {nullptr, nullptr, nullptr};
   double* d_v = nullptr;
   float* d_vf = nullptr;
-  df* d_vdf = nullptr;       // V(r) in double-float (refinement transforms)
-  df* d_kindf = nullptr;
+  long long* d_vfx = nullptr;  // V(r) as integers (FP64 transforms)
+  uint32_t* d_fx[3] = {nullptr, nullptr, nullptr};  // digit tables of the x-, y-, z-lines
   double* d_psi = nullptr;   // [n_occ][ld]
   float* d_psif = nullptr;
   float* d_psit5 = nullptr;  // d_psif as TF32 hi / lo tiles of the tcgen05 coefficients
@@ -99,9 +97,9 @@ struct SysData {
   float* d_kprec32 = nullptr;
   std::vector<double> eps;   // n_occ + 1
   double vmax = 0;           // max_r V(r)
+  int v_exp = 0;             // scale of d_vfx: V = d_vfx 2^v_exp
   SphereDev<double> sd{};
   SphereDev<float> sf{};
-  SphereDev<df> sdf{};
 };
 
 }  // namespace pdep
@@ -374,34 +372,26 @@ int upload_tables(pdep_ctx* c, SysData& s) {
       k64[k] = 0.5 * s.g2[k];
       k32[k] = (float)k64[k];
     }
-    std::vector<df> kdf(k64.begin(), k64.end());
     RET(persistent(c, &s.d_kin64, k64.size()));
     RET(persistent(c, &s.d_kin32, k32.size()));
-    RET(persistent(c, &s.d_kindf, kdf.size()));
     CK(cudaMemcpy(s.d_kin64, k64.data(), sizeof(double) * k64.size(), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(s.d_kin32, k32.data(), sizeof(float) * k32.size(), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(s.d_kindf, kdf.data(), sizeof(df) * kdf.size(), cudaMemcpyHostToDevice));
   }
   const double two_pi = 6.283185307179586476925286766559;
   for (int a = 0; a < 3; ++a) {
     const int N = s.N[a];
-    std::vector<cpx<double>> td(N);
     std::vector<cpx<float>> tf(N);
-    std::vector<cpx<df>> tdf(N);
     for (int j = 0; j < N; ++j) {
       double ang = two_pi * j / N;
-      td[j] = mk(cos(ang), sin(ang));
       tf[j] = mk((float)cos(ang), (float)sin(ang));
-      tdf[j] = mk(df(cos(ang)), df(sin(ang)));
     }
-    RET(persistent(c, &s.d_tw64[a], N));
     RET(persistent(c, &s.d_tw32[a], N));
-    RET(persistent(c, &s.d_twdf[a], N));
-    CK(cudaMemcpy(s.d_tw64[a], td.data(), sizeof(cpx<double>) * N, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(s.d_tw32[a], tf.data(), sizeof(cpx<float>) * N, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(s.d_twdf[a], tdf.data(), sizeof(cpx<df>) * N, cudaMemcpyHostToDevice));
+    const std::vector<uint32_t> tab = fx_line_table(N);
+    RET(persistent(c, &s.d_fx[a], tab.size()));
+    CK(cudaMemcpy(s.d_fx[a], tab.data(), sizeof(uint32_t) * tab.size(), cudaMemcpyHostToDevice));
   }
-  auto fill = [&](auto& d, auto tw) {
+  auto fill = [&](auto& d) {
     d.N1 = s.N[0];
     d.N2 = s.N[1];
     d.N3 = s.N[2];
@@ -413,29 +403,28 @@ int upload_tables(pdep_ctx* c, SysData& s) {
     d.ucol = s.d_ucol;
     d.slot = s.d_slot;
     d.g2 = s.d_g2;
-    d.tw1 = tw[0];
-    d.tw2 = tw[1];
-    d.tw3 = tw[2];
+    d.fx1 = s.d_fx[0];
+    d.fx2 = s.d_fx[1];
+    d.fx3 = s.d_fx[2];
+    d.vfx = s.d_vfx;
+    d.v_exp = s.v_exp;
 #ifdef PDEP_BOUNDS_CHECK
     d.status = c->d_status;
 #endif
   };
-  fill(s.sd, s.d_tw64);
-  fill(s.sf, s.d_tw32);
-  fill(s.sdf, s.d_twdf);
+  fill(s.sd);
+  fill(s.sf);
   s.sd.kin = s.d_kin64;
   s.sf.kin = s.d_kin32;
-  s.sdf.kin = s.d_kindf;
+  s.sf.tw1 = s.d_tw32[0];
+  s.sf.tw2 = s.d_tw32[1];
+  s.sf.tw3 = s.d_tw32[2];
   return PDEP_OK;
 }
 
 // precision selectors
 inline const SphereDev<double>& sph(const SysData& s, double*) { return s.sd; }
 inline const SphereDev<float>& sph(const SysData& s, float*) { return s.sf; }
-inline const SphereDev<df>& sph(const SysData& s, df*) { return s.sdf; }
-inline const double* vgrid(const SysData& s, double*) { return s.d_v; }
-inline const float* vgrid(const SysData& s, float*) { return s.d_vf; }
-inline const df* vgrid(const SysData& s, df*) { return s.d_vdf; }
 inline const double* psi_of(const SysData& s, double*) { return s.d_psi; }
 inline const float* psi_of(const SysData& s, float*) { return s.d_psif; }
 inline const double* kprec_of(const SysData& s, double*) { return s.d_kprec64; }
@@ -507,13 +496,14 @@ std::string shape_key(const char* what, const SysData& s) {
 
 // d_count (with d_list): device length of the list; n_list is then the
 // largest length, which sizes the launches (kernels read the count).
-// C is the arithmetic type of the transforms (float, double, or df: double-
-// float on FP32 vectors... on FP64 vectors); the vectors and the projection
-// term use its storage type R (FP64 for df).
-template <typename C, typename R = typename Io<C>::T>
+// R: FP32 or FP64.  refine (FP64): the product of a mixed-mode refinement, whose
+// transforms take seven digits (far below the FP32 inner solve's needs and
+// above double-float).
+template <typename R>
 int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list, int n_list,
             bool with_shift, bool with_pv, cudaStream_t st, double* dn = nullptr,
-            const int* d_count = nullptr) {
+            const int* d_count = nullptr, bool refine = false) {
+  const int digits = refine ? 7 : 8;
   ItemMap map{n, (n + 1) / 2};
   int n_items = (n + 1) / 2;
   if (d_list) {
@@ -523,7 +513,7 @@ int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list,
     n_items = (n_list + 1) / 2;
   }
   bool fused = false;
-  if constexpr (std::is_same<C, float>::value) {
+  if constexpr (std::is_same<R, float>::value) {
     // FP32 on 24^3 .. 48^3: the whole transform in one launch, the column
     // scratch in shared memory
     if (n_items > 0 && !dn && c->opt.fused_hpsi && hpsi_fused_smem(s.sf) > 0) {
@@ -552,15 +542,13 @@ int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list,
     }
   }
   if (n_items > 0 && !fused) {
-    cpx<C>* b1;   // double-float shares the FP64 scratch (16 bytes per complex)
-    RET(ws(c, sizeof(C) == 8 ? "b1_64" : "b1_32", b1_count(s, n_items), &b1));
-    const SphereDev<C>& sd = sph(s, (C*)nullptr);
-    CK(launch_cols_fwd<C>(sd, X, s.ld, map, n_items, COEF_ONE, b1, st));
-    SlabArgs<C> a{};
+    cpx<R>* b1;
+    RET(ws(c, sizeof(R) == 8 ? "b1_64" : "b1_32", b1_count(s, n_items), &b1));
+    const SphereDev<R>& sd = sph(s, (R*)nullptr);
+    SlabArgs<R> a{};
     a.mode = SLAB_HPSI;
     a.b1 = b1;
     a.n_items = n_items;
-    a.v = vgrid(s, (C*)nullptr);
     a.map = map;
     if (dn) {
       a.dn = dn;
@@ -569,19 +557,28 @@ int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list,
       a.dn_stride = s.n_r;
       a.dn_scale = 4.0 / s.omega;
     }
-    CK(launch_slab<C>(sd, a, st));
-    Epilogue<C> ep{};
+    Epilogue<R> ep{};
     ep.y = Y;
     ep.ldy = s.ld;
     ep.x_in = X;
     ep.ldx = s.ld;
     ep.shift = with_shift ? negeps_of(s, (R*)nullptr) : nullptr;
     ep.shift_period = with_shift ? s.n_occ : 1;
-    ep.scale = C(1.0 / s.n_r);
-    ep.kin = C(1);
+    ep.scale = R(1.0 / s.n_r);
+    ep.kin = R(1);
     ep.beta = R(0);
     ep.coef = COEF_ONE;
-    CK(launch_cols_bwd<C>(sd, b1, map, n_items, ep, st));
+    if constexpr (std::is_same<R, float>::value) {
+      a.v = s.d_vf;
+      CK(launch_cols_fwd(sd, X, s.ld, map, n_items, COEF_ONE, b1, st));
+      CK(launch_slab(sd, a, st));
+      CK(launch_cols_bwd(sd, b1, map, n_items, ep, st));
+    } else {
+      a.digits = digits;
+      CK(launch_cols_fwd(sd, X, s.ld, map, n_items, COEF_ONE, b1, st, digits));
+      CK(launch_slab(sd, a, st));
+      CK(launch_cols_bwd(sd, b1, map, n_items, ep, st, digits));
+    }
   }
   if (with_pv) {
     // only the listed columns when a list is given
@@ -650,19 +647,17 @@ int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list,
     R* S;
     // shift of the occupied and the deflated empty states: state w moves to
     // eps_{n_ext} - eps_v, the bottom of the spectrum the CG still sees
-    // (after double-float transforms too; df names their profile class)
-    using G = typename std::conditional<std::is_same<C, df>::value, df, R>::type;
     RET(ws(c, sizeof(R) == 8 ? "pv_64" : "pv_32", (size_t)s.n_ext * std::max(m, 1), &S));
     const R* P = psi_of(s, (R*)nullptr);
     // split-K of the pair, autotuned per problem shape
-    RET(tuned_call(c, shape_key(std::is_same<G, df>::value ? "pv_df" : "pv_64", s), 4, 0, m, st,
+    RET(tuned_call(c, shape_key("pv_64", s), 4, 0, m, st,
                    [&](int k) -> int {
                      const int sh = kGemmSplits[k];
-                     CK(gemm<G>(true, s.n_ext, m, s.n_pw, 1.0, P, s.ld, X, s.ld, 0.0, S,
-                                s.n_ext, st, d_list, nullptr, d_count, sh));
+                     CK(gemm<R>(true, s.n_ext, m, s.n_pw, 1.0, P, s.ld, X, s.ld, 0.0, S,
+                                s.n_ext, st, d_list, nullptr, d_count, sh, refine));
                      CK(scale_rows<R>(S, s.n_ext, s.n_ext, m, sigma_of(s, (R*)nullptr), st));
-                     CK(gemm<G>(false, s.n_pw, m, s.n_ext, 1.0, P, s.ld, S, s.n_ext, 1.0, Y, s.ld,
-                                st, nullptr, d_list, d_count, sh));
+                     CK(gemm<R>(false, s.n_pw, m, s.n_ext, 1.0, P, s.ld, S, s.n_ext, 1.0, Y, s.ld,
+                                st, nullptr, d_list, d_count, sh, refine));
                      return PDEP_OK;
                    }));
   }
@@ -672,31 +667,24 @@ int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list,
 // RHS split for deflation: S = Psi_ext^T B; the deflated states' part of the
 // solution is Xd = sum_c psi_c S_c,i / (eps_c - eps_v(i)) (exact, H psi_c =
 // eps_c psi_c); then B <- B - Psi_ext S leaves the part the CG solves.
-// (G: FP64, or df for the mixed modes' profile class)
-template <typename G>
-int split_rhs_t(pdep_ctx* c, SysData& s, double* B, int n, double* Xd, cudaStream_t st) {
+int split_rhs(pdep_ctx* c, SysData& s, double* B, int n, double* Xd, cudaStream_t st) {
+  const bool mixed = c->opt.precision != PDEP_FP64;
   double* S;
   RET(ws(c, "pc_64", (size_t)s.n_ext * n, &S));
-  RET(tuned_call(c, shape_key(std::is_same<G, df>::value ? "split_df" : "split_64", s), 4, 0, n, st,
-                 [&](int k) -> int {
-                   const int sh = kGemmSplits[k];
-                   CK(gemm<G>(true, s.n_ext, n, s.n_pw, 1.0, s.d_psi, s.ld, B, s.ld, 0.0, S,
-                              s.n_ext, st, nullptr, nullptr, nullptr, sh));
-                   CK(gemm<G>(false, s.n_pw, n, s.n_ext, -1.0, s.d_psi, s.ld, S, s.n_ext, 1.0, B,
-                              s.ld, st, nullptr, nullptr, nullptr, sh));
-                   return PDEP_OK;
-                 }));
+  RET(tuned_call(c, shape_key("split_64", s), 4, 0, n, st, [&](int k) -> int {
+    const int sh = kGemmSplits[k];
+    CK(gemm<double>(true, s.n_ext, n, s.n_pw, 1.0, s.d_psi, s.ld, B, s.ld, 0.0, S, s.n_ext, st,
+                    nullptr, nullptr, nullptr, sh, mixed));
+    CK(gemm<double>(false, s.n_pw, n, s.n_ext, -1.0, s.d_psi, s.ld, S, s.n_ext, 1.0, B, s.ld, st,
+                    nullptr, nullptr, nullptr, sh, mixed));
+    return PDEP_OK;
+  }));
   if (s.n_defl > 0) {
     CK(deflation_coefficients(S, s.n_ext, s.n_occ, s.n_defl, n, s.d_eps_ext, st));
-    CK(gemm<G>(false, s.n_pw, n, s.n_defl, 1.0, s.d_psi + (size_t)s.n_occ * s.ld, s.ld,
-               S + s.n_occ, s.n_ext, 0.0, Xd, s.ld, st));
+    CK(gemm<double>(false, s.n_pw, n, s.n_defl, 1.0, s.d_psi + (size_t)s.n_occ * s.ld, s.ld,
+                    S + s.n_occ, s.n_ext, 0.0, Xd, s.ld, st, nullptr, nullptr, nullptr, 0, mixed));
   }
   return PDEP_OK;
-}
-int split_rhs(pdep_ctx* c, SysData& s, double* B, int n, double* Xd, cudaStream_t st) {
-  if (c->opt.precision != PDEP_FP64 && c->opt.df_refine)
-    return split_rhs_t<df>(c, s, B, n, Xd, st);
-  return split_rhs_t<double>(c, s, B, n, Xd, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -1079,7 +1067,7 @@ int setup_states(pdep_ctx* c, SysData& s, cudaStream_t st) {
     const int n_items = (nocc + 1) / 2;
     cpx<double>* b1;
     RET(ws(c, "b1_64", b1_count(s, n_items), &b1));
-    CK(launch_cols_fwd<double>(s.sd, s.d_psi, s.ld, map, n_items, COEF_ONE, b1, st));
+    CK(launch_cols_fwd(s.sd, s.d_psi, s.ld, map, n_items, COEF_ONE, b1, st));
     SlabArgs<double> a{};
     a.mode = SLAB_TO_GRID;
     a.b1 = b1;
@@ -1088,7 +1076,7 @@ int setup_states(pdep_ctx* c, SysData& s, cudaStream_t st) {
     a.out_stride = s.n_r;
     a.out_scale = 1.0;
     a.map = map;
-    CK(launch_slab<double>(s.sd, a, st));
+    CK(launch_slab(s.sd, a, st));
   }
   RET(sync(st));
   return PDEP_OK;
@@ -1424,10 +1412,8 @@ int refine_rounds(pdep_ctx* c, SysData& s, const double* b, const double* xd, do
                          n_un));
       continue;
     }
-    if (!fp64 && c->opt.df_refine)
-      RET(apply_h<df>(c, s, dl, ad, n, list, n, true, true, st, dn, n_un));
-    else
-      RET(apply_h<double>(c, s, dl, ad, n, list, n, true, true, st, dn, n_un));
+    RET(apply_h<double>(c, s, dl, ad, n, list, n, true, true, st, dn, n_un,
+                        !fp64 && c->opt.df_refine));
     CK(residual_update(r64, ad, b, s.ld, s.n_pw, n, rel, list, xr, s.d_sigma64, s.n_occ, st,
                        n_un));
   }
@@ -1470,17 +1456,17 @@ int solve_rhs(pdep_ctx* c, SysData& s, const double* b, const double* xd, double
 // and xdefl [m*n_occ][ld] receives their exact share of the solution.
 // occupied_only: bvec = -P_c [dV_j psi_v] with P_c over the occupied states
 // alone (no deflation split; xdefl unused).
-// The products dV_j psi_v and their transforms to the sphere (C: FP64, or
-// double-float in the mixed modes; vectors FP64 either way).
-template <typename C>
-int rhs_transform(pdep_ctx* c, SysData& s, const double* dv, int m, double* bvec,
+// The products dV_j psi_v and their transforms to the sphere (digits: eight, or
+// seven in the mixed modes).
+int rhs_transform(pdep_ctx* c, SysData& s, const double* dv, int m, double* bvec, int digits,
                   cudaStream_t st) {
   const int nocc = s.n_occ;
   ItemMap map{nocc, (nocc + 1) / 2};
   const int n_items = m * ((nocc + 1) / 2);
-  cpx<C>* b1;
+  cpx<double>* b1;
   RET(ws(c, "b1_64", b1_count(s, n_items), &b1));
-  SlabArgs<C> a{};
+  SlabArgs<double> a{};
+  a.digits = digits;
   a.mode = SLAB_FROM_GRID;
   a.b1 = b1;
   a.n_items = n_items;
@@ -1489,25 +1475,22 @@ int rhs_transform(pdep_ctx* c, SysData& s, const double* dv, int m, double* bvec
   a.src.g = s.d_u;
   a.src.g_stride = s.n_r;
   a.map = map;
-  const SphereDev<C>& sd = sph(s, (C*)nullptr);
-  CK(launch_slab<C>(sd, a, st));
-  Epilogue<C> ep{};
+  CK(launch_slab(s.sd, a, st));
+  Epilogue<double> ep{};
   ep.y = bvec;
   ep.ldy = s.ld;
   ep.shift_period = 1;
-  ep.scale = C(-1.0 / s.n_r);
+  ep.scale = -1.0 / s.n_r;
   ep.coef = COEF_ONE;
-  CK(launch_cols_bwd<C>(sd, b1, map, n_items, ep, st));
+  CK(launch_cols_bwd(s.sd, b1, map, n_items, ep, st, digits));
   return PDEP_OK;
 }
 
 int build_rhs(pdep_ctx* c, SysData& s, const double* dv, int m, double* bvec, double* xdefl,
               cudaStream_t st, bool occupied_only = false) {
   const int nocc = s.n_occ;
-  if (c->opt.precision != PDEP_FP64 && c->opt.df_refine)
-    RET(rhs_transform<df>(c, s, dv, m, bvec, st));
-  else
-    RET(rhs_transform<double>(c, s, dv, m, bvec, st));
+  RET(rhs_transform(c, s, dv, m, bvec, c->opt.precision != PDEP_FP64 && c->opt.df_refine ? 7 : 8,
+                    st));
   if (occupied_only) {
     double* S;
     RET(ws(c, "po_S", (size_t)nocc * m * nocc, &S));
@@ -1528,7 +1511,7 @@ int perturbation_grids(pdep_ctx* c, SysData& s, const double* phi, int m, double
   const int n_items = (m + 1) / 2;
   cpx<double>* b1;
   RET(ws(c, "b1_64", b1_count(s, n_items), &b1));
-  CK(launch_cols_fwd<double>(s.sd, phi, s.ld, map, n_items, COEF_SQRT_COULOMB, b1, st));
+  CK(launch_cols_fwd(s.sd, phi, s.ld, map, n_items, COEF_SQRT_COULOMB, b1, st));
   SlabArgs<double> a{};
   a.mode = SLAB_TO_GRID;
   a.b1 = b1;
@@ -1537,7 +1520,7 @@ int perturbation_grids(pdep_ctx* c, SysData& s, const double* phi, int m, double
   a.out_stride = s.n_r;
   a.out_scale = 1.0 / std::sqrt(s.omega);
   a.map = map;
-  CK(launch_slab<double>(s.sd, a, st));
+  CK(launch_slab(s.sd, a, st));
   return PDEP_OK;
 }
 
@@ -1587,14 +1570,14 @@ int chi0_internal(pdep_ctx* c, SysData& s, const double* phi, int m, double* out
       a.src.g = dn;
       a.src.g_stride = s.n_r;
       a.map = map;
-      CK(launch_slab<double>(s.sd, a, st));
+      CK(launch_slab(s.sd, a, st));
       Epilogue<double> ep{};
       ep.y = out + (size_t)j0 * s.ld;
       ep.ldy = s.ld;
       ep.shift_period = 1;
       ep.scale = std::sqrt(s.omega) / s.n_r;
       ep.coef = COEF_SQRT_COULOMB;
-      CK(launch_cols_bwd<double>(s.sd, b1, map, n_items, ep, st));
+      CK(launch_cols_bwd(s.sd, b1, map, n_items, ep, st));
     }
   }
   return PDEP_OK;
@@ -1701,13 +1684,11 @@ int solve_one(pdep_ctx* c, int si, const double* phi0, double* eigvals, double* 
 }  // namespace
 
 namespace pdep {
-// Sphere description and potential of one system for pdep_apply_hamiltonian_noalloc.
-int noalloc_sphere(pdep_ctx* c, int sys, SphereDev<double>* sd, const double** v, int* n_pw,
-                   int* device) {
+// Sphere description of one system for pdep_apply_hamiltonian_noalloc.
+int noalloc_sphere(pdep_ctx* c, int sys, SphereDev<double>* sd, int* n_pw, int* device) {
   RET(check_sys(c, sys));
   const SysData& s = c->sys[sys];
   *sd = s.sd;
-  *v = s.d_v;
   *n_pw = s.n_pw;
   *device = c->device;
   return PDEP_OK;
@@ -1908,15 +1889,12 @@ int pdep_setup(const pdep_system_desc* sys, int n_sys, const pdep_options* opt, 
     if (s.n_pdep > s.n_pw - 1) return bail(fail(PDEP_ERR_INVALID_ARG, "n_pdep too large"));
     const size_t smem = slab_smem_bytes(s.n_col, s.R3, s.N[1], sizeof(double));
     if (smem > 200 * 1024) return bail(fail(PDEP_ERR_UNSUPPORTED, "slab does not fit shared memory"));
-    r = upload_tables(c, s);
-    if (r != PDEP_OK) return bail(r);
     if ((r = persistent(c, &s.d_v, s.n_r)) != PDEP_OK) return bail(r);
     if ((r = persistent(c, &s.d_vf, s.n_r)) != PDEP_OK) return bail(r);
-    if ((r = persistent(c, &s.d_vdf, s.n_r)) != PDEP_OK) return bail(r);
+    if ((r = persistent(c, &s.d_vfx, s.n_r)) != PDEP_OK) return bail(r);
     if (cudaMemcpyAsync(s.d_v, d.v_r, sizeof(double) * s.n_r, kind_to_dev(d.v_r), st) != cudaSuccess)
       return bail(fail(PDEP_ERR_CUDA, "potential upload"));
-    if (convert<float, double>(s.d_vf, s.n_r, s.d_v, s.n_r, s.n_r, 1, st) != cudaSuccess ||
-        convert<df, double>(s.d_vdf, s.n_r, s.d_v, s.n_r, s.n_r, 1, st) != cudaSuccess)
+    if (convert<float, double>(s.d_vf, s.n_r, s.d_v, s.n_r, s.n_r, 1, st) != cudaSuccess)
       return bail(fail(PDEP_ERR_CUDA, "potential conversion"));
     // the potential must be finite
     std::vector<double> hv(s.n_r);
@@ -1925,10 +1903,20 @@ int pdep_setup(const pdep_system_desc* sys, int n_sys, const pdep_options* opt, 
         cudaStreamSynchronize(st) != cudaSuccess)
       return bail(fail(PDEP_ERR_CUDA, "potential check"));
     s.vmax = -1e300;
+    double vabs = 0.0;
     for (double v : hv) {
       if (!std::isfinite(v)) return bail(fail(PDEP_ERR_NONFINITE, "non-finite potential"));
       s.vmax = std::max(s.vmax, v);
+      vabs = std::max(vabs, std::fabs(v));
     }
+    unsigned long long vbits;
+    memcpy(&vbits, &vabs, sizeof(vbits));
+    const int er = std::max(1, (int)(vbits >> 52));
+    s.v_exp = er - 1084;
+    if (fixed_potential(s.d_v, s.n_r, er, s.d_vfx, st) != cudaSuccess)
+      return bail(fail(PDEP_ERR_CUDA, "potential conversion"));
+    r = upload_tables(c, s);
+    if (r != PDEP_OK) return bail(r);
     r = setup_states(c, s, st);
     if (r != PDEP_OK) return bail(r);
     if ((r = check_status(c, st)) != PDEP_OK) return bail(r);
@@ -2366,7 +2354,7 @@ int pdep_apply_hamiltonian(pdep_ctx* c, int sys, const double* x, int n, double*
   if (precision == PDEP_FP64) {
     RET(apply_h<double>(c, s, in, outv, n, nullptr, 0, false, false, st));
   } else if (precision == PDEP_APPLY_DF64) {
-    RET(apply_h<df>(c, s, in, outv, n, nullptr, 0, false, false, st));
+    RET(apply_h<double>(c, s, in, outv, n, nullptr, 0, false, false, st, nullptr, nullptr, true));
   } else {
     float *in32, *out32;
     RET(ws(c, "api_in32", (size_t)n * s.ld, &in32));
@@ -2396,7 +2384,7 @@ int pdep_to_grid(pdep_ctx* c, int sys, const double* x, int n, double* u, void* 
   const int n_items = (n + 1) / 2;
   cpx<double>* b1;
   RET(ws(c, "b1_64", b1_count(s, n_items), &b1));
-  CK(launch_cols_fwd<double>(s.sd, in, s.ld, map, n_items, COEF_ONE, b1, st));
+  CK(launch_cols_fwd(s.sd, in, s.ld, map, n_items, COEF_ONE, b1, st));
   SlabArgs<double> a{};
   a.mode = SLAB_TO_GRID;
   a.b1 = b1;
@@ -2405,7 +2393,7 @@ int pdep_to_grid(pdep_ctx* c, int sys, const double* x, int n, double* u, void* 
   a.out_stride = s.n_r;
   a.out_scale = 1.0;
   a.map = map;
-  CK(launch_slab<double>(s.sd, a, st));
+  CK(launch_slab(s.sd, a, st));
   CK(cudaMemcpyAsync(u, grid, sizeof(double) * (size_t)n * s.n_r, kind_from_dev(u), st));
   return sync(st);
 }

@@ -17,10 +17,7 @@
 // unnormalised), S = -1 the forward transform (grid -> sphere).
 #pragma once
 
-#include <type_traits>
-
 #include "common.cuh"
-#include "df64.cuh"
 
 namespace pdep {
 
@@ -34,19 +31,10 @@ __host__ __device__ constexpr int local_tw_offset(int M) {
 constexpr int LOCAL_TW_SIZE = 240;
 
 // defined here: fft.cuh is included by a single translation unit (no -rdc)
-__constant__ double2 c_local_tw_d[LOCAL_TW_SIZE];
 __constant__ float2 c_local_tw_f[LOCAL_TW_SIZE];
-__constant__ float4 c_local_tw_df[LOCAL_TW_SIZE];  // (re.hi, re.lo, im.hi, im.lo)
 
 template <typename R>
 struct LocalTw;
-template <>
-struct LocalTw<double> {
-  static __device__ __forceinline__ cpx<double> get(int i) {
-    double2 v = c_local_tw_d[i];
-    return mk(v.x, v.y);
-  }
-};
 template <>
 struct LocalTw<float> {
   static __device__ __forceinline__ cpx<float> get(int i) {
@@ -54,14 +42,6 @@ struct LocalTw<float> {
     return mk(v.x, v.y);
   }
 };
-template <>
-struct LocalTw<df> {
-  static __device__ __forceinline__ cpx<df> get(int i) {
-    float4 v = c_local_tw_df[i];
-    return mk(df(v.x, v.y), df(v.z, v.w));
-  }
-};
-
 // exp(S * 2 pi i j / M) for the local DFT of size M
 template <typename R, int S, int M>
 __device__ __forceinline__ cpx<R> local_w(int j) {
@@ -179,31 +159,18 @@ __device__ __forceinline__ int bitrev(int t, int bits) {
 template <typename R, int S>
 __device__ __forceinline__ cpx<R> table_w(const cpx<R>* __restrict__ tw, int j) {
   cpx<R> w;
-  if constexpr (std::is_same<R, df>::value) {
-    // double-float: one 16-byte load of (re.hi, re.lo, im.hi, im.lo)
-    const float4 v = __ldg(reinterpret_cast<const float4*>(tw + j));
-    w = mk(R(v.x, v.y), R(v.z, v.w));
-  } else {
-    w.x = __ldg(&tw[j].x);
-    w.y = __ldg(&tw[j].y);
-  }
+  w.x = __ldg(&tw[j].x);
+  w.y = __ldg(&tw[j].y);
   return S > 0 ? w : conj(w);
 }
 
 // p + v (lower lane of a butterfly) or p - v (upper lane): one fused
-// multiply-add per component in FP32 / FP64, a sign flip and one addition in
-// double-float
+// multiply-add per component
 template <typename R>
 __device__ __forceinline__ cpx<R> pm(cpx<R> p, cpx<R> v, bool up) {
   const R sgn = up ? R(-1) : R(1);
   return mk(p.x + sgn * v.x, p.y + sgn * v.y);
 }
-template <>
-__device__ __forceinline__ cpx<df> pm<df>(cpx<df> p, cpx<df> v, bool up) {
-  const cpx<df> w = up ? mk(-v.x, -v.y) : v;
-  return mk(p.x + w.x, p.y + w.y);
-}
-
 // Twiddle sources of the cross-lane line FFTs.  TableTw reads e^{2 pi i j/N}
 // from the global table per use; RegTw holds, for one lane position t, the
 // M twiddles w^{t k2} and the twiddles of the cross-lane stages with span

@@ -32,13 +32,13 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "fx.cuh"
 #include "linalg.cuh"
 #include "profile.cuh"
 
 namespace pdep {
 namespace {
 
-constexpr int FX_S = 8;                       // digits per operand
 constexpr int FX_BM = 32, FX_BN = 32;         // CTA tile, four warps of 16 x 16
 constexpr int FX_KS = 32;                     // k-values per stage (and per exact accumulation)
 constexpr int FX_THREADS = 128;
@@ -49,54 +49,12 @@ constexpr int FX_LD = 40;
 constexpr int FX_SMEM = FX_S * FX_ROWS * FX_LD * 2;
 // K range of one CTA: the high sum stays below 2^51 (2^38 per k-value)
 constexpr int FX_KMAX = 4096;
-constexpr uint32_t FX_MAGIC = 0x4B400000u;    // bits of 1.5 * 2^23
-
-__device__ __forceinline__ int exp_of(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
-
-// x as a 63-bit fixed-point number scaled by its row's exponent field er
-// (>= 1 and >= that of x): x = v 2^(er - 1084)
-__device__ __forceinline__ long long fx_of(double x, int er) {
-  const int hi = __double2hiint(x);
-  const int e = (hi >> 20) & 0x7ff;
-  unsigned long long m =
-      ((unsigned long long)(unsigned)((hi & 0xfffff) | (e ? 0x100000 : 0)) << 32) |
-      (unsigned)__double2loint(x);
-  const int sh = er - (e > 1 ? e : 1);
-  m = sh < 64 ? (m << 9) >> sh : 0ull;
-  return hi < 0 ? -(long long)m : (long long)m;
-}
-
-// digit s (0 = most significant) of two biased fixed-point numbers as a pair
-// of FP16 integers: the bytes go into the mantissas of 1024 + byte, then
-// 1024 + 128 is subtracted (all exact)
-__device__ __forceinline__ uint32_t digit_pair(uint2 u0, uint2 u1, int s) {
-  const uint32_t w0 = s < 4 ? u0.y : u0.x, w1 = s < 4 ? u1.y : u1.x;
-  const int j = 3 - (s & 3);
-  uint32_t p = __byte_perm(w0, w1, (uint32_t)(j | (4 + j) << 8));
-  p = (p & 0x00ff00ffu) | 0x64006400u;
-  uint32_t r;
-  asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(p), "r"(0xE480E480u));
-  return r;
-}
-__device__ __forceinline__ uint2 biased(long long v) {
-  const unsigned long long u = (unsigned long long)v + 0x8080808080808080ull;
-  return make_uint2((uint32_t)u, (uint32_t)(u >> 32));
-}
 
 __device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(addr));
 }
-__device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
-                                        uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
 // (hi 2^-24 + lo 2^-56) 2^q2 rounded to FP64 (integer arithmetic: the FP64
 // pipe would take as long for this as the tensor cores for the products)
 __device__ __forceinline__ double fx_result(long long hi, long long lo, int q2) {
@@ -317,7 +275,7 @@ __global__ void k_scale_fx(double* C, long long ldc, int m, int n, double beta, 
 cudaError_t gemm_fx(bool transA, int m, int n, int k, double alpha, const double* A, long long lda,
                     const double* B, long long ldb, double beta, double* C, long long ldc, int sms,
                     cudaStream_t st, const int* bmap, const int* cmap, const int* ndev,
-                    int split_x8, bool df_class) {
+                    int split_x8, bool mixed) {
   const int tm = (m + FX_BM - 1) / FX_BM, tn = (n + FX_BN - 1) / FX_BN;
   const long long tiles = (long long)tm * tn;
   // about three resident CTAs per SM, at least four stages each
@@ -341,7 +299,7 @@ cudaError_t gemm_fx(bool transA, int m, int n, int k, double alpha, const double
   }
   dim3 grid(tm, tn, splits);
   if (tn > 65535 || splits > 65535) return cudaErrorInvalidValue;
-  ProfScope ps(df_class ? PC_GEMM_DF : PC_GEMM_F64, st, 2.0 * m * n * (double)k,
+  ProfScope ps(mixed ? PC_GEMM_DF : PC_GEMM_F64, st, 2.0 * m * n * (double)k,
                ((double)m * k + (double)k * n + (beta != 0.0 ? 2.0 : 1.0) * m * n) * sizeof(double),
                ndev, n);
   count_launch();

@@ -182,16 +182,15 @@ __global__ void k_scale_mat(R* C, long long ldc, int m, int n, R beta, const int
   }
 }
 
-// FP64 matrices; R = df marks the mixed modes' products in the profile
 template <typename R>
-cudaError_t gemm(bool transA, int m, int n, int k, double alpha, const typename Io<R>::T* A,
-                 long long lda, const typename Io<R>::T* B, long long ldb, double beta,
-                 typename Io<R>::T* C, long long ldc, cudaStream_t st, const int* bmap,
-                 const int* cmap, const int* ndev, int split_x8) {
+cudaError_t gemm(bool transA, int m, int n, int k, double alpha, const R* A,
+                 long long lda, const R* B, long long ldb, double beta,
+                 R* C, long long ldc, cudaStream_t st, const int* bmap,
+                 const int* cmap, const int* ndev, int split_x8, bool mixed) {
   if (m <= 0 || n <= 0) return cudaSuccess;
-  if constexpr (sizeof(typename Io<R>::T) == 8) {
+  if constexpr (sizeof(R) == 8) {
     return gemm_fx(transA, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, num_sms(), st, bmap, cmap,
-                   ndev, split_x8, std::is_same<R, df>::value);
+                   ndev, split_x8, mixed);
   } else {
     // 80-row tiles when they pad m less than 64-row tiles do
     const bool t80 = ((m + 79) / 80) * 80 < ((m + 63) / 64) * 64;
@@ -235,13 +234,10 @@ cudaError_t gemm(bool transA, int m, int n, int k, double alpha, const typename 
 
 template cudaError_t gemm<double>(bool, int, int, int, double, const double*, long long,
                                   const double*, long long, double, double*, long long,
-                                  cudaStream_t, const int*, const int*, const int*, int);
-template cudaError_t gemm<df>(bool, int, int, int, double, const double*, long long,
-                              const double*, long long, double, double*, long long, cudaStream_t,
-                              const int*, const int*, const int*, int);
-template cudaError_t gemm<float>(bool, int, int, int, double, const float*, long long,
-                                 const float*, long long, double, float*, long long, cudaStream_t,
-                                 const int*, const int*, const int*, int);
+                                  cudaStream_t, const int*, const int*, const int*, int, bool);
+template cudaError_t gemm<float>(bool, int, int, int, double, const float*, long long, const float*,
+                                 long long, double, float*, long long, cudaStream_t, const int*,
+                                 const int*, const int*, int, bool);
 
 // ---------------------------------------------------------------------------
 // one-sided Jacobi eigensolver
@@ -542,8 +538,6 @@ template cudaError_t convert<double, double>(double*, long long, const double*, 
                                              cudaStream_t);
 template cudaError_t convert<float, double>(float*, long long, const double*, long long, int, int,
                                             cudaStream_t);
-template cudaError_t convert<df, double>(df*, long long, const double*, long long, int, int,
-                                         cudaStream_t);
 template cudaError_t convert<double, float>(double*, long long, const float*, long long, int, int,
                                             cudaStream_t);
 

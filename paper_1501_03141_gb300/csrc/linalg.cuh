@@ -7,7 +7,6 @@
 #include <vector>
 
 #include "common.cuh"
-#include "df64.cuh"
 
 namespace pdep {
 
@@ -16,19 +15,20 @@ namespace pdep {
 // column maps: column j of B is B[:, bmap[j]] and column j of C is C[:, cmap[j]].
 // ndev (optional): device count of the mapped columns (<= n); the launch is
 // sized for n and columns from *ndev on are left untouched.  R: float, or
-// double / df on FP64 matrices, both by exact integer products on the FP16
-// tensor cores (fx_gemm.cu; df only names another profile class).
+// double by exact integer products on the FP16 tensor cores (fx_gemm.cu).
 // split_x8 (FP64; optional): split-K multiplier of the default split
-// (split_x8 / 8, 0 = default); the autotuner picks it per GEMM shape.
+// (split_x8 / 8, 0 = default); the autotuner picks it per GEMM shape.  mixed:
+// profiled with the mixed modes' refinement.
 template <typename R>
-cudaError_t gemm(bool transA, int m, int n, int k, double alpha, const typename Io<R>::T* A,
-                 long long lda, const typename Io<R>::T* B, long long ldb, double beta,
-                 typename Io<R>::T* C, long long ldc, cudaStream_t st, const int* bmap = nullptr,
-                 const int* cmap = nullptr, const int* ndev = nullptr, int split_x8 = 0);
+cudaError_t gemm(bool transA, int m, int n, int k, double alpha, const R* A,
+                 long long lda, const R* B, long long ldb, double beta,
+                 R* C, long long ldc, cudaStream_t st, const int* bmap = nullptr,
+                 const int* cmap = nullptr, const int* ndev = nullptr, int split_x8 = 0,
+                 bool mixed = false);
 cudaError_t gemm_fx(bool transA, int m, int n, int k, double alpha, const double* A, long long lda,
                     const double* B, long long ldb, double beta, double* C, long long ldc, int sms,
                     cudaStream_t st, const int* bmap, const int* cmap, const int* ndev,
-                    int split_x8, bool df_class);
+                    int split_x8, bool mixed);
 
 // Symmetric eigendecomposition of the n x n matrix M (lda), FP64:
 // one-sided (Hestenes) Jacobi on M - sigma I (sigma = twice the Gershgorin

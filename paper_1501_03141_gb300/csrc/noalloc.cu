@@ -68,8 +68,7 @@ bool on_device(const void* p) {
 
 // Sphere description of one system and the context's device, filled from the
 // context (no copies).
-int noalloc_sphere(pdep_ctx* ctx, int sys, SphereDev<double>* sd, const double** v, int* n_pw,
-                   int* device);
+int noalloc_sphere(pdep_ctx* ctx, int sys, SphereDev<double>* sd, int* n_pw, int* device);
 
 }  // namespace pdep
 
@@ -78,9 +77,8 @@ using namespace pdep;
 extern "C" int pdep_apply_hamiltonian_noalloc(pdep_ctx* ctx, int sys, const double* x, int n,
                                               double* y, void* stream) {
   SphereDev<double> sd{};
-  const double* v = nullptr;
   int n_pw = 0, device = 0;
-  int r = noalloc_sphere(ctx, sys, &sd, &v, &n_pw, &device);
+  int r = noalloc_sphere(ctx, sys, &sd, &n_pw, &device);
   if (r != PDEP_OK) return r;
   if (n < 0 || (n > 0 && (!x || !y))) {
     set_last_error(__FILE__, __LINE__, "bad arguments");
@@ -111,15 +109,14 @@ extern "C" int pdep_apply_hamiltonian_noalloc(pdep_ctx* ctx, int sys, const doub
     ItemMap map{m, n_items};
     const double* xs = x + v0 * n_pw;
     double* ys = y + v0 * n_pw;
-    cudaError_t e = launch_cols_fwd<double>(sd, xs, n_pw, map, n_items, COEF_ONE, b1, st);
+    cudaError_t e = launch_cols_fwd(sd, xs, n_pw, map, n_items, COEF_ONE, b1, st);
     if (e == cudaSuccess) {
       SlabArgs<double> a{};
       a.mode = SLAB_HPSI;
       a.b1 = b1;
       a.n_items = n_items;
-      a.v = v;
       a.map = map;
-      e = launch_slab<double>(sd, a, st);
+      e = launch_slab(sd, a, st);
     }
     if (e == cudaSuccess) {
       Epilogue<double> ep{};
@@ -131,7 +128,7 @@ extern "C" int pdep_apply_hamiltonian_noalloc(pdep_ctx* ctx, int sys, const doub
       ep.scale = 1.0 / ((double)sd.N1 * sd.N2 * sd.N3);
       ep.kin = 1.0;
       ep.coef = COEF_ONE;
-      e = launch_cols_bwd<double>(sd, b1, map, n_items, ep, st);
+      e = launch_cols_bwd(sd, b1, map, n_items, ep, st);
     }
     if (e != cudaSuccess) {
       set_last_error(__FILE__, __LINE__, cudaGetErrorString(e));

@@ -12,8 +12,10 @@
 //                  two real fields and a fused epilogue
 #pragma once
 
+#include <cmath>
+#include <vector>
+
 #include "common.cuh"
-#include "df64.cuh"
 
 namespace pdep {
 
@@ -32,9 +34,16 @@ struct SphereDev {
   const int2* slot;         // [2 R3 + 1]: (R2(n3), first full-column index)
   const double* g2;         // |G_k|^2, [n_half]
   const R* kin;             // |G_k|^2 / 2 in the kernel's precision, [n_half]
-  const cpx<R>* tw1;        // exp(+2 pi i j/N1), j < N1
+  const cpx<R>* tw1;        // FP32: exp(+2 pi i j/N1), j < N1
   const cpx<R>* tw2;
   const cpx<R>* tw3;
+  // FP64 transforms (transforms_fx.cu): digit tables of the x-, y- and z-lines,
+  // the potential as integers and their scale, V = vfx 2^v_exp
+  const uint32_t* fx1;
+  const uint32_t* fx2;
+  const uint32_t* fx3;
+  const long long* vfx;
+  int v_exp;
 #ifdef PDEP_BOUNDS_CHECK
   unsigned* status = nullptr;  // device status word the bounds tests report to
 #endif
@@ -109,11 +118,9 @@ enum CoefKind : int { COEF_ONE = 0, COEF_SQRT_COULOMB = 1 };
 // Epilogue of the column pass back:
 //   y = scale * coef(G) * (transform) + (kin * |G|^2/2 + shift[vec]) * x_in
 //       (+ beta * y_old)
-// R is the arithmetic type of the transform; vectors are stored in
-// Io<R>::T (FP64 for the double-float transforms, else R itself).
 template <typename R>
 struct Epilogue {
-  using T = typename Io<R>::T;
+  using T = R;
   T* y;                 // output vectors (real layout)
   long long ldy;
   const T* x_in;        // vectors for the diagonal term (may be null)
@@ -129,7 +136,7 @@ struct Epilogue {
 // Grid source of the grid -> sphere slab pass: field = f(r) * (ga(r) + i gb(r))
 template <typename R>
 struct GridSrc {
-  using T = typename Io<R>::T;
+  using T = R;
   const T* f;          // may be null (f = 1)
   long long f_stride;  // per group (item_map group)
   const T* g;          // ga/gb are vectors of g with stride g_stride
@@ -147,8 +154,8 @@ struct SlabArgs {
   int mode;
   cpx<R>* b1;            // [n_items][N1][n_col]
   int n_items;
-  const R* v;            // local potential [N_r] (HPSI), in the arithmetic type
-  typename Io<R>::T* out;  // TO_GRID: two fields per item at vec(item,s)*out_stride
+  const R* v;            // local potential [N_r] (HPSI; FP32 only, FP64 takes s.vfx)
+  R* out;                // TO_GRID: two fields per item at vec(item,s)*out_stride
   long long out_stride;
   double out_scale;
   GridSrc<R> src;        // FROM_GRID (f: one grid per group, g: per-vector grids)
@@ -160,18 +167,24 @@ struct SlabArgs {
   int dn_nocc = 1;
   long long dn_stride = 0;
   double dn_scale = 0.0;
+  int digits = 8;             // FP64: digits of the tensor-core products
 };
 
-// Host launchers (stream-ordered; no synchronisation).  R = float, double or
-// df (double-float arithmetic on FP64 vectors).
-template <typename R>
-cudaError_t launch_cols_fwd(const SphereDev<R>& s, const typename Io<R>::T* x, long long ldx,
-                            ItemMap map, int n_items, int coef, cpx<R>* b1, cudaStream_t st);
-template <typename R>
-cudaError_t launch_slab(const SphereDev<R>& s, const SlabArgs<R>& a, cudaStream_t st);
-template <typename R>
-cudaError_t launch_cols_bwd(const SphereDev<R>& s, const cpx<R>* b1, ItemMap map, int n_items,
-                            const Epilogue<R>& ep, cudaStream_t st);
+// Host launchers (stream-ordered; no synchronisation): FP32 transforms, and
+// FP64 ones on the tensor cores (transforms_fx.cu; digits: those of the
+// operands, FX_S for FP64 accuracy, seven in the mixed modes' refinement).
+cudaError_t launch_cols_fwd(const SphereDev<float>& s, const float* x, long long ldx, ItemMap map,
+                            int n_items, int coef, cpx<float>* b1, cudaStream_t st);
+cudaError_t launch_slab(const SphereDev<float>& s, const SlabArgs<float>& a, cudaStream_t st);
+cudaError_t launch_cols_bwd(const SphereDev<float>& s, const cpx<float>* b1, ItemMap map,
+                            int n_items, const Epilogue<float>& ep, cudaStream_t st);
+cudaError_t launch_cols_fwd(const SphereDev<double>& s, const double* x, long long ldx, ItemMap map,
+                            int n_items, int coef, cpx<double>* b1, cudaStream_t st,
+                            int digits = 8);
+cudaError_t launch_slab(const SphereDev<double>& s, const SlabArgs<double>& a, cudaStream_t st);
+cudaError_t launch_cols_bwd(const SphereDev<double>& s, const cpx<double>* b1, ItemMap map,
+                            int n_items, const Epilogue<double>& ep, cudaStream_t st,
+                            int digits = 8);
 
 // H x in FP32 by one fused launch (column scratch in shared memory) for the
 // cubic grids 24^3 .. 48^3: the same result as cols_fwd + slab (HPSI) +
@@ -185,6 +198,43 @@ int hpsi_fused_planes(const SphereDev<float>& s, int planes = 0);
 cudaError_t launch_hpsi_fused(const SphereDev<float>& s, const float* x, long long ldx, ItemMap map,
                               int n_items, const float* v, const Epilogue<float>& ep,
                               cudaStream_t st, int planes = 0);
+
+// Digit tables of the FP64 transforms for lines of N points (empty for other
+// lengths), and the potential v [n] as 63-bit integers scaled by the exponent
+// field er of its largest magnitude (>= 1): v = out 2^(er - 1084).
+std::vector<uint32_t> fx_line_table(int N);
+cudaError_t fixed_potential(const double* v, int n, int er, long long* out, cudaStream_t st);
+
+// algorithmic work of a slab launch: y-lines over the |n3| <= R3 planes and
+// z-lines over the N2 rows of each x-plane, 5 L log2 L flops per complex line FFT
+template <typename R>
+void slab_work(const SphereDev<R>& s, const SlabArgs<R>& a, double& fl, double& by) {
+  const double ylines = (double)(2 * s.R3 + 1), zlines = (double)s.N2;
+  const double fy = 5.0 * s.N2 * std::log2((double)s.N2), fz = 5.0 * s.N3 * std::log2((double)s.N3);
+  const double planes = (double)a.n_items * s.N1, pts = (double)s.N2 * s.N3;
+  const double colb = (double)s.n_col * 2.0 * sizeof(R);  // one plane of B1
+  const double gridb = pts * sizeof(R);                   // one plane of a real grid
+  switch (a.mode) {
+    case SLAB_HPSI:
+      fl = planes * (2 * ylines * fy + 2 * zlines * fz + 2.0 * pts);
+      by = planes * 2 * colb + s.N1 * gridb;
+      if (a.dn) {
+        // density response: 2 products per point and vector; dn read and
+        // written once per perturbation, u read once
+        fl += planes * 4.0 * pts;
+        by += (2.0 * a.n_items / a.dn_nocc) * s.N1 * 2.0 * gridb + (double)a.dn_nocc * s.N1 * gridb;
+      }
+      break;
+    case SLAB_TO_GRID:
+      fl = planes * (ylines * fy + zlines * fz);
+      by = planes * (colb + 2 * gridb);
+      break;
+    case SLAB_FROM_GRID:
+      fl = planes * (ylines * fy + zlines * fz + 3.0 * pts);
+      by = planes * (colb + 3 * gridb);
+      break;
+  }
+}
 
 bool grid_supported(int N1, int N2, int N3);
 cudaError_t upload_local_twiddles();
