@@ -123,6 +123,7 @@ struct Tune {
 // valid for the buffers and settings it was captured with.
 struct CgGraph {
   int prec, sys, n, max_iter, cg_variant, proj_variant, tune_gen;
+  int prologue, body;  // kernels before the loop, and per step
   double tol;
   const void *b, *x, *sc, *mask, *tolv;
   unsigned long long ws_gen, budget_ns;
@@ -146,8 +147,9 @@ struct pdep_ctx {
   unsigned long long ws_gen = 0;  // bumped whenever a workspace buffer is reallocated
   unsigned long long budget_ns = 0;   // clock_budget_cycles in ns of %globaltimer
   std::vector<CgGraph> cg_graphs;     // executable CG-loop graphs, released in pdep_destroy
-  int body_launches[2] = {0, 0};      // kernels per CG step in the graphs (FP32, FP64)
+  int body_launches[2] = {0, 0};      // kernels per CG step of the last graph (FP32, FP64)
   long long graph_launches = 0;       // CG graphs launched
+  long long prologue_launches = 0;    // kernels before their loops
   long long eager_steps[2] = {0, 0};  // CG steps launched from the host loop (FP32, FP64)
   long long st_launch0 = 0;           // launch counter at the last statistics reset
   pdep_stats last_dav{};              // statistics of the last pdep_solve
@@ -496,6 +498,8 @@ std::string shape_key(const char* what, const SysData& s) {
 
 // d_count (with d_list): device length of the list; n_list is then the
 // largest length, which sizes the launches (kernels read the count).
+constexpr int kFewItems = 38;  // a quarter of the SMs
+
 // R: FP32 or FP64.  refine (FP64): the product of a mixed-mode refinement, whose
 // transforms take seven digits (far below the FP32 inner solve's needs and
 // above double-float).
@@ -516,7 +520,10 @@ int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list,
   if constexpr (std::is_same<R, float>::value) {
     // FP32 on 24^3 .. 48^3: the whole transform in one launch, the column
     // scratch in shared memory
-    if (n_items > 0 && !dn && c->opt.fused_hpsi && hpsi_fused_smem(s.sf) > 0) {
+    // (few items leave it a block or less per four SMs, and an item's time is
+    // then its block's: 21 us on 24^3 and 90 us on 48^3 against 9 and about 50
+    // in three launches over all planes)
+    if (n_items > kFewItems && !dn && c->opt.fused_hpsi && hpsi_fused_smem(s.sf) > 0) {
       Epilogue<float> ep{};
       ep.y = Y;
       ep.ldy = s.ld;
@@ -1100,7 +1107,7 @@ bool tuned(const pdep_ctx* c, const SysData& s, int pi) {
   return c->cg_variant[pi] >= 0 && pv_ok && fused_ok;
 }
 int cg_variant_of(const pdep_ctx* c, int pi) {
-  return c->cg_variant[pi] >= 0 ? c->cg_variant[pi] : (int)CG_STREAM256;
+  return c->cg_variant[pi] >= 0 ? c->cg_variant[pi] : 0;
 }
 
 // Workspace the step of a CG loop over n RHS needs (allocated before a
@@ -1126,14 +1133,55 @@ int cg_workspace(pdep_ctx* c, SysData& s, int n, R** r, R** p, R** ap, int** lis
   return PDEP_OK;
 }
 
+// Whether the CG step adds the projection itself: the states pass through L2
+// twice per RHS, which up to about 64 MB (some 8 us) costs less than the
+// coefficient and update launches (on 24^3 with 8 RHS 18 us against 3; on 64^3
+// with 84 RHS of 44 states 26 us against some 60).
+template <typename R>
+bool few_projection(const pdep_ctx* c, const SysData& s, int n) {
+  if (sizeof(R) == 4 && (c->opt.proj_variant >= 0 || s.d_psib16)) return false;
+  return cg_proj_fits(s.n_pw, (int)sizeof(R), s.n_ext) &&
+         2.0 * n * s.n_ext * s.n_pw * sizeof(R) <= 64e6;
+}
+
+template <typename R>
+CgProj<R> step_projection(const SysData& s) {
+  CgProj<R> pj;
+  pj.states = psi_of(s, (R*)nullptr);
+  pj.sigma = sigma_of(s, (R*)nullptr);
+  pj.n = s.n_ext;
+  return pj;
+}
+CgTail step_tail(const pdep_ctx* c, int* list, int max_iter, int prec,
+                 cudaGraphConditionalHandle h, int has_handle) {
+  CgTail t;
+  t.on = 1;
+  t.ticket = c->d_counter;
+  t.list = list;
+  t.loop = c->d_loop;
+  t.max_iter = max_iter;
+  t.prec = prec;
+  t.budget_ns = c->budget_ns;
+  t.handle = h;
+  t.has_handle = has_handle;
+  return t;
+}
+
 // Captures one CG loop over n RHS into an executable graph:
 //   prologue: active = 0, cg_start (r = b, p = K b, active count), loop_begin
 //   while (go): active list, A p on the listed RHS, PCG step, loop_next
+// Up to CG_TAIL_MAX RHS the step's last cluster builds the next list and takes
+// the loop decision (the first list comes with the prologue), and where the
+// states are read within few_projection's limit the step adds the projection:
+// a step is then the transform's launches and one more.
 // Launches inside are sized for n; the kernels read the list length from
 // the device loop state.  All workspace is allocated beforehand (cg_workspace).
 template <typename R>
 int capture_cg_graph(pdep_ctx* c, SysData& s, CgArgs<R> a, const R* b, int n, int max_iter,
-                     int* list, cudaGraphExec_t* out) {
+                     int* list, CgGraph* gr) {
+  cudaGraphExec_t* out = &gr->exec;
+  const bool tail = n <= CG_TAIL_MAX, fuse = tail && few_projection<R>(c, s, n);
+  if (tail) a.variant = n < 256 ? (int)CG_FEW : a.variant;
   const int pi = sizeof(R) == 8 ? 1 : 0;
   cudaStream_t cs = c->cap_stream;
   const unsigned long long gen = c->ws_gen;
@@ -1158,8 +1206,11 @@ int capture_cg_graph(pdep_ctx* c, SysData& s, CgArgs<R> a, const R* b, int n, in
       chk(cudaStreamBeginCapture(cs, cudaStreamCaptureModeRelaxed))) {
     capture_begin();
     bool ok = chk(cudaMemsetAsync(&c->d_loop->active, 0, sizeof(int), cs)) &&
-              chk(cg_start<R>(a, b, s.ld, cs)) && chk(loop_begin(c->d_loop, max_iter, h, 1, cs));
-    capture_end();
+              chk(cudaMemsetAsync(c->d_counter, 0, sizeof(int), cs)) &&
+              chk(cg_start<R>(a, b, s.ld, cs)) &&
+              (!tail || chk(active_list(a.sc, n, list, &c->d_loop->listed, cs))) &&
+              chk(loop_begin(c->d_loop, max_iter, h, 1, cs));
+    gr->prologue = capture_end();
     if (ok) {
       chk(cudaStreamEndCapture(cs, &pro));
     } else {
@@ -1178,9 +1229,9 @@ int capture_cg_graph(pdep_ctx* c, SysData& s, CgArgs<R> a, const R* b, int n, in
   if (status == PDEP_OK &&
       chk(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed))) {
     capture_begin();
-    bool ok = chk(active_list_reset(a.sc, n, list, &c->d_loop->listed, &c->d_loop->active, cs));
+    bool ok = tail || chk(active_list_reset(a.sc, n, list, &c->d_loop->listed, &c->d_loop->active, cs));
     if (ok) {
-      const int r = apply_h<R>(c, s, a.p, (R*)a.ap, n, list, n, true, true, cs, nullptr,
+      const int r = apply_h<R>(c, s, a.p, (R*)a.ap, n, list, n, true, !fuse, cs, nullptr,
                                &c->d_loop->listed);
       if (r != PDEP_OK) {
         status = r;
@@ -1188,8 +1239,11 @@ int capture_cg_graph(pdep_ctx* c, SysData& s, CgArgs<R> a, const R* b, int n, in
       }
     }
     a.list_count = &c->d_loop->listed;
-    ok = ok && chk(cg_step<R>(a, list, n, cs)) &&
-         chk(loop_next(c->d_loop, max_iter, c->budget_ns, c->d_status, pi, h, 1, cs));
+    const CgProj<R> pj = step_projection<R>(s);
+    const CgTail tl = step_tail(c, list, max_iter, pi, h, 1);
+    ok = ok && chk(cg_step<R>(a, list, n, cs, fuse ? &pj : nullptr, tail ? &tl : nullptr)) &&
+         (tail ||
+          chk(loop_next(c->d_loop, max_iter, c->budget_ns, c->d_status, pi, h, 1, cs)));
     launches = capture_end();
     if (ok) {
       cudaGraph_t got = body;
@@ -1203,7 +1257,7 @@ int capture_cg_graph(pdep_ctx* c, SysData& s, CgArgs<R> a, const R* b, int n, in
   if (status == PDEP_OK) chk(cudaGraphInstantiate(out, g, 0));
   if (pro) cudaGraphDestroy(pro);
   cudaGraphDestroy(g);
-  if (status == PDEP_OK) c->body_launches[pi] = launches;
+  gr->body = launches;
   return status;
 }
 
@@ -1250,12 +1304,17 @@ int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int ma
   // current (or default) shapes and are captured right away
   const bool graph = c->opt.use_graph && (tuned(c, s, pi) || n < 256);
   if (!graph) {
-    // eager: host loop, one 8-byte read of the loop state per step
+    // eager: host loop, one 16-byte read of the loop state per step
+    const bool tail = n <= CG_TAIL_MAX, fuse = tail && few_projection<R>(c, s, n);
+    const CgProj<R> pj = step_projection<R>(s);
+    const CgTail tl = step_tail(c, list, max_iter, pi, 0, 0);
     CK(cudaMemsetAsync(&c->d_loop->active, 0, sizeof(int), st));
+    CK(cudaMemsetAsync(c->d_counter, 0, sizeof(int), st));
     CK(cg_start<R>(a, b, s.ld, st));
+    if (tail) CK(active_list(sc, n, list, &c->d_loop->listed, st));
     CK(loop_begin(c->d_loop, max_iter, 0, 0, st));
     for (;;) {
-      // active, listed, iter, go: one 16-byte read per step
+      // active, listed, iter, go
       CK(cudaMemcpyAsync(c->h_pin, &c->d_loop->active, 4 * sizeof(int), cudaMemcpyDeviceToHost,
                          st));
       CK(cudaStreamSynchronize(st));
@@ -1263,16 +1322,17 @@ int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int ma
       memcpy(h, c->h_pin, sizeof(h));
       if (!h[3]) break;
       const int n_act = h[0];
-      CK(active_list_reset(sc, n, list, &c->d_loop->listed, &c->d_loop->active, st));
-      RET(apply_h<R>(c, s, p, ap, n, list, n_act, true, true, st));
+      if (!tail) CK(active_list_reset(sc, n, list, &c->d_loop->listed, &c->d_loop->active, st));
+      RET(apply_h<R>(c, s, p, ap, n, list, n_act, true, !fuse, st));
       // Autotuner: while untuned, each large step tries the next launch shape
       // (all shapes compute the same update) and its time per RHS is kept;
       // afterwards the fastest shape is used.
       const bool tuning = c->opt.autotune && c->cg_variant[pi] < 0 && n_act >= 256;
       a.variant = tuning ? c->cg_tune_next[pi] : cg_variant_of(c, pi);
+      if (tail && n < 256) a.variant = CG_FEW;
       a.list_count = nullptr;
       if (tuning) CK(cudaEventRecord(c->ev[0], st));
-      CK(cg_step<R>(a, list, n_act, st));
+      CK(cg_step<R>(a, list, n_act, st, fuse ? &pj : nullptr, tail ? &tl : nullptr));
       if (tuning) {
         CK(cudaEventRecord(c->ev[1], st));
         CK(cudaEventSynchronize(c->ev[1]));
@@ -1286,7 +1346,7 @@ int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int ma
           c->cg_variant[pi] = best;
         }
       }
-      CK(loop_next(c->d_loop, max_iter, c->budget_ns, c->d_status, pi, 0, 0, st));
+      if (!tail) CK(loop_next(c->d_loop, max_iter, c->budget_ns, c->d_status, pi, 0, 0, st));
       ++c->eager_steps[pi];
     }
     return PDEP_OK;
@@ -1321,7 +1381,7 @@ int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int ma
     e.proj_variant = pv;
     e.budget_ns = c->budget_ns;
     e.tune_gen = c->tune_gen;
-    RET(capture_cg_graph<R>(c, s, a, b, n, max_iter, list, &e.exec));
+    RET(capture_cg_graph<R>(c, s, a, b, n, max_iter, list, &e));
     if (c->cg_graphs.size() >= 16) {
       cudaGraphExecDestroy(c->cg_graphs.front().exec);
       c->cg_graphs.erase(c->cg_graphs.begin());
@@ -1334,6 +1394,8 @@ int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int ma
     CK(cudaGraphLaunch(g->exec, st));
   }
   ++c->graph_launches;
+  c->prologue_launches += g->prologue;
+  c->body_launches[pi] = g->body;
   return PDEP_OK;
 }
 
@@ -1593,6 +1655,7 @@ int reset_stats(pdep_ctx* c, cudaStream_t st) {
   c->st_solves = 0;
   c->st_chunks = 0;
   c->graph_launches = 0;
+  c->prologue_launches = 0;
   c->eager_steps[0] = c->eager_steps[1] = 0;
   c->st_launch0 = launch_count();
   CK(cudaMemsetAsync(c->d_dstats, 0, sizeof(DevStats), st));
@@ -1620,9 +1683,8 @@ int read_stats(pdep_ctx* c, pdep_stats* out, cudaStream_t st) {
                           : (c->opt.proj_variant >= 0 ? c->opt.proj_variant : c->proj_variant);
   out->chi0_chunks = c->st_chunks;
   // launches outside graphs are counted on the host; a graph contributes its
-  // prologue (2 kernels) per launch and its body per step, the steps counted
-  // on the device (loop_next counts eager steps too: those are subtracted)
-  long long in_graphs = 2 * c->graph_launches;
+  // prologue per launch and its body per step, the steps counted on the device (loop_next counts eager steps too: those are subtracted)
+  long long in_graphs = c->prologue_launches;
   for (int pi = 0; pi < 2; ++pi)
     in_graphs += ((long long)steps[pi] - c->eager_steps[pi]) * c->body_launches[pi];
   out->kernel_launches = (launch_count() - c->st_launch0) + in_graphs;

@@ -1148,7 +1148,7 @@ cudaError_t fill_zero(void* p, size_t bytes, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------------------
-// preconditioned CG on (H - eps_v + alpha P_v) x = b, one CTA per RHS
+// preconditioned CG on (H - eps_v + alpha P_v) x = b (the step: cg_step.cu)
 // ---------------------------------------------------------------------------
 // Teter-Payne-Allan kinetic preconditioner (Phys. Rev. B 40, 12255 (1989)):
 // K(x) = (27 + 18x + 12x^2 + 8x^3) / (27 + 18x + 12x^2 + 8x^3 + 16x^4),
@@ -1219,153 +1219,6 @@ __global__ void k_cg_start(CgArgs<R> a, const R* __restrict__ b, long long ldb) 
   }
 }
 
-// finish one RHS's step (thread 0): scalars, convergence, active count
-template <typename R>
-__device__ __forceinline__ void cg_finish(const CgArgs<R>& a, int i, const CgScal& s, double rn,
-                                          double rkr, bool done) {
-  CgScal n = s;
-  n.iters = s.iters + 1;
-  n.rnorm = rn;
-  n.rz = rkr;
-  n.active = done ? 0 : 1;
-  if (!isfinite(rn)) {
-    n.active = 0;
-    atomicOr(a.status, (unsigned)DEV_NONFINITE);
-  }
-  a.sc[i] = n;
-  if (n.active) atomicAdd(a.n_active, 1);
-}
-
-// Register-cached step: each thread keeps its E elements of p, Ap and r, so
-// the RHS is read once (p, Ap, x, r) and written once (x, r, p).  Element
-// arithmetic runs in R (FP32 costs 1/64 of FP64 on this part); only the
-// per-thread partial sums are promoted to FP64 for the block reductions.
-template <typename R, int E>
-__global__ void __launch_bounds__(512) k_cg_step_reg(CgArgs<R> a, const int* __restrict__ list) {
-  if (a.list_count && (int)blockIdx.x >= *a.list_count) return;
-  const int i = list ? list[blockIdx.x] : blockIdx.x;
-  __shared__ CgScal s;
-  __shared__ R coef[2];  // alpha, then beta
-  __shared__ int flag;   // 1: breakdown, 2: converged
-  if (threadIdx.x == 0) s = a.sc[i];
-  __syncthreads();
-  if (!s.active) return;
-  const long long o = (long long)i * a.ld;
-  const R* K = a.kprec + (long long)(i % a.n_occ) * a.ld;
-  R pv[E], av[E], rv[E];
-  R pap = R(0);
-#pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int j = threadIdx.x + e * blockDim.x;
-    if (j < a.n_pw) {
-      pv[e] = a.p[o + j];
-      av[e] = a.ap[o + j];
-      pap += pv[e] * av[e];
-    } else {
-      pv[e] = R(0);
-      av[e] = R(0);
-    }
-  }
-  const double2 t1 = block_sum2_r<R>(pap, R(0));
-  if (threadIdx.x == 0) {
-    const double al = s.rz / t1.x;
-    flag = (!(t1.x > 0.0) || !isfinite(al)) ? 1 : 0;
-    coef[0] = (R)al;
-    if (flag) {
-      atomicOr(a.status, isfinite(t1.x) ? (unsigned)DEV_BREAKDOWN : (unsigned)DEV_NONFINITE);
-      a.sc[i].active = 0;
-    }
-  }
-  __syncthreads();
-  if (flag) return;
-  const R alpha = coef[0];
-  R rr = R(0), rkr = R(0);
-#pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int j = threadIdx.x + e * blockDim.x;
-    if (j < a.n_pw) {
-      a.x[o + j] = a.x[o + j] + alpha * pv[e];
-      const R r = a.r[o + j] - alpha * av[e];
-      rv[e] = r;
-      rr += r * r;
-      rkr += K[j] * r * r;
-    } else {
-      rv[e] = R(0);
-    }
-  }
-  const double2 t2 = block_sum2_r<R>(rr, rkr);
-  if (threadIdx.x == 0) {
-    const double rn = sqrt(t2.x);
-    const bool done = rn <= (a.tolv ? a.tolv[i] : a.tol) * s.bnorm;
-    flag = done ? 2 : 0;
-    coef[1] = (R)(t2.y / s.rz);
-    cg_finish(a, i, s, rn, t2.y, done);
-  }
-  __syncthreads();
-  const bool done = flag == 2;
-  const R beta = coef[1];
-#pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int j = threadIdx.x + e * blockDim.x;
-    if (j < a.n_pw) {
-      a.r[o + j] = rv[e];
-      if (!done) a.p[o + j] = K[j] * rv[e] + beta * pv[e];
-    }
-  }
-}
-
-// Streaming step (three passes over the RHS, re-reads served by L1/L2):
-// fewer registers, so more RHS in flight per SM than the cached variant.
-template <typename R>
-__global__ void __launch_bounds__(512) k_cg_step(CgArgs<R> a, const int* __restrict__ list) {
-  if (a.list_count && (int)blockIdx.x >= *a.list_count) return;
-  const int i = list ? list[blockIdx.x] : blockIdx.x;
-  __shared__ CgScal s;
-  __shared__ R coef[2];
-  __shared__ int flag;
-  if (threadIdx.x == 0) s = a.sc[i];
-  __syncthreads();
-  if (!s.active) return;
-  const long long o = (long long)i * a.ld;
-  const R* K = a.kprec + (long long)(i % a.n_occ) * a.ld;
-  R pap = R(0);
-  for (int j = threadIdx.x; j < a.n_pw; j += blockDim.x) pap += a.p[o + j] * a.ap[o + j];
-  const double2 t1 = block_sum2_r<R>(pap, R(0));
-  if (threadIdx.x == 0) {
-    const double al = s.rz / t1.x;
-    flag = (!(t1.x > 0.0) || !isfinite(al)) ? 1 : 0;
-    coef[0] = (R)al;
-    if (flag) {
-      atomicOr(a.status, isfinite(t1.x) ? (unsigned)DEV_BREAKDOWN : (unsigned)DEV_NONFINITE);
-      a.sc[i].active = 0;
-    }
-  }
-  __syncthreads();
-  if (flag) return;
-  const R alpha = coef[0];
-  R rr = R(0), rkr = R(0);
-  for (int j = threadIdx.x; j < a.n_pw; j += blockDim.x) {
-    a.x[o + j] = a.x[o + j] + alpha * a.p[o + j];
-    const R r = a.r[o + j] - alpha * a.ap[o + j];
-    a.r[o + j] = r;
-    rr += r * r;
-    rkr += K[j] * r * r;
-  }
-  const double2 t2 = block_sum2_r<R>(rr, rkr);
-  if (threadIdx.x == 0) {
-    const double rn = sqrt(t2.x);
-    const bool done = rn <= (a.tolv ? a.tolv[i] : a.tol) * s.bnorm;
-    flag = done ? 2 : 0;
-    coef[1] = (R)(t2.y / s.rz);
-    cg_finish(a, i, s, rn, t2.y, done);
-  }
-  __syncthreads();
-  if (flag == 2) return;
-  const R beta = coef[1];
-  for (int j = threadIdx.x; j < a.n_pw; j += blockDim.x)
-    a.p[o + j] = K[j] * a.r[o + j] + beta * a.p[o + j];
-}
-
 template <typename R>
 cudaError_t cg_start(const CgArgs<R>& a, const R* b, long long ldb, cudaStream_t st) {
   if (a.n_rhs <= 0) return cudaSuccess;
@@ -1373,30 +1226,8 @@ cudaError_t cg_start(const CgArgs<R>& a, const R* b, long long ldb, cudaStream_t
   k_cg_start<R><<<a.n_rhs, 256, 0, st>>>(a, b, ldb);
   return cudaGetLastError();
 }
-template <typename R>
-cudaError_t cg_step(const CgArgs<R>& a, const int* list, int n_list, cudaStream_t st) {
-  const int nb = list ? n_list : a.n_rhs;
-  if (nb <= 0) return cudaSuccess;
-  // x, r, p, Ap read once; x, r, p written once: 7 vector passes per active RHS
-  ProfScope ps(sizeof(R) == 8 ? PC_CG_F64 : PC_CG_F32, st, 12.0 * nb * (double)a.n_pw,
-               7.0 * nb * (double)a.n_pw * sizeof(R), list ? a.list_count : nullptr, nb);
-  count_launch();
-  int v = a.variant;
-  if ((v == CG_REG256 && a.n_pw > 16 * 256) || (v == CG_REG512 && a.n_pw > 16 * 512))
-    v = CG_STREAM256;
-  switch (v) {
-    case CG_REG256: k_cg_step_reg<R, 16><<<nb, 256, 0, st>>>(a, list); break;
-    case CG_REG512: k_cg_step_reg<R, 16><<<nb, 512, 0, st>>>(a, list); break;
-    case CG_STREAM128: k_cg_step<R><<<nb, 128, 0, st>>>(a, list); break;
-    case CG_STREAM512: k_cg_step<R><<<nb, 512, 0, st>>>(a, list); break;
-    default: k_cg_step<R><<<nb, 256, 0, st>>>(a, list); break;
-  }
-  return cudaGetLastError();
-}
 template cudaError_t cg_start<double>(const CgArgs<double>&, const double*, long long, cudaStream_t);
 template cudaError_t cg_start<float>(const CgArgs<float>&, const float*, long long, cudaStream_t);
-template cudaError_t cg_step<double>(const CgArgs<double>&, const int*, int, cudaStream_t);
-template cudaError_t cg_step<float>(const CgArgs<float>&, const int*, int, cudaStream_t);
 
 // ordered compaction with one block of 1024 threads (contiguous chunks + scan)
 template <typename Pred>

@@ -160,7 +160,7 @@ cudaError_t tc5_proj_coeffs(int n_ext, int N, int K, const void* Pt, const float
                             long long lds, cudaStream_t st, const int* ndev, unsigned* status,
                             bool bf16 = false);
 
-// Per-RHS preconditioned CG kernels (one CTA per RHS vector).
+// Per-RHS preconditioned CG kernels.
 // State of one RHS: x, r, p (length n_pw, stride ld), scalars in CgScal.
 struct CgScal {
   double rz;      // r . K r
@@ -185,7 +185,7 @@ struct CgArgs {
   double tol;
   unsigned* status;
   int* n_active;        // counter (atomic) of RHS still active after the step
-  int variant;          // CgVariant (picked by the autotuner)
+  int variant;          // block shape (picked by the autotuner), or CG_FEW
   const int* list_count = nullptr;  // device length of the active list (cg_step sized for
                                     // the largest; blocks past it exit)
   const double* mask = nullptr;     // cg_start: RHS i takes part only if mask[i] != 0
@@ -230,21 +230,40 @@ cudaError_t cg_collect(const CgScal* sc, int n, int* its_total, DevStats* ds, cu
 // sets DEV_NOT_CONVERGED; ds->refine_max = max(refine_max, rounds_cur).
 cudaError_t solve_finish(const double* rel, int n, double tol, DevStats* ds, unsigned* status,
                          cudaStream_t st);
-// launch shapes of one CG step: register-cached (the RHS read once) or
-// streaming (three passes, more RHS resident per SM)
-enum CgVariant : int {
-  CG_REG256 = 0,
-  CG_REG512 = 1,
-  CG_STREAM128 = 2,
-  CG_STREAM256 = 3,
-  CG_STREAM512 = 4,
-  CG_NUM_VARIANTS = 5
+// block shapes of one CG step (cg_step.cu) the autotuner times; CG_FEW: as many
+// blocks per RHS as a cluster holds, for few RHS
+enum CgVariant : int { CG_FEW = -1, CG_NUM_VARIANTS = 4 };
+// The projection term sum_w sigma_w |w><w| p added to A p inside the step:
+// states [n][ld] (the step's ld), n <= CG_PROJ_MAX.
+constexpr int CG_PROJ_MAX = 128;
+template <typename R>
+struct CgProj {
+  const R* states = nullptr;
+  const R* sigma = nullptr;
+  int n = 0;
+};
+// Loop control by the step's last cluster instead of active_list_reset and
+// loop_next (loops of at most CG_TAIL_MAX RHS): ticket is a device counter,
+// zero before the first step.
+constexpr int CG_TAIL_MAX = 1024;
+struct CgTail {
+  int on = 0;
+  int* ticket = nullptr;
+  int* list = nullptr;
+  CgLoopState* loop = nullptr;
+  int max_iter = 0, prec = 0;
+  unsigned long long budget_ns = 0;
+  cudaGraphConditionalHandle handle = 0;
+  int has_handle = 0;  // the decision also drives the enclosing while node
 };
 template <typename R>
 cudaError_t cg_start(const CgArgs<R>& a, const R* b, long long ldb, cudaStream_t st);
 // one PCG step for the n_list RHS of list (all n_rhs when list is null)
 template <typename R>
-cudaError_t cg_step(const CgArgs<R>& a, const int* list, int n_list, cudaStream_t st);
+cudaError_t cg_step(const CgArgs<R>& a, const int* list, int n_list, cudaStream_t st,
+                    const CgProj<R>* proj = nullptr, const CgTail* tail = nullptr);
+// whether the step can take the projection of n_ext states of n_pw elements
+bool cg_proj_fits(int n_pw, int elem, int n_ext);
 // K[v][j] = Teter-Payne-Allan K(|G_j|^2/2 / ekin[v]) (1 at G = 0), FP64 and FP32 copies
 cudaError_t build_precond(const double* g2, int n_half, int n_pw, const double* ekin, int n_occ,
                           double* k64, float* k32, long long ld, cudaStream_t st);
