@@ -11,35 +11,43 @@
 namespace pdep {
 namespace {
 
-// One warp per eight upper columns: the eight lines and their mirror lines are
-// two tiles of rows made from the same sphere members.  Each warp scales by
+// Two warps per eight upper columns: the eight lines and their mirror lines are
+// two tiles of rows made from the same sphere members.  A column group scales by
 // its own largest member, and the scratch holds FP64 numbers.
-constexpr int COLS_WARPS = 4;
+//
+// Bound by the latency of a warp's chain (conversion, digits, products, sums):
+// a tile per warp, with the members (in) or the coefficients (out) exchanged
+// through shared memory, halves it against one warp for both tiles.
+constexpr int COLS_PAIRS = 2;  // column groups per block
+constexpr int COLS_THREADS = 64 * COLS_PAIRS;
 
-// Frequencies |n| <= 15: the digit tables' entries of |n| >= N1 / 4 are zero.
 struct Member {
   double ax, ay, bx, by;
 };
 
+// Frequencies |n| <= 15: the digit tables' entries of |n| >= N1 / 4 are zero.
 template <int N1, int S, bool COUL>
-__global__ void __launch_bounds__(32 * COLS_WARPS, 3)
+__global__ void __launch_bounds__(COLS_THREADS, 3)
     k_cols_fx_fwd(SphereDev<double> s, const double* __restrict__ x, long long ldx, ItemMap map,
                   int n_items, cpx<double>* __restrict__ b1) {
   using L = FxLine<N1>;
+  __shared__ __align__(16) long long mem[COLS_PAIRS][32 * 8][4];
+  __shared__ int exps[2 * COLS_PAIRS];
   const int nl = listed_count(map);
-  const int units = (s.n_ucol + 7) / 8;
-  const long long unit = (long long)blockIdx.x * COLS_WARPS + (threadIdx.x >> 5);
-  const int item = (int)(unit / units);
-  if (item >= items_of(map, n_items, nl)) return;
+  const int units = (s.n_ucol + 7) / 8, warp = threadIdx.x >> 5, pair = warp >> 1, mirror = warp & 1;
+  const long long unit = (long long)blockIdx.x * COLS_PAIRS + pair;
+  int item = (int)(unit / units);
+  if ((long long)blockIdx.x * COLS_PAIRS / units >= items_of(map, n_items, nl)) return;
+  const bool any = item < items_of(map, n_items, nl);
+  if (!any) item = 0;
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int uc = (int)(unit - (long long)item * units) * 8 + g;
+  const int uc = any ? (int)(unit - (long long)item * units) * 8 + g : s.n_ucol;
   const UCol c = s.ucol[min(uc, s.n_ucol - 1)];
   const bool live = uc < s.n_ucol && ucol_in_range(s, c), self = c.col == c.mcol;
   const int R1 = live ? c.R1 : -1;
   const int ia = map.vec(item, 0, nl), ib = map.vec(item, 1, nl);
   const double* xa = ia >= 0 ? x + (long long)ia * ldx : nullptr;
   const double* xb = ib >= 0 ? x + (long long)ib * ldx : nullptr;
-  cpx<double>* base = b1 + (long long)item * N1 * s.n_col;
 
   // member n1 of this thread's column (|n| for the self-mirrored one, whose
   // n = 0 holds c(0), sqrt 2 below the others' scale)
@@ -72,84 +80,86 @@ __global__ void __launch_bounds__(32 * COLS_WARPS, 3)
     }
     return m;
   };
-  // the warp's members as integers below 2^60 in shared memory (their packed
-  // sums stay below 2^61), each read once from the sphere
-  __shared__ __align__(16) long long mem[COLS_WARPS][32 * 8][4];
-  long long(*mine)[4] = mem[threadIdx.x >> 5] + g * 32;
-  Member m[8];
+  // the group's members as integers below 2^60 (their packed sums stay below
+  // 2^61), each read once: n >= 0 by the first warp, n < 0 by the second
+  long long(*mine)[4] = mem[pair] + g * 32;
+  Member m[4];
   int ex = 1;
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const int n = 4 * t + (q & 3);
-    m[q] = member(q < 4 ? n : -n);
+  for (int q = 0; q < 4; ++q) {
+    const int n = 4 * t + q;
+    m[q] = member(mirror ? -n : n);
     ex = max(ex, max(max(exp_of(m[q].ax), exp_of(m[q].ay)), max(exp_of(m[q].bx), exp_of(m[q].by))));
   }
-  const int er = __reduce_max_sync(0xffffffffu, ex);
-  const double scale = er == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
-                                   : fx_unit(er - 1082 + 50 - SH_Y) * 0.70710678118654752440;
+  ex = __reduce_max_sync(0xffffffffu, ex);
+  if (lane == 0) exps[warp] = ex;
+  __syncthreads();
+  const int er = max(exps[2 * pair], exps[2 * pair + 1]);
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const int n = 4 * t + (q & 3);
-    longlong2* d = reinterpret_cast<longlong2*>(mine[q < 4 ? 16 + n : 16 - n]);
-    if (q >= 4 && n == 0) continue;
+  for (int q = 0; q < 4; ++q) {
+    const int n = 4 * t + q;
+    if (mirror && n == 0) continue;
+    longlong2* d = reinterpret_cast<longlong2*>(mine[mirror ? 16 - n : 16 + n]);
     d[0] = make_longlong2(fx_of(m[q].ax, er) >> 2, fx_of(m[q].ay, er) >> 2);
     d[1] = make_longlong2(fx_of(m[q].bx, er) >> 2, fx_of(m[q].by, er) >> 2);
   }
-  __syncwarp();
-#pragma unroll 1
-  for (int mirror = 0; mirror < 2; ++mirror) {
-    // (a + i b)(n) on the column, its mirror's conj(a + i b)(-n) on the mirror
-    auto ld = [&](int n) {
-      const bool flip = mirror != (self && n < 0);
-      const longlong2* d = reinterpret_cast<const longlong2*>(mine[16 + (mirror ? -n : n)]);
-      const longlong2 a = d[0], b = d[1];
-      return flip ? cl{a.x + b.y, b.x - a.y} : cl{a.x - b.y, b.x + a.y};
-    };
-    auto chunk = [&](auto nt2, int nt0) {
-      constexpr int NT2 = decltype(nt2)::value;
-      long long q[4][NT2][4];
-      line_inverse<N1, S, SH_Y, NT2>(s.fx1, nt0, ld, 0, q);
-      if (!live || (mirror && self)) return;
-      const int col = mirror ? c.mcol : c.col;
+  __syncthreads();
+  const double scale = er == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
+                                   : fx_unit(er - 1082 + 50 - SH_Y) * 0.70710678118654752440;
+  // (a + i b)(n) on the column, its mirror's conj(a + i b)(-n) on the mirror
+  auto ld = [&](int n) {
+    const bool flip = mirror != (self && n < 0);
+    const longlong2* d = reinterpret_cast<const longlong2*>(mine[16 + (mirror ? -n : n)]);
+    const longlong2 a = d[0], b = d[1];
+    return flip ? cl{a.x + b.y, b.x - a.y} : cl{a.x - b.y, b.x + a.y};
+  };
+  const int col = mirror ? c.mcol : c.col;
+  cpx<double>* base = b1 + (long long)item * N1 * s.n_col + col;
+  auto chunk = [&](auto nt2, int nt0) {
+    constexpr int NT2 = decltype(nt2)::value;
+    long long q[4][NT2][4];
+    line_inverse<N1, S, SH_Y, NT2>(s.fx1, nt0, ld, 0, q);
+    if (!live || (mirror && self)) return;
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
+    for (int k = 0; k < 4; ++k)
 #pragma unroll
-        for (int i = 0; i < NT2; ++i)
+      for (int i = 0; i < NT2; ++i)
 #pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const int j = 8 * (nt0 + i) + 2 * t + e;
-            if (!quad_new<N1>(k, j)) continue;
-            base[(long long)quad_pos<N1>(k, j) * s.n_col + col] =
-                mk(fx_frac(q[k][i][e]) * scale, fx_frac(q[k][i][e + 2]) * scale);
-          }
-    };
-    if constexpr (L::NTJ >= 2) chunk(std::integral_constant<int, 2>{}, 0);
-    if constexpr (L::NTJ % 2) chunk(std::integral_constant<int, 1>{}, L::NTJ - 1);
-  }
+        for (int e = 0; e < 2; ++e) {
+          const int j = 8 * (nt0 + i) + 2 * t + e;
+          if (!quad_new<N1>(k, j)) continue;
+          base[(long long)quad_pos<N1>(k, j) * s.n_col] =
+              mk(fx_frac(q[k][i][e]) * scale, fx_frac(q[k][i][e + 2]) * scale);
+        }
+  };
+  if constexpr (L::NTJ >= 2) chunk(std::integral_constant<int, 2>{}, 0);
+  if constexpr (L::NTJ % 2) chunk(std::integral_constant<int, 1>{}, L::NTJ - 1);
 }
 
 template <int N1, int S>
-__global__ void __launch_bounds__(32 * COLS_WARPS, 3)
+__global__ void __launch_bounds__(COLS_THREADS, 3)
     k_cols_fx_bwd(SphereDev<double> s, const cpx<double>* __restrict__ b1, ItemMap map, int n_items,
                   Epilogue<double> ep) {
   using L = FxLine<N1>;
+  // coefficients of the warps' lines at n and -n (element 2 (2 par + e) and the
+  // next) in units of their own scale
+  __shared__ __align__(16) cl coef[2 * COLS_PAIRS][8][32];
+  __shared__ int exps[2 * COLS_PAIRS];
   const int nl = listed_count(map);
-  const int units = (s.n_ucol + 7) / 8;
-  const long long unit = (long long)blockIdx.x * COLS_WARPS + (threadIdx.x >> 5);
-  const int item = (int)(unit / units);
-  if (item >= items_of(map, n_items, nl)) return;
+  const int units = (s.n_ucol + 7) / 8, warp = threadIdx.x >> 5, pair = warp >> 1, mirror = warp & 1;
+  const long long unit = (long long)blockIdx.x * COLS_PAIRS + pair;
+  int item = (int)(unit / units);
+  if ((long long)blockIdx.x * COLS_PAIRS / units >= items_of(map, n_items, nl)) return;
+  const bool any = item < items_of(map, n_items, nl);
+  if (!any) item = 0;
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int uc = (int)(unit - (long long)item * units) * 8 + g;
+  const int uc = any ? (int)(unit - (long long)item * units) * 8 + g : s.n_ucol;
   const UCol c = s.ucol[min(uc, s.n_ucol - 1)];
   const bool live = uc < s.n_ucol && ucol_in_range(s, c), self = c.col == c.mcol;
-  const cpx<double>* base = b1 + (long long)item * N1 * s.n_col;
-
-  // F[par][e][0 / 1]: the line's coefficients at +-n, n = 2 (2 t + e) + par
-  cpx<double> f[2][2][2][2];
-#pragma unroll
-  for (int mirror = 0; mirror < 2; ++mirror) {
+  {
     const bool use = live && !(mirror && self);
-    const cpx<double>* column = base + (mirror ? c.mcol : c.col);
+    const cpx<double>* column =
+        b1 + (long long)item * N1 * s.n_col + (mirror ? c.mcol : c.col);
     long long co[2][4], so[2][4];
 #pragma unroll
     for (int par = 0; par < 2; ++par)
@@ -218,59 +228,69 @@ __global__ void __launch_bounds__(32 * COLS_WARPS, 3)
     };
     if constexpr (L::NTJ >= 2) chunk(std::integral_constant<int, 2>{}, 0);
     if constexpr (L::NTJ % 2) chunk(std::integral_constant<int, 1>{}, L::NTJ / 2);
-    const double scale = er == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
-                                     : fx_unit(er - 1082 + 50 - SH_YB);
+    // one bit of headroom for the sum with the mirror line
 #pragma unroll
     for (int par = 0; par < 2; ++par)
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
-        f[mirror][par][e][0] = mk(fx_frac(co[par][e] + so[par][e]) * scale,
-                                  fx_frac(co[par][e + 2] + so[par][e + 2]) * scale);
-        f[mirror][par][e][1] = mk(fx_frac(co[par][e] - so[par][e]) * scale,
-                                  fx_frac(co[par][e + 2] - so[par][e + 2]) * scale);
+        coef[warp][2 * (2 * par + e)][lane] =
+            cl{(co[par][e] + so[par][e]) >> 1, (co[par][e + 2] + so[par][e + 2]) >> 1};
+        coef[warp][2 * (2 * par + e) + 1][lane] =
+            cl{(co[par][e] - so[par][e]) >> 1, (co[par][e + 2] - so[par][e + 2]) >> 1};
       }
+    if (lane == 0) exps[warp] = er;
   }
+  __syncthreads();
   if (!live) return;
-  // Hermitian unpacking of the two real fields and the epilogue
+  // Hermitian unpacking of the two real fields, both lines in the larger unit,
+  // and the epilogue: the first warp writes the members at n, the second those
+  // at -n
+  const int e0 = exps[2 * pair], e1 = exps[2 * pair + 1], em = max(e0, e1);
+  const int r0 = min(em - e0, 63), r1 = min(em - e1, 63);
+  const double fu = em == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
+                                : fx_unit(em - 1082 + 50 - SH_YB + 1) * ep.scale;
   const int ia = map.vec(item, 0, nl), ib = map.vec(item, 1, nl);
-  const double rs2 = 0.70710678118654752440084436210485 * ep.scale;
-  auto write = [&](int vec, int j, double val, double diag) {
-    if (vec < 0) return;
-    double* y = ep.y + (long long)vec * ep.ldy;
-    double r = val;
-    if (ep.x_in) {
-      const double sh = ep.shift ? ep.shift[vec % ep.shift_period] : 0.0;
-      r += (diag + sh) * ep.x_in[(long long)vec * ep.ldx + j];
-    }
+  double* ya = ia >= 0 ? ep.y + (long long)ia * ep.ldy : nullptr;
+  double* yb = ib >= 0 ? ep.y + (long long)ib * ep.ldy : nullptr;
+  const double* xa = ep.x_in && ia >= 0 ? ep.x_in + (long long)ia * ep.ldx : nullptr;
+  const double* xb = ep.x_in && ib >= 0 ? ep.x_in + (long long)ib * ep.ldx : nullptr;
+  const double sa = xa && ep.shift ? ep.shift[ia % ep.shift_period] : 0.0;
+  const double sb = xb && ep.shift ? ep.shift[ib % ep.shift_period] : 0.0;
+  auto write = [&](double* y, const double* x, int j, long long v, double cf, double diag) {
+    if (!y) return;
+    double r = cf * fx_frac(v);
+    if (x) r += diag * x[j];
     if (ep.beta != 0) r += ep.beta * y[j];
     y[j] = r;
   };
+  const int w0 = 2 * pair;
 #pragma unroll
-  for (int par = 0; par < 2; ++par)
-#pragma unroll
-    for (int e = 0; e < 2; ++e)
-#pragma unroll
-      for (int neg = 0; neg < 2; ++neg) {
-        const int n = 2 * (2 * t + e) + par;
-        if (n > c.R1 || (neg && (n == 0 || self))) continue;
-        const cpx<double> d = f[0][par][e][neg];
-        if (self && n == 0) {
-          const double cf = ep.coef == COEF_ONE ? ep.scale : 0.0;
-          write(ia, 2 * s.n_half, cf * d.x, 0.0);
-          write(ib, 2 * s.n_half, cf * d.y, 0.0);
-          continue;
-        }
-        // the mirror line at -n (the self-mirrored column's own)
-        const cpx<double> dm = self ? f[0][par][e][1] : f[1][par][e][1 - neg];
-        const int k = self ? c.h0 + n - 1 : c.h0 + (neg ? -n : n) + c.R1;
-        const double cf =
-            ep.coef == COEF_SQRT_COULOMB ? rs2 * sqrt(12.566370614359172953850573533118 / s.g2[k]) : rs2;
-        const double dg = ep.kin * s.kin[k];
-        write(ia, 2 * k, cf * (d.x + dm.x), dg);
-        write(ia, 2 * k + 1, cf * (d.y - dm.y), dg);
-        write(ib, 2 * k, cf * (d.y + dm.y), dg);
-        write(ib, 2 * k + 1, -(cf * (d.x - dm.x)), dg);
-      }
+  for (int q = 0; q < 4; ++q) {
+    const int n = 2 * (2 * t + (q & 1)) + (q >> 1);
+    if (n > c.R1 || (mirror && (n == 0 || self))) continue;
+    cl d = coef[w0][2 * q + mirror][lane];
+    d.x >>= r0;
+    d.y >>= r0;
+    if (self && n == 0) {
+      const double cf = ep.coef == COEF_ONE ? fu : 0.0;
+      write(ya, xa, 2 * s.n_half, d.x, cf, sa);
+      write(yb, xb, 2 * s.n_half, d.y, cf, sb);
+      continue;
+    }
+    // the mirror line at -n (the self-mirrored column's own)
+    cl dm = self ? coef[w0][2 * q + 1][lane] : coef[w0 + 1][2 * q + 1 - mirror][lane];
+    const int rm = self ? r0 : r1;
+    dm.x >>= rm;
+    dm.y >>= rm;
+    const int k = self ? c.h0 + n - 1 : c.h0 + (mirror ? -n : n) + c.R1;
+    double cf = fu * 0.70710678118654752440084436210485;
+    if (ep.coef == COEF_SQRT_COULOMB) cf *= sqrt(12.566370614359172953850573533118 / s.g2[k]);
+    const double dg = ep.kin != 0 ? s.kin[k] : 0.0;
+    write(ya, xa, 2 * k, d.x + dm.x, cf, dg + sa);
+    write(ya, xa, 2 * k + 1, d.y - dm.y, cf, dg + sa);
+    write(yb, xb, 2 * k, d.y + dm.y, cf, dg + sb);
+    write(yb, xb, 2 * k + 1, dm.x - d.x, cf, dg + sb);
+  }
 }
 
 template <int N1>
@@ -278,7 +298,7 @@ cudaError_t cols_fwd_fx_impl(const SphereDev<double>& s, const double* x, long l
                              const ItemMap& map, int n_items, int coef, cpx<double>* b1,
                              int digits, cudaStream_t st) {
   const long long units = (long long)n_items * ((s.n_ucol + 7) / 8);
-  const unsigned blocks = (unsigned)((units + COLS_WARPS - 1) / COLS_WARPS);
+  const unsigned blocks = (unsigned)((units + COLS_PAIRS - 1) / COLS_PAIRS);
   const double lines = (double)n_items * s.n_col;
   ProfScope ps(digits < FX_S ? PC_COLS_DF : PC_COLS_F64, st, lines * 5.0 * N1 * std::log2((double)N1),
                (double)n_items * 2.0 * s.n_pw * sizeof(double) + lines * N1 * 2.0 * sizeof(double),
@@ -287,14 +307,14 @@ cudaError_t cols_fwd_fx_impl(const SphereDev<double>& s, const double* x, long l
   auto kern = coef == COEF_SQRT_COULOMB ? k_cols_fx_fwd<N1, 8, true>
               : digits < FX_S           ? k_cols_fx_fwd<N1, 7, false>
                                         : k_cols_fx_fwd<N1, 8, false>;
-  kern<<<blocks, 32 * COLS_WARPS, 0, st>>>(s, x, ldx, map, n_items, b1);
+  kern<<<blocks, COLS_THREADS, 0, st>>>(s, x, ldx, map, n_items, b1);
   return cudaGetLastError();
 }
 template <int N1>
 cudaError_t cols_bwd_fx_impl(const SphereDev<double>& s, const cpx<double>* b1, const ItemMap& map,
                              int n_items, const Epilogue<double>& ep, int digits, cudaStream_t st) {
   const long long units = (long long)n_items * ((s.n_ucol + 7) / 8);
-  const unsigned blocks = (unsigned)((units + COLS_WARPS - 1) / COLS_WARPS);
+  const unsigned blocks = (unsigned)((units + COLS_PAIRS - 1) / COLS_PAIRS);
   const double lines = (double)n_items * s.n_col;
   const double vecs = (double)n_items * 2.0 * s.n_pw * sizeof(double);
   ProfScope ps(digits < FX_S ? PC_COLS_DF : PC_COLS_F64, st, lines * 5.0 * N1 * std::log2((double)N1),
@@ -303,7 +323,7 @@ cudaError_t cols_bwd_fx_impl(const SphereDev<double>& s, const cpx<double>* b1, 
                map.list ? map.n_dev : nullptr, map.n_list);
   count_launch();
   auto kern = digits < FX_S ? k_cols_fx_bwd<N1, 7> : k_cols_fx_bwd<N1, 8>;
-  kern<<<blocks, 32 * COLS_WARPS, 0, st>>>(s, b1, map, n_items, ep);
+  kern<<<blocks, COLS_THREADS, 0, st>>>(s, b1, map, n_items, ep);
   return cudaGetLastError();
 }
 
