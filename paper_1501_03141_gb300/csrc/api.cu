@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstring>
 #include <functional>
+#include <initializer_list>
 #include <map>
 #include <string>
 #include <type_traits>
@@ -236,6 +237,24 @@ cudaMemcpyKind kind_to_dev(const void* src) {
 }
 cudaMemcpyKind kind_from_dev(const void* dst) {
   return is_device_ptr(dst) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+}
+
+// Whether a call can work on the caller's arrays in place of staged copies: all
+// on the device, aligned for FP64 loads, and the written one apart from the read
+// ones (vectors that overlap were always accepted, through the copies).
+struct Span {
+  const void* p;
+  size_t bytes;
+};
+bool direct_io(const Span& out, std::initializer_list<Span> in) {
+  const char* o = (const char*)out.p;
+  if (!is_device_ptr(out.p) || ((uintptr_t)o & 7)) return false;
+  for (const Span& x : in) {
+    const char* q = (const char*)x.p;
+    if (!is_device_ptr(q) || ((uintptr_t)q & 7)) return false;
+    if (q < o + out.bytes && o < q + x.bytes) return false;
+  }
+  return true;
 }
 
 // host source -> host or device destination
@@ -506,8 +525,13 @@ constexpr int kFewItems = 38;  // a quarter of the SMs
 template <typename R>
 int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list, int n_list,
             bool with_shift, bool with_pv, cudaStream_t st, double* dn = nullptr,
-            const int* d_count = nullptr, bool refine = false) {
+            const int* d_count = nullptr, bool refine = false, long long ldx = 0,
+            long long ldy = 0) {
   const int digits = refine ? 7 : 8;
+  // row strides of X and Y (the library's own vectors: s.ld; others without
+  // the projection only)
+  if (!ldx) ldx = s.ld;
+  if (!ldy) ldy = s.ld;
   ItemMap map{n, (n + 1) / 2};
   int n_items = (n + 1) / 2;
   if (d_list) {
@@ -526,9 +550,9 @@ int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list,
     if (n_items > kFewItems && !dn && c->opt.fused_hpsi && hpsi_fused_smem(s.sf) > 0) {
       Epilogue<float> ep{};
       ep.y = Y;
-      ep.ldy = s.ld;
+      ep.ldy = ldy;
       ep.x_in = X;
-      ep.ldx = s.ld;
+      ep.ldx = ldx;
       ep.shift = with_shift ? s.d_negeps32 : nullptr;
       ep.shift_period = with_shift ? s.n_occ : 1;
       ep.scale = 1.0f / s.n_r;
@@ -542,7 +566,7 @@ int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list,
                             hpsi_fused_smem(s.sf, 2 * G0) ? 2 * G0 : G0};
       RET(tuned_call(c, "fused_planes:" + std::to_string(s.N[0]), 3, 0, 2.0 * n_items, st,
                      [&](int k) -> int {
-                       CK(launch_hpsi_fused(s.sf, X, s.ld, map, n_items, s.d_vf, ep, st, cands[k]));
+                       CK(launch_hpsi_fused(s.sf, X, ldx, map, n_items, s.d_vf, ep, st, cands[k]));
                        return PDEP_OK;
                      }));
       fused = true;
@@ -566,9 +590,9 @@ int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list,
     }
     Epilogue<R> ep{};
     ep.y = Y;
-    ep.ldy = s.ld;
+    ep.ldy = ldy;
     ep.x_in = X;
-    ep.ldx = s.ld;
+    ep.ldx = ldx;
     ep.shift = with_shift ? negeps_of(s, (R*)nullptr) : nullptr;
     ep.shift_period = with_shift ? s.n_occ : 1;
     ep.scale = R(1.0 / s.n_r);
@@ -577,12 +601,12 @@ int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list,
     ep.coef = COEF_ONE;
     if constexpr (std::is_same<R, float>::value) {
       a.v = s.d_vf;
-      CK(launch_cols_fwd(sd, X, s.ld, map, n_items, COEF_ONE, b1, st));
+      CK(launch_cols_fwd(sd, X, ldx, map, n_items, COEF_ONE, b1, st));
       CK(launch_slab(sd, a, st));
       CK(launch_cols_bwd(sd, b1, map, n_items, ep, st));
     } else {
       a.digits = digits;
-      CK(launch_cols_fwd(sd, X, s.ld, map, n_items, COEF_ONE, b1, st, digits));
+      CK(launch_cols_fwd(sd, X, ldx, map, n_items, COEF_ONE, b1, st, digits));
       CK(launch_slab(sd, a, st));
       CK(launch_cols_bwd(sd, b1, map, n_items, ep, st, digits));
     }
@@ -2072,30 +2096,46 @@ int pdep_screening_apply(pdep_ctx* c, int sys, int kind, const double* eigvals,
       return fail(PDEP_ERR_INVALID_ARG, "eigenvalue with lambda >= 1 or non-finite");
     g[i] = lam[i] / (1.0 - lam[i]);
   }
-  double *phi, *fx, *S, *dg, *o;
-  RET(ws(c, "sc_phi", (size_t)n_pdep * s.ld, &phi));
-  RET(ws(c, "sc_f", (size_t)n * s.ld, &fx));
-  RET(ws(c, "sc_o", (size_t)n * s.ld, &o));
+  const size_t vb = sizeof(double) * (size_t)dim;
+  const bool direct = direct_io({out, vb * n}, {{f, vb * n}, {eigvecs, vb * n_pdep}});
+  double *S, *dg;
   RET(ws(c, "sc_s", (size_t)n_pdep * n, &S));
   RET(ws(c, "sc_g", (size_t)n_pdep, &dg));
   CK(cudaMemcpyAsync(dg, g.data(), sizeof(double) * n_pdep, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpy2DAsync(phi, s.ld * sizeof(double), eigvecs, dim * sizeof(double),
-                       dim * sizeof(double), n_pdep, kind_to_dev(eigvecs), st));
-  CK(cudaMemcpy2DAsync(fx, s.ld * sizeof(double), f, dim * sizeof(double), dim * sizeof(double), n,
-                       kind_to_dev(f), st));
-  if (kind == PDEP_SCREEN_WP) CK(scale_sqrt_coulomb(fx, s.ld, s.n_half, n, s.sd.g2, st));
+  const double *phi = eigvecs, *fx = f;
+  double* o = out;
+  long long ld = dim;
+  if (!direct) {
+    double *sp, *sf;
+    ld = s.ld;
+    RET(ws(c, "sc_phi", (size_t)n_pdep * s.ld, &sp));
+    RET(ws(c, "sc_f", (size_t)n * s.ld, &sf));
+    RET(ws(c, "sc_o", (size_t)n * s.ld, &o));
+    CK(cudaMemcpy2DAsync(sp, s.ld * sizeof(double), eigvecs, vb, vb, n_pdep, kind_to_dev(eigvecs),
+                         st));
+    CK(cudaMemcpy2DAsync(sf, s.ld * sizeof(double), f, vb, vb, n, kind_to_dev(f), st));
+    phi = sp;
+    fx = sf;
+  }
+  if (kind == PDEP_SCREEN_WP) {
+    double* sf;
+    RET(ws(c, "sc_f", (size_t)n * s.ld, &sf));
+    CK(scale_sqrt_coulomb(sf, s.ld, fx, ld, s.n_half, n, s.sd.g2, st));
+    fx = sf;
+  }
   // S = Phi^T f, scaled per row by lambda/(1-lambda); out = Phi S (+ f)
-  CK(gemm<double>(true, n_pdep, n, dim, 1.0, phi, s.ld, fx, s.ld, 0.0, S, n_pdep, st));
+  const long long ldf = kind == PDEP_SCREEN_WP ? s.ld : ld;
+  CK(gemm<double>(true, n_pdep, n, dim, 1.0, phi, ld, fx, ldf, 0.0, S, n_pdep, st));
   CK(scale_rows<double>(S, n_pdep, n_pdep, n, dg, st));
   double beta = 0.0;
   if (kind == PDEP_SCREEN_EPSINV) {
-    CK(cudaMemcpyAsync(o, fx, sizeof(double) * (size_t)n * s.ld, cudaMemcpyDeviceToDevice, st));
+    CK(cudaMemcpyAsync(o, fx, sizeof(double) * (size_t)n * ld, cudaMemcpyDeviceToDevice, st));
     beta = 1.0;
   }
-  CK(gemm<double>(false, dim, n, n_pdep, 1.0, phi, s.ld, S, n_pdep, beta, o, s.ld, st));
-  if (kind == PDEP_SCREEN_WP) CK(scale_sqrt_coulomb(o, s.ld, s.n_half, n, s.sd.g2, st));
-  CK(cudaMemcpy2DAsync(out, dim * sizeof(double), o, s.ld * sizeof(double), dim * sizeof(double),
-                       n, kind_from_dev(out), st));
+  CK(gemm<double>(false, dim, n, n_pdep, 1.0, phi, ld, S, n_pdep, beta, o, ld, st));
+  if (kind == PDEP_SCREEN_WP) CK(scale_sqrt_coulomb(o, ld, o, ld, s.n_half, n, s.sd.g2, st));
+  if (!direct)
+    CK(cudaMemcpy2DAsync(out, vb, o, s.ld * sizeof(double), vb, n, kind_from_dev(out), st));
   RET(sync(st));
   return PDEP_OK;
 }
@@ -2407,26 +2447,36 @@ int pdep_apply_hamiltonian(pdep_ctx* c, int sys, const double* x, int n, double*
   if (n == 0) return PDEP_OK;
   cudaStream_t st = (cudaStream_t)stream;
   SysData& s = c->sys[sys];
-  double *in, *outv;
-  RET(ws(c, "api_in", (size_t)n * s.ld, &in));
-  RET(ws(c, "api_out", (size_t)n * s.ld, &outv));
-  CK(cudaMemsetAsync(in, 0, sizeof(double) * (size_t)n * s.ld, st));
-  CK(cudaMemcpy2DAsync(in, s.ld * sizeof(double), x, s.n_pw * sizeof(double),
-                       s.n_pw * sizeof(double), n, kind_to_dev(x), st));
-  if (precision == PDEP_FP64) {
-    RET(apply_h<double>(c, s, in, outv, n, nullptr, 0, false, false, st));
-  } else if (precision == PDEP_APPLY_DF64) {
-    RET(apply_h<double>(c, s, in, outv, n, nullptr, 0, false, false, st, nullptr, nullptr, true));
+  const size_t bytes = sizeof(double) * (size_t)n * s.n_pw;
+  const bool direct = direct_io({y, bytes}, {{x, bytes}});
+  // rows n_pw apart in the caller's arrays, s.ld apart in staged ones
+  const double* in = x;
+  double* outv = y;
+  long long ld = s.n_pw;
+  if (!direct) {
+    double *si, *so;
+    ld = s.ld;
+    RET(ws(c, "api_in", (size_t)n * s.ld, &si));
+    RET(ws(c, "api_out", (size_t)n * s.ld, &so));
+    CK(cudaMemcpy2DAsync(si, s.ld * sizeof(double), x, s.n_pw * sizeof(double),
+                         s.n_pw * sizeof(double), n, kind_to_dev(x), st));
+    in = si;
+    outv = so;
+  }
+  if (precision == PDEP_FP64 || precision == PDEP_APPLY_DF64) {
+    RET(apply_h<double>(c, s, in, outv, n, nullptr, 0, false, false, st, nullptr, nullptr,
+                        precision == PDEP_APPLY_DF64, ld, ld));
   } else {
     float *in32, *out32;
     RET(ws(c, "api_in32", (size_t)n * s.ld, &in32));
     RET(ws(c, "api_out32", (size_t)n * s.ld, &out32));
-    CK((convert<float, double>(in32, s.ld, in, s.ld, s.ld, n, st)));
+    CK((convert<float, double>(in32, s.ld, in, ld, s.n_pw, n, st)));
     RET(apply_h<float>(c, s, in32, out32, n, nullptr, 0, false, false, st));
-    CK((convert<double, float>(outv, s.ld, out32, s.ld, s.n_pw, n, st)));
+    CK((convert<double, float>(outv, ld, out32, s.ld, s.n_pw, n, st)));
   }
-  CK(cudaMemcpy2DAsync(y, s.n_pw * sizeof(double), outv, s.ld * sizeof(double),
-                       s.n_pw * sizeof(double), n, kind_from_dev(y), st));
+  if (!direct)
+    CK(cudaMemcpy2DAsync(y, s.n_pw * sizeof(double), outv, s.ld * sizeof(double),
+                         s.n_pw * sizeof(double), n, kind_from_dev(y), st));
   return sync(st);
 }
 
@@ -2436,17 +2486,25 @@ int pdep_to_grid(pdep_ctx* c, int sys, const double* x, int n, double* u, void* 
   if (n == 0) return PDEP_OK;
   cudaStream_t st = (cudaStream_t)stream;
   SysData& s = c->sys[sys];
-  double *in, *grid;
-  RET(ws(c, "api_in", (size_t)n * s.ld, &in));
-  RET(ws(c, "api_grid", (size_t)n * s.n_r, &grid));
-  CK(cudaMemsetAsync(in, 0, sizeof(double) * (size_t)n * s.ld, st));
-  CK(cudaMemcpy2DAsync(in, s.ld * sizeof(double), x, s.n_pw * sizeof(double),
-                       s.n_pw * sizeof(double), n, kind_to_dev(x), st));
+  const bool direct = direct_io({u, sizeof(double) * (size_t)n * s.n_r},
+                                {{x, sizeof(double) * (size_t)n * s.n_pw}});
+  const double* in = x;
+  double* grid = u;
+  long long ld = s.n_pw;
+  if (!direct) {
+    double* si;
+    ld = s.ld;
+    RET(ws(c, "api_in", (size_t)n * s.ld, &si));
+    RET(ws(c, "api_grid", (size_t)n * s.n_r, &grid));
+    CK(cudaMemcpy2DAsync(si, s.ld * sizeof(double), x, s.n_pw * sizeof(double),
+                         s.n_pw * sizeof(double), n, kind_to_dev(x), st));
+    in = si;
+  }
   ItemMap map{n, (n + 1) / 2};
   const int n_items = (n + 1) / 2;
   cpx<double>* b1;
   RET(ws(c, "b1_64", b1_count(s, n_items), &b1));
-  CK(launch_cols_fwd(s.sd, in, s.ld, map, n_items, COEF_ONE, b1, st));
+  CK(launch_cols_fwd(s.sd, in, ld, map, n_items, COEF_ONE, b1, st));
   SlabArgs<double> a{};
   a.mode = SLAB_TO_GRID;
   a.b1 = b1;
@@ -2456,7 +2514,8 @@ int pdep_to_grid(pdep_ctx* c, int sys, const double* x, int n, double* u, void* 
   a.out_scale = 1.0;
   a.map = map;
   CK(launch_slab(s.sd, a, st));
-  CK(cudaMemcpyAsync(u, grid, sizeof(double) * (size_t)n * s.n_r, kind_from_dev(u), st));
+  if (!direct)
+    CK(cudaMemcpyAsync(u, grid, sizeof(double) * (size_t)n * s.n_r, kind_from_dev(u), st));
   return sync(st);
 }
 

@@ -514,24 +514,21 @@ cudaError_t symmetrize(R* M, int n, long long ld, cudaStream_t st) {
 }
 template cudaError_t symmetrize<double>(double*, int, long long, cudaStream_t);
 
+// one column per blockIdx.y (strided), its rows over blockIdx.x: no division
 template <typename Rd, typename Rs>
 __global__ void k_convert(Rd* dst, long long ldd, const Rs* __restrict__ src, long long lds,
                           int rows, int cols) {
-  const long long tot = (long long)rows * cols;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(e % rows), c = (int)(e / rows);
-    dst[r + (long long)c * ldd] = (Rd)src[r + (long long)c * lds];
-  }
+  for (int c = blockIdx.y; c < cols; c += gridDim.y)
+    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += gridDim.x * blockDim.x)
+      dst[r + (long long)c * ldd] = (Rd)src[r + (long long)c * lds];
 }
 template <typename Rd, typename Rs>
 cudaError_t convert(Rd* dst, long long ldd, const Rs* src, long long lds, int rows, int cols,
                     cudaStream_t st) {
-  const long long tot = (long long)rows * cols;
-  if (tot == 0) return cudaSuccess;
-  const int blocks = (int)std::min<long long>((tot + 255) / 256, 8192);
+  if (rows <= 0 || cols <= 0) return cudaSuccess;
+  const dim3 grid(std::min((rows + 255) / 256, 4096), std::min(cols, 65535));
   count_launch();
-  k_convert<Rd, Rs><<<blocks, 256, 0, st>>>(dst, ldd, src, lds, rows, cols);
+  k_convert<Rd, Rs><<<grid, 256, 0, st>>>(dst, ldd, src, lds, rows, cols);
   return cudaGetLastError();
 }
 template cudaError_t convert<double, double>(double*, long long, const double*, long long, int, int,
@@ -743,23 +740,25 @@ cudaError_t cholesky_winv(const double* G, int m, double rel_thr, double* W, int
   return cudaGetLastError();
 }
 
-// X[d][j] *= sqrt(4 pi / |G_{d/2}|^2) for the 2 n_half PDEP components d
-// (v^{1/2} of Eq. symmoperator on the real-coefficient layout)
-__global__ void k_sqrt_coulomb(double* X, long long ld, int n_half, int n,
+// Y[d][j] = X[d][j] sqrt(4 pi / |G_{d/2}|^2) for the 2 n_half PDEP components d
+// (v^{1/2} of Eq. symmoperator on the real-coefficient layout); Y may be X
+__global__ void k_sqrt_coulomb(double* Y, long long ldy, const double* X, long long ldx, int n_half,
                                const double* __restrict__ g2) {
   const int j = blockIdx.y;
   const int dim = 2 * n_half;
   for (int d = blockIdx.x * blockDim.x + threadIdx.x; d < dim; d += gridDim.x * blockDim.x)
-    X[d + (long long)j * ld] *= sqrt(4.0 * 3.14159265358979323846 / g2[d >> 1]);
+    Y[d + (long long)j * ldy] =
+        X[d + (long long)j * ldx] * sqrt(4.0 * 3.14159265358979323846 / g2[d >> 1]);
 }
-cudaError_t scale_sqrt_coulomb(double* X, long long ld, int n_half, int n, const double* g2,
-                               cudaStream_t st) {
+cudaError_t scale_sqrt_coulomb(double* Y, long long ldy, const double* X, long long ldx, int n_half,
+                               int n, const double* g2, cudaStream_t st) {
   if (n <= 0 || n_half <= 0) return cudaSuccess;
   const int bx = std::min((2 * n_half + 255) / 256, 64);
   for (int j0 = 0; j0 < n; j0 += 65535) {
     const int nj = std::min(65535, n - j0);
     count_launch();
-    k_sqrt_coulomb<<<dim3(bx, nj), 256, 0, st>>>(X + (long long)j0 * ld, ld, n_half, nj, g2);
+    k_sqrt_coulomb<<<dim3(bx, nj), 256, 0, st>>>(Y + (long long)j0 * ldy, ldy,
+                                                 X + (long long)j0 * ldx, ldx, n_half, g2);
   }
   return cudaGetLastError();
 }

@@ -81,9 +81,10 @@ cudaError_t ritz_residual(const double* AX, const double* X, long long ld, int r
                           const double* theta, double* Rout, cudaStream_t st);
 cudaError_t philox_normal(double* X, long long ld, int rows, int cols, unsigned long long seed,
                           unsigned long long offset, cudaStream_t st);
-// X[d][j] *= sqrt(4 pi)/|G| on the 2 n_half PDEP components of n columns
-cudaError_t scale_sqrt_coulomb(double* X, long long ld, int n_half, int n, const double* g2,
-                               cudaStream_t st);
+// Y[d][j] = X[d][j] sqrt(4 pi)/|G| on the 2 n_half PDEP components of n columns
+// (Y may be X)
+cudaError_t scale_sqrt_coulomb(double* Y, long long ldy, const double* X, long long ldx, int n_half,
+                               int n, const double* g2, cudaStream_t st);
 // Lanczos chains (Sec. II D), Q_k blocks [n][ld], alpha/beta [n][K]:
 // q_0 = r/||r|| and beta[j][0] = ||r||; one three-term step per call; the
 // tridiagonal eigen-decompositions (K <= 64; d ascending, U[j][m][k]); the
