@@ -131,32 +131,31 @@ __global__ void __launch_bounds__(T)
       }
     }
     if constexpr (PROJ) {
-      // S_w = sigma_w <w|p> over the cluster, then A p += sum_w S_w |w>
-      __shared__ R part[CG_PROJ_MAX][T / 32];
+      // S_w = sigma_w <w|p> over the cluster, then A p += sum_w S_w |w>.  The
+      // block's stripe of p goes through shared memory and each warp takes whole
+      // states of it: a warp sum per state and block instead of one per warp
+      // (in FP64 its five additions take 320 clocks)
+      __shared__ __align__(16) R stripe[T * V * E];
       __shared__ R S[CG_PROJ_MAX], sums[CG_PROJ_MAX];
-#pragma unroll 4
-      for (int w = 0; w < pj.n; ++w) {
+#pragma unroll
+      for (int v = 0; v < V; ++v) Vec<R>::st(stripe + (v * T + tid) * E, pv[v]);
+      __syncthreads();
+      for (int w = tid >> 5; w < pj.n; w += T / 32) {
         const R* P = pj.states + (long long)w * a.ld;
         R d = R(0);
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-          const int j = ((v * C + rank) * T + tid) * E;
+#pragma unroll 4
+        for (int q = tid & 31; q < T * V; q += 32) {
+          const int j = ((q / T * C + rank) * T + q % T) * E;
           if (j < a.n_pw) {
-            R q[E];
-            Vec<R>::ld(P + j, q);
+            R x[E], y[E];
+            Vec<R>::ld(P + j, x);
+            Vec<R>::ld(stripe + q * E, y);
 #pragma unroll
-            for (int e = 0; e < E; ++e) d += q[e] * pv[v][e];
+            for (int e = 0; e < E; ++e) d += x[e] * y[e];
           }
         }
         d = warp_sum(d);
-        if ((tid & 31) == 0) part[w][tid >> 5] = d;
-      }
-      __syncthreads();
-      for (int w = tid; w < pj.n; w += T) {
-        R t = R(0);
-#pragma unroll
-        for (int k = 0; k < T / 32; ++k) t += part[w][k];
-        sums[w] = t;
+        if ((tid & 31) == 0) sums[w] = d;
       }
       if (C > 1)
         cl.sync();
