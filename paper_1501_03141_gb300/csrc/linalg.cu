@@ -274,18 +274,48 @@ __global__ void k_jacobi_init(const double* __restrict__ M, long long ldm, int n
   }
 }
 
-// One round of the cyclic (round-robin) ordering, one CTA of two warps per
+// Start of a sweep: the column weights go into the columns (weight 1) and the
+// squared norms are summed anew.
+__global__ void k_jacobi_sweep_start(double* A, int n, double* __restrict__ wt,
+                                     double* __restrict__ norm, int first) {
+  const int c = blockIdx.x;
+  const double f = first ? 1.0 : sqrt(wt[c]);
+  double ss = 0.0;
+  for (int r = threadIdx.x; r < n; r += blockDim.x) {
+    const double v = f * A[r + (long long)c * n];
+    A[r + (long long)c * n] = v;
+    ss += v * v;
+  }
+  const double2 t = block_sum2(ss, 0.0);
+  if (threadIdx.x == 0) {
+    wt[c] = 1.0;
+    norm[c] = t.x;
+  }
+}
+
+// One round of the cyclic (round-robin) ordering, one CTA of T threads per
 // column pair (p, q): the pair is rotated so that A_p . A_q = 0.  V is not
 // carried: at convergence the columns of A = (M - sigma I) V are the
 // eigenvectors scaled by lambda_i - sigma, and with sigma twice the
 // Gershgorin bound every |lambda_i - sigma| lies in [sigma/2, 3 sigma/2]
 // (condition number at most 3), so normalising them gives V to working
-// accuracy.  E > 0: the
-// two columns (n <= 64 E) are held in registers, one memory round trip per
-// round; E = 0 streams them.
-template <int E>
-__global__ void __launch_bounds__(64) k_jacobi_pair(double* A, int n, int nn, int round,
-                                                    unsigned* counter) {
+// accuracy.  E > 0: the two columns (n <= T E) are held in registers, one
+// memory round trip per round; E = 0 streams them.
+//
+// Bound by the FP64 pipe (an instruction of a warp takes 64 clocks of its
+// sub-partition's), so a rotation uses as few FP64 operations as it can: fast
+// rotations (Gentleman, J. Inst. Math. Appl. 12, 329 (1973)), P' = P - a Q and
+// Q' = Q + b P with the columns' weights W (true column = sqrt(W) P) instead of
+// c and s; the squared true norms N follow from the rotation instead of two
+// more dot products; and the angle comes from FP32: any k gives an exactly
+// orthogonal rotation a = W_q k, b = W_p k, W' = W / (1 + a b), and one that is
+// right to 1e-7 leaves the pair 1e-7 of its product for the next sweep.  With
+// the squares and square root, two dot products and c, s rotation in FP64 a
+// round of 64 columns took 4.6 us and a 768-column eigenproblem's sweep 3.5 ms.
+template <int E, int T>
+__global__ void __launch_bounds__(T) k_jacobi_pair(double* A, int n, int nn, int round,
+                                                   double* __restrict__ wt,
+                                                   double* __restrict__ norm, unsigned* counter) {
   const int pair = blockIdx.x;
   int p, q;
   if (pair == 0) {
@@ -298,75 +328,84 @@ __global__ void __launch_bounds__(64) k_jacobi_pair(double* A, int n, int nn, in
   if (p >= n || q >= n) return;
   double* ap = A + (long long)p * n;
   double* aq = A + (long long)q * n;
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  __shared__ double red[2][3];
-  double al = 0.0, be = 0.0, ga = 0.0;
+  const int t = threadIdx.x;
+  const double Wp = wt[p], Wq = wt[q], Np = norm[p], Nq = norm[q];
+  double u = 0.0;
   double x[E > 0 ? E : 1], y[E > 0 ? E : 1];
   if constexpr (E > 0) {
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-      const int r = t + 64 * e;
+      const int r = t + T * e;
       const bool in = r < n;
       x[e] = in ? ap[r] : 0.0;
       y[e] = in ? aq[r] : 0.0;
     }
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      al += x[e] * x[e];
-      be += y[e] * y[e];
-      ga += x[e] * y[e];
-    }
+    for (int e = 0; e < E; ++e) u += x[e] * y[e];
   } else {
-    for (int r = t; r < n; r += 64) {
-      const double u = ap[r], w = aq[r];
-      al += u * u;
-      be += w * w;
-      ga += u * w;
-    }
+    for (int r = t; r < n; r += T) u += ap[r] * aq[r];
   }
-  al = warp_sum(al);
-  be = warp_sum(be);
-  ga = warp_sum(ga);
-  if (lane == 0) {
-    red[warp][0] = al;
-    red[warp][1] = be;
-    red[warp][2] = ga;
+  u = warp_sum(u);
+  if constexpr (T > 32) {
+    __shared__ double red[T / 32];
+    if ((t & 31) == 0) red[t >> 5] = u;
+    __syncthreads();
+    u = red[0];
+#pragma unroll
+    for (int w = 1; w < T / 32; ++w) u += red[w];
   }
-  __syncthreads();
-  al = red[0][0] + red[1][0];
-  be = red[0][1] + red[1][1];
-  ga = red[0][2] + red[1][2];
-  // every thread holds the same sums, so this exit is uniform
-  if (ga == 0.0 || ga * ga <= 1e-28 * (al * be)) return;
-  const double zeta = (be - al) / (2.0 * ga);
-  const double tt = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-  const double c = rsqrt(1.0 + tt * tt);
-  const double s = c * tt;
+  // every thread holds the same sums, so this exit is uniform; g2 is the square
+  // of the true columns' product
+  const double wu = Wp * u, g2 = wu * u * Wq;
+  if (g2 == 0.0 || g2 <= 1e-28 * (Np * Nq)) return;
+  // k = u / (X + sgn(X) sqrt(X^2 + g2)), X = (N_q - N_p) / 2, by FP32 numbers
+  // scaled by the larger of |X| and sqrt(g2)
+  const double X = 0.5 * (Nq - Np);
+  const int ex = (__double2hiint(X) >> 20) & 0x7ff, eg = (__double2hiint(g2) >> 20) & 0x7ff;
+  const int sc = min(max(1023 - max(ex, (eg + 1023) / 2), -1000), 1000);  // 2^sc scales X
+  const double s1 = __hiloint2double((1023 + sc) << 20, 0);
+  const float xf = (float)(X * s1), gf = (float)(g2 * s1 * s1);
+  const float den = xf + copysignf(sqrtf(xf * xf + gf), xf);
+  const double k = u * ((double)(1.0f / den) * s1);
+  const double a = Wq * k, b = Wp * k;
   if constexpr (E > 0) {
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-      const int r = t + 64 * e;
+      const int r = t + T * e;
       if (r < n) {
-        ap[r] = c * x[e] - s * y[e];
-        aq[r] = s * x[e] + c * y[e];
+        ap[r] = x[e] - a * y[e];
+        aq[r] = y[e] + b * x[e];
       }
     }
   } else {
-    for (int r = t; r < n; r += 64) {
-      const double u = ap[r], w = aq[r];
-      ap[r] = c * u - s * w;
-      aq[r] = s * u + c * w;
+    for (int r = t; r < n; r += T) {
+      const double v = ap[r], w = aq[r];
+      ap[r] = v - a * w;
+      aq[r] = w + b * v;
     }
   }
-  if (t == 0) atomicAdd(counter, 1u);
+  if (t == 0) {
+    const double f = 1.0 / (1.0 + a * b), d = wu * a;  // d = t ga
+    wt[p] = Wp * f;
+    wt[q] = Wq * f;
+    norm[p] = Np - d;
+    norm[q] = Nq + d;
+    atomicAdd(counter, 1u);
+  }
 }
 
-using JacobiRound = void (*)(double*, int, int, int, unsigned*);
-static JacobiRound jacobi_round_for(int n) {
-  if (n <= 128) return k_jacobi_pair<2>;
-  if (n <= 256) return k_jacobi_pair<4>;
-  if (n <= 512) return k_jacobi_pair<8>;
-  return k_jacobi_pair<0>;
+using JacobiRound = void (*)(double*, int, int, int, double*, double*, unsigned*);
+// one warp per pair leaves each FP64 pipe one pair up to 608 pairs; two halve a
+// short pair's chain
+static JacobiRound jacobi_round_for(int n, int* threads) {
+  *threads = n <= 512 ? 64 : 32;
+  if (n <= 64) return k_jacobi_pair<1, 64>;
+  if (n <= 128) return k_jacobi_pair<2, 64>;
+  if (n <= 256) return k_jacobi_pair<4, 64>;
+  if (n <= 512) return k_jacobi_pair<8, 64>;
+  if (n <= 768) return k_jacobi_pair<24, 32>;
+  *threads = 64;
+  return k_jacobi_pair<0, 64>;
 }
 
 // V_i = -A_i / ||A_i|| (one block per column)
@@ -429,14 +468,17 @@ cudaError_t eigh(int n, const double* M, long long ldm, double* W, double* V, lo
   k_jacobi_init<<<blocks, 256, 0, st>>>(M, ldm, n, sigma, wk.a);
   const int nn = n + (n & 1);
   const int jb = nn / 2;  // one CTA per column pair
-  const int tpb = 64;
-  const JacobiRound round_k = jacobi_round_for(n);
+  int tpb = 64;
+  const JacobiRound round_k = jacobi_round_for(n, &tpb);
+  // column weights and squared norms: the tail of the scratch, unused until the
+  // sweeps are done (n >= 2; a single column needs neither)
+  double *wt = wk.tmp, *norm = wk.tmp + n;
   // One sweep = nn - 1 dependent rounds; they are replayed from a CUDA graph
   // captured once per (size, buffers) to avoid nn - 1 stream launches.
   cudaGraphExec_t sweep = nullptr;
   if (nn - 1 > 8 && wk.graphs) {
     for (const EighGraphCache::Entry& k : wk.graphs->entries)
-      if (k.n == n && k.a == wk.a && k.counter == counter) sweep = k.exec;
+      if (k.n == n && k.a == wk.a && k.tmp == wk.tmp && k.counter == counter) sweep = k.exec;
     if (!sweep) {
       cudaStream_t cap;
       cudaError_t e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
@@ -444,20 +486,23 @@ cudaError_t eigh(int n, const double* M, long long ldm, double* W, double* V, lo
       cudaGraph_t g = nullptr;
       e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
-        for (int r = 0; r < nn - 1; ++r) round_k<<<jb, tpb, 0, cap>>>(wk.a, n, nn, r, counter);
+        for (int r = 0; r < nn - 1; ++r) round_k<<<jb, tpb, 0, cap>>>(wk.a, n, nn, r, wt, norm, counter);
         e = cudaStreamEndCapture(cap, &g);
       }
       if (e == cudaSuccess) e = cudaGraphInstantiate(&sweep, g, 0);
       if (g) cudaGraphDestroy(g);
       cudaStreamDestroy(cap);
       if (e != cudaSuccess) return e;
-      wk.graphs->entries.push_back(EighGraphCache::Entry{n, wk.a, counter, sweep});
+      wk.graphs->entries.push_back(EighGraphCache::Entry{n, wk.a, wk.tmp, counter, sweep});
     }
   }
   unsigned hcount = 1;
   for (int sweep_i = 0; sweep_i < max_sweeps && hcount != 0; ++sweep_i) {
+    if (nn - 1 == 0) break;
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), st);
     if (e != cudaSuccess) return e;
+    count_launch();
+    k_jacobi_sweep_start<<<n, 128, 0, st>>>(wk.a, n, wt, norm, sweep_i == 0 ? 1 : 0);
     if (sweep) {
       for (int r = 0; r < nn - 1; ++r) count_launch();
       e = cudaGraphLaunch(sweep, st);
@@ -465,10 +510,9 @@ cudaError_t eigh(int n, const double* M, long long ldm, double* W, double* V, lo
     } else {
       for (int r = 0; r < nn - 1; ++r) {
         count_launch();
-        round_k<<<jb, tpb, 0, st>>>(wk.a, n, nn, r, counter);
+        round_k<<<jb, tpb, 0, st>>>(wk.a, n, nn, r, wt, norm, counter);
       }
     }
-    if (nn - 1 == 0) break;
     e = cudaMemcpyAsync(&hcount, counter, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
     if (e != cudaSuccess) return e;
     e = cudaStreamSynchronize(st);

@@ -45,6 +45,7 @@ struct EighGraphCache {
   struct Entry {
     int n;
     const void* a;
+    const void* tmp;
     const void* counter;
     cudaGraphExec_t exec;
   };
