@@ -396,10 +396,21 @@ __device__ __forceinline__ void y_forward(const SphereDev<float>& s, const cpx<f
   }
 }
 
-// one x-plane i1 of one item
-template <int N2, int N3>
+// FP32 to FP64 on the integer pipe (an FP64 conversion of a warp takes 64 clocks
+// of its pipe); subnormal and non-finite values by the conversion
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x), e = (b >> 23) & 0xffu;
+  if (e - 1u >= 254u) return (double)x;
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))),
+                          (int)(b << 29));
+}
+
+// one x-plane i1 of one item; DN: its density response is added to acc (this
+// thread's positions of its z-line)
+template <int N2, int N3, bool DN>
 __device__ __forceinline__ void slab_unit(const SphereDev<float>& s, const SlabArgs<float>& a, int nl,
-                                          int item, int i1, cpx<float>* S1, cpx<float>* T2) {
+                                          int item, int i1, cpx<float>* S1, cpx<float>* T2,
+                                          double* acc) {
   constexpr int TL3 = Tpl<float, N3>::v;
   constexpr int M3 = N3 / TL3;
   constexpr int TS = T2Stride<N2>::v;
@@ -458,36 +469,24 @@ __device__ __forceinline__ void slab_unit(const SphereDev<float>& s, const SlabA
         }
         continue;
       }
-      {
-        if (a.dn && act) {
-          // density response of the two vectors of the item on this z-line
-          // (Eq. deltani), accumulated over the occupied states v
-          const int ia = a.map.vec(item, 0, nl), ib = a.map.vec(item, 1, nl);
-          const long long off = plane + (long long)i2 * N3;
-          const int ja = ia / a.dn_nocc, vb_a = ia - ja * a.dn_nocc;
-          const double* ua = a.u + (long long)vb_a * a.dn_stride + off;
-          double* da = a.dn + (long long)ja * a.dn_stride + off;
-          const int jb = ib >= 0 ? ib / a.dn_nocc : -1;
-          const double* ub = ib >= 0 ? a.u + (long long)(ib - jb * a.dn_nocc) * a.dn_stride + off
-                                     : nullptr;
-          double* db = ib >= 0 ? a.dn + (long long)jb * a.dn_stride + off : nullptr;
-          const double sc = a.dn_scale;
+      if (DN && act) {
+        // density response of the two vectors of the item on this z-line
+        // (Eq. deltani), summed over the items of one perturbation
+        const int ia = a.map.vec(item, 0, nl), ib = a.map.vec(item, 1, nl);
+        const long long off = plane + (long long)i2 * N3;
+        const int ja = ia / a.dn_nocc, jb = ib >= 0 ? ib / a.dn_nocc : -1;
+        const double* ua = a.u + (long long)(ia - ja * a.dn_nocc) * a.dn_stride + off;
+        const double* ub = ib >= 0 ? a.u + (long long)(ib - jb * a.dn_nocc) * a.dn_stride + off : ua;
+        const bool same = jb == ja;
 #pragma unroll
-          for (int i = 0; i < M3; ++i) {
-            const int i3 = pos_b<N3, TL3>(t3, i);
-            const double ca = sc * (double)v[i].x * ua[i3];
-            if (ub) {
-              const double cb = sc * (double)v[i].y * ub[i3];
-              if (jb == ja) {
-                atomicAdd(da + i3, ca + cb);
-              } else {
-                atomicAdd(da + i3, ca);
-                atomicAdd(db + i3, cb);
-              }
-            } else {
-              atomicAdd(da + i3, ca);
-            }
-          }
+        for (int i = 0; i < M3; ++i) {
+          const int i3 = pos_b<N3, TL3>(t3, i);
+          acc[i] = fma(widen(v[i].x), ua[i3], acc[i]);
+          const double xb = widen(v[i].y);
+          if (same)
+            acc[i] = fma(xb, ub[i3], acc[i]);
+          else if (ib >= 0)
+            atomicAdd(a.dn + (long long)jb * a.dn_stride + off + i3, a.dn_scale * (xb * ub[i3]));
         }
       }
       // SLAB_HPSI: multiply by the local potential on the grid
@@ -513,21 +512,58 @@ __device__ __forceinline__ void slab_unit(const SphereDev<float>& s, const SlabA
 
 // A persistent grid of the resident blocks strides over the (item, plane)
 // units, so a launch sized for a whole batch whose device count has shrunk
-// costs no empty blocks.
-template <int N2, int N3>
+// costs no empty blocks.  DN: a unit is 'group' items of one plane, whose
+// density response stays in registers until the perturbation changes: the FP64
+// pipe's conversions and products and an atomic per point bound this form (the
+// slab passes of one application to 128 perturbations on 48^3: 8.0 ms with two
+// conversions, four operations and an atomic per point and item, 5.4 ms with
+// two multiply-adds).
+template <int N2, int N3, bool DN>
 __global__ void __launch_bounds__(SlabThreads<N2, N3>::v, (SlabMinBlocks<N2, N3>::v))
-    k_slab(SphereDev<float> s, SlabArgs<float> a) {
+    k_slab(SphereDev<float> s, SlabArgs<float> a, int group) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<float>* S1 = reinterpret_cast<cpx<float>*>(smem_raw);
   cpx<float>* T2 = S1 + s.n_col;
   const int nl = listed_count(a.map);
   const int n_items = items_of(a.map, a.n_items, nl);
-  const int units = n_items * s.N1;
+  if constexpr (!DN) {
+    const int units = n_items * s.N1;
 #pragma unroll 1
-  for (int w = blockIdx.x; w < units; w += gridDim.x) {
-    const int item = w / s.N1;
-    __syncthreads();  // the previous unit's shared-memory reads are done
-    slab_unit<N2, N3>(s, a, nl, item, w - item * s.N1, S1, T2);
+    for (int w = blockIdx.x; w < units; w += gridDim.x) {
+      const int item = w / s.N1;
+      __syncthreads();  // the previous unit's shared-memory reads are done
+      slab_unit<N2, N3, false>(s, a, nl, item, w - item * s.N1, S1, T2, nullptr);
+    }
+  } else {
+    constexpr int TL3 = Tpl<float, N3>::v, M3 = N3 / TL3;
+    const int t3 = threadIdx.x & (TL3 - 1), i2 = threadIdx.x / TL3;
+    const int units = (n_items + group - 1) / group * s.N1;
+    double acc[M3];
+#pragma unroll
+    for (int i = 0; i < M3; ++i) acc[i] = 0.0;
+#pragma unroll 1
+    for (int w = blockIdx.x; w < units; w += gridDim.x) {
+      const int g0 = w / s.N1 * group, i1 = w % s.N1;
+      auto flush = [&](int j) {
+        if (i2 >= N2) return;
+        double* dn = a.dn + (long long)j * a.dn_stride + ((long long)i1 * N2 + i2) * N3;
+#pragma unroll
+        for (int i = 0; i < M3; ++i) {
+          atomicAdd(dn + pos_b<N3, TL3>(t3, i), a.dn_scale * acc[i]);
+          acc[i] = 0.0;
+        }
+      };
+      int cur = -1;
+#pragma unroll 1
+      for (int item = g0; item < min(n_items, g0 + group); ++item) {
+        const int j = a.map.vec(item, 0, nl) / a.dn_nocc;
+        if (cur >= 0 && j != cur) flush(cur);
+        cur = j;
+        __syncthreads();
+        slab_unit<N2, N3, true>(s, a, nl, item, i1, S1, T2, acc);
+      }
+      if (cur >= 0) flush(cur);
+    }
   }
 }
 
@@ -741,14 +777,15 @@ static cudaError_t cols_bwd_impl(const SphereDev<R>& s, const cpx<R>* b1, ItemMa
   return cudaGetLastError();
 }
 
-template <int N2, int N3>
-static cudaError_t slab_impl(const SphereDev<float>& s, const SlabArgs<float>& a, cudaStream_t st) {
+template <int N2, int N3, bool DN>
+static cudaError_t slab_impl_dn(const SphereDev<float>& s, const SlabArgs<float>& a,
+                                cudaStream_t st) {
   int nt = threads_for<float, N3>(N2);
   int ny = threads_for<float, N2>(2 * s.R3 + 1);
   if (ny > nt) nt = ny;
   if (nt > SlabThreads<N2, N3>::v) return cudaErrorInvalidConfiguration;
   const size_t smem = slab_smem_bytes(s.n_col, s.R3, N2, sizeof(float));
-  auto kern = k_slab<N2, N3>;
+  auto kern = k_slab<N2, N3, DN>;
   static std::atomic<bool> attr_set{false};  // per instantiation; raised once
   if (!attr_set.load()) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
@@ -757,15 +794,24 @@ static cudaError_t slab_impl(const SphereDev<float>& s, const SlabArgs<float>& a
   }
   const int gx = a.n_items;
   if (gx == 0) return cudaSuccess;
-  const long long units = (long long)gx * s.N1;
-  const dim3 grid((unsigned)std::min<long long>(units, (long long)occupancy(kern, nt, smem) * sm_count()));
+  const long long resident = (long long)occupancy(kern, nt, smem) * sm_count();
+  // as many items per unit as leave some eight units per resident block
+  const int group =
+      DN ? (int)std::max<long long>(1, std::min<long long>(8, (long long)gx * s.N1 / (8 * resident)))
+         : 1;
+  const long long units = (long long)((gx + group - 1) / group) * s.N1;
+  const dim3 grid((unsigned)std::min<long long>(units, resident));
   double fl = 0, by = 0;
   slab_work(s, a, fl, by);
-  ProfScope ps(PC_SLAB_F32, st, fl, by,
-               a.map.list ? a.map.n_dev : nullptr, a.map.n_list);
+  ProfScope ps(PC_SLAB_F32, st, fl, by, a.map.list ? a.map.n_dev : nullptr, a.map.n_list);
   count_launch();
-  kern<<<grid, nt, smem, st>>>(s, a);
+  kern<<<grid, nt, smem, st>>>(s, a, group);
   return cudaGetLastError();
+}
+template <int N2, int N3>
+static cudaError_t slab_impl(const SphereDev<float>& s, const SlabArgs<float>& a, cudaStream_t st) {
+  return a.mode == SLAB_HPSI && a.dn ? slab_impl_dn<N2, N3, true>(s, a, st)
+                                     : slab_impl_dn<N2, N3, false>(s, a, st);
 }
 
 cudaError_t launch_cols_fwd(const SphereDev<float>& s, const float* x, long long ldx,
