@@ -82,6 +82,7 @@ struct SysData {
   cpx<float>* d_tw32[3] = {nullptr, nullptr, nullptr};
   double* d_v = nullptr;
   float* d_vf = nullptr;
+  float* d_vft = nullptr;  // V(r) / n_r in FP32, each x-plane transposed (fused FP32 H x)
   long long* d_vfx = nullptr;  // V(r) as integers (FP64 transforms)
   uint32_t* d_fx[3] = {nullptr, nullptr, nullptr};  // digit tables of the x-, y-, z-lines
   double* d_psi = nullptr;   // [n_occ][ld]
@@ -517,7 +518,15 @@ std::string shape_key(const char* what, const SysData& s) {
 
 // d_count (with d_list): device length of the list; n_list is then the
 // largest length, which sizes the launches (kernels read the count).
-constexpr int kFewItems = 38;  // a quarter of the SMs
+//
+// Items (vector pairs) up to which FP32 H x takes three launches over all planes
+// instead of one with a block per item, whose time is then one item's (11, 17, 37
+// and 54 us on 24^3 .. 48^3).  One chi0 application in us, three launches against
+// one: 24^3, 4 to 24 items 1633 to 1709 against 1515 to 1599; 32^3, 44 items 3000
+// and 3000, 88 items 3443 against 3235; 40^3, 34 items 3401 against 3926, 51 items
+// 3854 against 4145; 48^3, 64 items 6267 against 6961, 128 items 10032 against 7904.
+int few_items(int N) { return N <= 24 ? 0 : N <= 32 ? 38 : 76; }
+
 
 // R: FP32 or FP64.  refine (FP64): the product of a mixed-mode refinement, whose
 // transforms take seven digits (far below the FP32 inner solve's needs and
@@ -544,10 +553,7 @@ int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list,
   if constexpr (std::is_same<R, float>::value) {
     // FP32 on 24^3 .. 48^3: the whole transform in one launch, the column
     // scratch in shared memory
-    // (few items leave it a block or less per four SMs, and an item's time is
-    // then its block's: 21 us on 24^3 and 90 us on 48^3 against 9 and about 50
-    // in three launches over all planes)
-    if (n_items > kFewItems && !dn && c->opt.fused_hpsi && hpsi_fused_smem(s.sf) > 0) {
+    if (n_items > few_items(s.N[0]) && !dn && c->opt.fused_hpsi && hpsi_fused_smem(s.sf) > 0) {
       Epilogue<float> ep{};
       ep.y = Y;
       ep.ldy = ldy;
@@ -555,18 +561,17 @@ int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list,
       ep.ldx = ldx;
       ep.shift = with_shift ? s.d_negeps32 : nullptr;
       ep.shift_period = with_shift ? s.n_occ : 1;
-      ep.scale = 1.0f / s.n_r;
+      ep.scale = 1.0f;  // d_vft carries 1 / n_r
       ep.kin = 1.0f;
       ep.beta = 0.0f;
       ep.coef = COEF_ONE;
-      // FFT batch: x-planes per group of the fused transform (half, the
-      // default, or twice the default when shared memory allows)
+      // FFT batch: x-planes a block of the fused transform works on at once
+      // (the default, half or a quarter of it)
       const int G0 = hpsi_fused_planes(s.sf);
-      const int cands[3] = {G0, G0 / 2 > 0 ? G0 / 2 : G0,
-                            hpsi_fused_smem(s.sf, 2 * G0) ? 2 * G0 : G0};
+      const int cands[3] = {G0, std::max(1, G0 / 2), std::max(1, G0 / 4)};
       RET(tuned_call(c, "fused_planes:" + std::to_string(s.N[0]), 3, 0, 2.0 * n_items, st,
                      [&](int k) -> int {
-                       CK(launch_hpsi_fused(s.sf, X, ldx, map, n_items, s.d_vf, ep, st, cands[k]));
+                       CK(launch_hpsi_fused(s.sf, X, ldx, map, n_items, s.d_vft, ep, st, cands[k]));
                        return PDEP_OK;
                      }));
       fused = true;
@@ -1720,7 +1725,7 @@ int read_stats(pdep_ctx* c, pdep_stats* out, cudaStream_t st) {
     if (kv.first.rfind("fused_planes:", 0) == 0 && !c->sys.empty()) {
       const int G0 = hpsi_fused_planes(c->sys[0].sf);
       const int k = kv.second.best;
-      out->fused_planes = k == 0 ? G0 : k == 1 ? std::max(1, G0 / 2) : 2 * G0;
+      out->fused_planes = hpsi_fused_planes(c->sys[0].sf, std::max(1, G0 >> k));
     }
     if (kv.first.rfind("pv_", 0) == 0) out->gemm_shape = kv.second.best;
   }
@@ -2003,6 +2008,11 @@ int pdep_setup(const pdep_system_desc* sys, int n_sys, const pdep_options* opt, 
       return bail(fail(PDEP_ERR_CUDA, "potential conversion"));
     r = upload_tables(c, s);
     if (r != PDEP_OK) return bail(r);
+    if (hpsi_fused_smem(s.sf) > 0) {
+      if ((r = persistent(c, &s.d_vft, s.n_r)) != PDEP_OK) return bail(r);
+      if (fused_potential(s.d_v, s.d_vft, s.N[0], 1.0 / s.n_r, st) != cudaSuccess)
+        return bail(fail(PDEP_ERR_CUDA, "potential conversion"));
+    }
     r = setup_states(c, s, st);
     if (r != PDEP_OK) return bail(r);
     if ((r = check_status(c, st)) != PDEP_OK) return bail(r);

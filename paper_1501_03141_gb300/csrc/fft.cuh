@@ -26,9 +26,10 @@ namespace pdep {
 // ---------------------------------------------------------------------------
 __host__ __device__ constexpr int local_tw_offset(int M) {
   return M == 6 ? 0 : M == 8 ? 6 : M == 10 ? 14 : M == 12 ? 24 : M == 16 ? 36
-       : M == 20 ? 52 : M == 24 ? 72 : M == 32 ? 96 : M == 48 ? 128 : M == 64 ? 176 : -1;
+       : M == 20 ? 52 : M == 24 ? 72 : M == 32 ? 96 : M == 48 ? 128 : M == 64 ? 176
+       : M == 40 ? 240 : -1;
 }
-constexpr int LOCAL_TW_SIZE = 240;
+constexpr int LOCAL_TW_SIZE = 280;
 
 // defined here: fft.cuh is included by a single translation unit (no -rdc)
 __constant__ float2 c_local_tw_f[LOCAL_TW_SIZE];
@@ -171,11 +172,8 @@ __device__ __forceinline__ cpx<R> pm(cpx<R> p, cpx<R> v, bool up) {
   const R sgn = up ? R(-1) : R(1);
   return mk(p.x + sgn * v.x, p.y + sgn * v.y);
 }
-// Twiddle sources of the cross-lane line FFTs.  TableTw reads e^{2 pi i j/N}
-// from the global table per use; RegTw holds, for one lane position t, the
-// M twiddles w^{t k2} and the twiddles of the cross-lane stages with span
-// L > 4 in registers, for kernels whose threads keep one lane position
-// across many lines.
+// Twiddle source of the cross-lane line FFTs: e^{2 pi i j/N} from the global
+// table per use
 template <typename R>
 struct TableTw {
   const cpx<R>* __restrict__ tw;
@@ -188,33 +186,6 @@ struct TableTw {
     return table_w<R, S>(tw, j * (N / L));
   }
 };
-template <typename R, int N, int TPL>
-struct RegTw {
-  static constexpr int M = N / TPL;
-  static constexpr int NS = 3;  // stages with L = 8, 16, 32 (TPL <= 32)
-  cpx<R> w[M];
-  cpx<R> sw[NS];
-  __device__ __forceinline__ void init(const cpx<R>* __restrict__ tw, int t) {
-#pragma unroll
-    for (int k2 = 0; k2 < M; ++k2) w[k2] = table_w<R, +1>(tw, t * k2);
-#pragma unroll
-    for (int si = 0; si < NS; ++si) {
-      const int half = 4 << si;  // L = 2 half
-      sw[si] = half < TPL ? table_w<R, +1>(tw, (t & (half - 1)) * (N / (2 * half))) : w[0];
-    }
-  }
-  template <int S>
-  __device__ __forceinline__ cpx<R> k2w(int, int k2) const {
-    return S > 0 ? w[k2] : conj(w[k2]);
-  }
-  // L: the stage's span (8, 16, ...), a constant once the stage loop unrolls
-  template <int S, int N_>
-  __device__ __forceinline__ cpx<R> stage(int, int L) const {
-    const int si = L >= 32 ? 2 : L >= 16 ? 1 : 0;  // L = 8, 16, 32
-    return S > 0 ? sw[si] : conj(sw[si]);
-  }
-};
-
 // Distribution A -> B.  t = lane index inside the group (0..TPL-1).
 template <typename R, int N, int TPL, int S, typename TW>
 __device__ __forceinline__ void fft_a2b(cpx<R> (&v)[N / TPL], int t, const TW& src) {
@@ -314,6 +285,135 @@ __host__ __device__ constexpr bool a_outside(int N, int TPL, int i) {
     if ((f < 0 ? -f : f) < N / 4) return false;
   }
   return true;
+}
+
+// ---------------------------------------------------------------------------
+// whole lines in one thread
+// ---------------------------------------------------------------------------
+// The same recursion as DFT for a line of which only the inputs of the bit mask
+// LIVE are not zero: what they do not reach is left out of the arithmetic
+// (adding a zero cannot be dropped by the compiler).  Every output is live.
+template <bool LA, bool LB, typename R>
+__device__ __forceinline__ cpx<R> live_add(cpx<R> a, cpx<R> b) {
+  return LA && LB ? a + b : LA ? a : LB ? b : mk(R(0), R(0));
+}
+template <bool LA, bool LB, typename R>
+__device__ __forceinline__ cpx<R> live_sub(cpx<R> a, cpx<R> b) {
+  return LA && LB ? a - b : LA ? a : LB ? mk(-b.x, -b.y) : mk(R(0), R(0));
+}
+// a exp(S 2 pi i j / M): quarter turns without a product
+template <typename R, int S, int M>
+__device__ __forceinline__ cpx<R> turn(cpx<R> a, int j) {
+  if (4 * j % M == 0) {
+    const int q = 4 * j / M & 3;
+    return q == 0 ? a : q == 1 ? mul_si<R, S>(a) : q == 2 ? mk(-a.x, -a.y) : mul_si<R, -S>(a);
+  }
+  return a * local_w<R, S, M>(j);
+}
+// inputs p + P q (q < Q) of a mask
+__host__ __device__ constexpr unsigned long long sub_mask(unsigned long long m, int p, int P, int Q) {
+  unsigned long long r = 0;
+  for (int q = 0; q < Q; ++q) r |= (m >> (p + P * q) & 1ull) << q;
+  return r;
+}
+__host__ __device__ constexpr unsigned long long all_live(int n) {
+  return n >= 64 ? ~0ull : (1ull << n) - 1;
+}
+
+template <typename R, int M, int S, unsigned long long LIVE>
+struct LineDFT {
+  static constexpr int P = pick_radix(M);
+  static constexpr int Q = M / P;
+  template <int p>
+  static __device__ __forceinline__ void subs(const cpx<R>* a, cpx<R> (&y)[P][Q]) {
+    if constexpr (p < P) {
+#pragma unroll
+      for (int q = 0; q < Q; ++q) y[p][q] = a[p + P * q];
+      LineDFT<R, Q, S, sub_mask(LIVE, p, P, Q)>::run(y[p]);
+      subs<p + 1>(a, y);
+    }
+  }
+  __host__ __device__ static constexpr unsigned long long outer() {
+    unsigned long long m = 0;
+    for (int p = 0; p < P; ++p) m |= (sub_mask(LIVE, p, P, Q) ? 1ull : 0ull) << p;
+    return m;
+  }
+  static __device__ __forceinline__ void run(cpx<R>* a) {
+    constexpr unsigned long long L = outer();
+    cpx<R> y[P][Q];
+    subs<0>(a, y);
+#pragma unroll
+    for (int k1 = 0; k1 < Q; ++k1) {
+      cpx<R> z[P];
+#pragma unroll
+      for (int p = 0; p < P; ++p)
+        z[p] = (L >> p & 1) ? turn<R, S, M>(y[p][k1], p * k1 % M) : y[p][k1];
+      LineDFT<R, P, S, L>::run(z);
+#pragma unroll
+      for (int k2 = 0; k2 < P; ++k2) a[k1 + Q * k2] = z[k2];
+    }
+  }
+};
+template <typename R, int S, unsigned long long LIVE>
+struct LineDFT<R, 1, S, LIVE> {
+  static __device__ __forceinline__ void run(cpx<R>*) {}
+};
+template <typename R, int S, unsigned long long LIVE>
+struct LineDFT<R, 2, S, LIVE> {
+  static __device__ __forceinline__ void run(cpx<R>* a) {
+    constexpr bool l0 = LIVE & 1, l1 = LIVE >> 1 & 1;
+    const cpx<R> t = a[0];
+    a[0] = live_add<l0, l1>(t, a[1]);
+    a[1] = live_sub<l0, l1>(t, a[1]);
+  }
+};
+template <typename R, int S, unsigned long long LIVE>
+struct LineDFT<R, 3, S, LIVE> {
+  static __device__ __forceinline__ void run(cpx<R>* a) {
+    constexpr bool l0 = LIVE & 1, l1 = LIVE >> 1 & 1, l2 = LIVE >> 2 & 1, l12 = l1 || l2;
+    const R h = R(0.8660254037844386467637231707529362);  // sqrt(3)/2
+    if constexpr (l12) {
+      const cpx<R> t1 = live_add<l1, l2>(a[1], a[2]);
+      const cpx<R> t2 = live_sub<l1, l2>(a[1], a[2]);
+      const cpx<R> m = l0 ? a[0] - scale(t1, R(0.5)) : scale(t1, R(-0.5));
+      const cpx<R> n = scale(mul_si<R, S>(t2), h);
+      a[0] = live_add<l0, true>(a[0], t1);
+      a[1] = m + n;
+      a[2] = m - n;
+    } else {
+      if constexpr (!l0) a[0] = mk(R(0), R(0));
+      a[1] = a[2] = a[0];
+    }
+  }
+};
+template <typename R, int S, unsigned long long LIVE>
+struct LineDFT<R, 4, S, LIVE> {
+  static __device__ __forceinline__ void run(cpx<R>* a) {
+    constexpr bool l0 = LIVE & 1, l1 = LIVE >> 1 & 1, l2 = LIVE >> 2 & 1, l3 = LIVE >> 3 & 1;
+    const cpx<R> t0 = live_add<l0, l2>(a[0], a[2]);
+    const cpx<R> t1 = live_sub<l0, l2>(a[0], a[2]);
+    const cpx<R> t2 = live_add<l1, l3>(a[1], a[3]);
+    const cpx<R> t3 = mul_si<R, S>(live_sub<l1, l3>(a[1], a[3]));
+    constexpr bool e = l0 || l2, o = l1 || l3;
+    a[0] = live_add<e, o>(t0, t2);
+    a[2] = live_sub<e, o>(t0, t2);
+    a[1] = live_add<e, o>(t1, t3);
+    a[3] = live_sub<e, o>(t1, t3);
+  }
+};
+template <typename R, int S, unsigned long long LIVE>
+struct LineDFT<R, 5, S, LIVE> {
+  static __device__ __forceinline__ void run(cpx<R>* a) { DFT<R, 5, S>::run(a); }
+};
+
+// The positions of a line that hold a frequency |n| < N/4: all a sphere has
+__host__ __device__ constexpr bool in_sphere_band(int p, int N) {
+  return p < N / 4 || p > N - N / 4;
+}
+__host__ __device__ constexpr unsigned long long band_mask(int N) {
+  unsigned long long m = 0;
+  for (int p = 0; p < N; ++p) m |= (in_sphere_band(p, N) ? 1ull : 0ull) << p;
+  return m;
 }
 
 }  // namespace pdep

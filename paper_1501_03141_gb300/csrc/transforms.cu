@@ -13,7 +13,7 @@ namespace pdep {
 
 
 cudaError_t upload_local_twiddles() {
-  static const int sizes[] = {6, 8, 10, 12, 16, 20, 24, 32, 48, 64};
+  static const int sizes[] = {6, 8, 10, 12, 16, 20, 24, 32, 40, 48, 64};
   float2 hf[LOCAL_TW_SIZE];
   const double two_pi = 6.283185307179586476925286766559;
   for (int M : sizes) {
@@ -571,128 +571,313 @@ __global__ void __launch_bounds__(SlabThreads<N2, N3>::v, (SlabMinBlocks<N2, N3>
 // fused FP32 H x: the whole transform of one item in one block
 // ---------------------------------------------------------------------------
 // For cubic grids whose column scratch of one item (N x n_col complex) fits
-// in shared memory (24^3 .. 48^3), one block of 512 threads runs, per item:
-// the x-line inverse FFTs of every column into shared memory, then the y and
-// z passes of G x-planes at a time (each plane on its own warp-aligned group
-// of 512/G threads, the potential multiplied between the z inverse and
-// forward FFTs), then the x-line forward FFTs with the epilogue.  The column
-// scratch never leaves the SM: per item the HBM traffic is the two input
-// vectors (read for the transform and for the diagonal term) and the two
-// outputs, against a write, a read-modify-write and a read of the whole
-// scratch by the three-launch form.  Blocks are persistent over the items.
-constexpr int FUSED_THREADS = 512;
-
-// z-lines of one x-plane (T2: its (n3 slot, i2) plane), the potential
-// multiplied on the grid between the inverse and forward FFTs
-template <int N, typename TW>
-__device__ __forceinline__ void z_hpsi(const SphereDev<float>& s, cpx<float>* T2,
-                                       const float* __restrict__ vplane, int tid, int nthreads,
-                                       const TW& tws) {
-  constexpr int TL3 = Tpl<float, N>::v;
-  constexpr int M3 = N / TL3;
-  constexpr int TS = T2Stride<N>::v;
-  const int R3 = s.R3;
-  const int t3 = tid & (TL3 - 1);
-  const int zper = nthreads / TL3;
-  for (int base = 0; base < N; base += zper) {
-    const int i2 = base + tid / TL3;
-    const bool act = i2 < N;
-    cpx<float> v[M3];
-#pragma unroll
-    for (int i = 0; i < M3; ++i) {
-      const int n3 = freq_of(pos_a<N, TL3>(t3, i), N);
-      v[i] = (!a_outside(N, TL3, i) && act && iabs(n3) <= R3) ? T2[t2_at(n3 + R3, i2, TS)]
-                                                              : zero<float>();
-    }
-    fft_a2b<float, N, TL3, +1>(v, t3, tws);
-    // this lane's M3 (even) potential values are consecutive: 8-byte loads
-    const float* vr = vplane + (act ? i2 : 0) * N + pos_b<N, TL3>(t3, 0);
-    static_assert(M3 % 2 == 0, "paired potential loads");
-#pragma unroll
-    for (int i = 0; i < M3; i += 2) {
-      const float2 f = act ? __ldg(reinterpret_cast<const float2*>(vr + i)) : make_float2(0.f, 0.f);
-      v[i] = scale(v[i], f.x);
-      v[i + 1] = scale(v[i + 1], f.y);
-    }
-    fft_b2a<float, N, TL3, -1>(v, t3, tws);
-    if (act) {
-#pragma unroll
-      for (int i = 0; i < M3; ++i) {
-        if (a_outside(N, TL3, i)) continue;
-        const int n3 = freq_of(pos_a<N, TL3>(t3, i), N);
-        if (iabs(n3) <= R3) T2[t2_at(n3 + R3, i2, TS)] = v[i];
-      }
-    }
-  }
-}
-
-// barrier of the warps of plane group g (nthreads of them, warp-aligned)
-__device__ __forceinline__ void group_sync(int g, int nthreads) {
-  if (nthreads == 32) {
-    __syncwarp();
-  } else {
-    asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(nthreads) : "memory");
-  }
+// in shared memory (24^3 .. 48^3), one block runs, per item: the x-line inverse
+// FFTs of every column into shared memory, then the y and z passes of the
+// x-planes (the potential multiplied between the z inverse and forward FFTs),
+// then the x-line forward FFTs and the epilogue.  The column scratch never
+// leaves the SM: per item the HBM traffic is the two input vectors (read for
+// the transform and for the diagonal term) and the two outputs.  Blocks are
+// persistent over the items.
+//
+// Every line is transformed by one thread, in registers: with a line on four
+// lanes the shuffles, selects, swizzled addresses and predicates outnumbered
+// the arithmetic two to one (443 thousand warp instructions per item of 48^3,
+// 57% of them floating point, and the kernel is bound by the issue slots).  In
+// one thread the positions are compile-time constants: offsets are immediate,
+// twiddles constant-bank operands, quarter turns free, and the zero half of a
+// sphere's line costs nothing.  Three warps form a group that takes as many
+// planes as its lanes cover z-lines (4, 3, 2, 2 planes of 24, 32, 40, 48 lines);
+// the groups share nothing but B1 and synchronise by named barriers.  168
+// registers (96 hold a line of 48) leave 12 warps.  Measured against four lanes
+// per line: 245 thousand instructions per item; 56 launches of up to 4096 items on
+// 48^3 87.0 -> 55.6 ms (68.1 ms with a group's planes beside the whole column
+// scratch, three groups; 74.3 ms with the three steps' code apart), 37 launches
+// on 32^3 3.22 -> 2.24 ms.  Error of H x against FP64 5.4e-8 -> 5.1e-8 on 48^3.
+// What is left is latency: the potential comes from L2 (48 loads a line), and two
+// of three warps have y-lines.
+constexpr int FG_THREADS = 96;  // threads of a group
+// PLANES: x-planes of a group at a time.  GROUPS: of a block, as many as the
+// registers leave (24: two blocks per SM).  OVER: 48^3 does not fit its planes'
+// (n3, i2) values beside the column scratch; a plane in work keeps some n3 rows
+// in its own row of the column scratch, which is dead meanwhile.
+template <int N>
+struct Fused {
+  static constexpr int PLANES = FG_THREADS / N;
+  static constexpr int GROUPS = N == 32 ? 6 : N == 40 ? 5 : 4;
+  static constexpr bool OVER = N > 40;
+};
+// n3 rows a plane keeps in the column scratch, and beside it: (i2, n3) with odd
+// strides, so that neither y-lines (lanes along n3) nor z-lines (along i2)
+// conflict in the banks
+struct FusedRows {
+  int in, out;
+};
+__host__ __device__ __forceinline__ FusedRows fused_rows(bool over, int n_col, int R3, int N) {
+  const int nslot = 2 * R3 + 1;
+  int k = over ? (n_col / N < nslot ? n_col / N : nslot) : 0;
+  if (k % 2 == 0 && k > 0) --k;
+  return {k, (nslot - k) | 1};
 }
 
 template <int N>
-__global__ void __launch_bounds__(FUSED_THREADS, 1)
+__global__ void __launch_bounds__(FG_THREADS * Fused<N>::GROUPS, (N <= 24 ? 2 : 1))
     k_hpsi_fused(SphereDev<float> s, const float* __restrict__ x, long long ldx, ItemMap map,
-                 int n_items, const float* __restrict__ v, Epilogue<float> ep, int G,
+                 int n_items, const float* __restrict__ vt, Epilogue<float> ep,
                  DevTimer* timer, double item_flops, double item_bytes) {
   const unsigned long long t0 = dev_clock_ns();
-  constexpr int TL = Tpl<float, N>::v;
-  constexpr int TS = T2Stride<N>::v;
+  constexpr unsigned long long BAND = band_mask(N), ALL = all_live(N);
+  constexpr int PG = Fused<N>::PLANES;
+  constexpr bool OVER = Fused<N>::OVER;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<float>* B1 = reinterpret_cast<cpx<float>*>(smem_raw);
+  cpx<float>* T = B1 + (size_t)N * s.n_col;
+  // between the passes T holds the item's members, (a, b) per half index, and
+  // the real G = 0 components last
+  float4* st = reinterpret_cast<float4*>(T);
+  float* stf = reinterpret_cast<float*>(T);
+  const int tid = threadIdx.x;
   const int nslot = 2 * s.R3 + 1;
   const int nl = listed_count(map);
   const int items = items_of(map, n_items, nl);
-  const int VT = blockDim.x / G;  // threads per plane: a multiple of 32
-  const int g = threadIdx.x / VT;
-  const int vt = threadIdx.x - g * VT;
-  cpx<float>* T2 = B1 + (size_t)N * s.n_col + (size_t)g * nslot * TS;
-  const int lines = blockDim.x / TL;
-  // a cubic grid: the x, y and z lines have one length and one twiddle
-  // table, and every pass keeps this thread at lane position t of its lines
-  RegTw<float, N, TL> rtw;
-  rtw.init(s.tw1, threadIdx.x & (TL - 1));
+  const int grp = tid / FG_THREADS, gt = tid - grp * FG_THREADS;
+  const int groups = blockDim.x / FG_THREADS;
+  const FusedRows rows = fused_rows(OVER, s.n_col, s.R3, N);
+  cpx<float>* T2 = T + (size_t)grp * PG * N * rows.out;
+  // this thread's y-line (plane yp of the group's, n3 slot, columns ymid - yR ..
+  // ymid + yR of the plane) and z-line (plane zp, i2)
+  // (threads without a line keep to the first line's addresses)
+  const bool yon = gt < PG * nslot, zon = gt < PG * N;
+  const int yp = yon ? gt / nslot : 0, ysl = yon ? gt - yp * nslot : 0;
+  const int2 info = s.slot[ysl];
+  const bool yact = yon && slot_in_range(s, info);
+  const int yR = info.x, ymid = info.y + info.x;
+  const bool yin = ysl < rows.in;
+  const int zp = zon ? gt / N : 0, i2 = zon ? gt - zp * N : 0;
+  // the field is carried at sqrt(2) times its size: the members' 1/sqrt(2) in and
+  // out become one exact 1/2
+  const float rt2 = 1.4142135623730950488016887242097f;
+  const int j0 = 2 * s.n_half;
+  auto group_sync = [&] {
+    asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "n"(FG_THREADS) : "memory");
+  };
 #pragma unroll 1
   for (int item = blockIdx.x; item < items; item += gridDim.x) {
-    __syncthreads();  // the previous item's reads of B1 are done
-#pragma unroll 1
-    for (int base = 0; base < s.n_ucol; base += lines) {
-      const int uc = base + threadIdx.x / TL;
-      xline_inverse<float, N>(s, x, ldx, map, nl, COEF_ONE, item, uc, uc < s.n_ucol, B1, rtw);
+    const int ia = map.vec(item, 0, nl), ib = map.vec(item, 1, nl);
+    const float* xa = x + (long long)ia * ldx;
+    const float* xb = ib >= 0 ? x + (long long)ib * ldx : nullptr;
+    __syncthreads();  // the previous item's reads of T are done
+#pragma unroll 8
+    for (int j = tid; j < j0; j += blockDim.x) {
+      float* d = stf + (j >> 1) * 4 + (j & 1);
+      d[0] = xa[j];
+      d[2] = xb ? xb[j] : 0.f;
     }
     __syncthreads();
-    // the plane groups touch disjoint data (their own plane row of B1 and
-    // their own T2), so each synchronises only its own warps: one warp with
-    // __syncwarp, several with a named barrier (ids 1..G)
+    // x-lines of the columns (which = 0) and of their mirror columns (1):
+    // A + i B at n1, conj(A) + i conj(B) at -n1
 #pragma unroll 1
-    for (int p0 = 0; p0 < N; p0 += G) {
-      const int i1 = p0 + g;
-      if (i1 < N) {  // uniform over the plane group's warps
-        cpx<float>* S1 = B1 + (size_t)i1 * s.n_col;
-        y_inverse<N>(s, S1, T2, vt, VT, rtw);
-        group_sync(g, VT);
-        z_hpsi<N>(s, T2, v + (size_t)i1 * N * N, vt, VT, rtw);
-        group_sync(g, VT);
-        y_forward<N>(s, T2, S1, vt, VT, rtw);
-        group_sync(g, VT);
+    for (int u = tid; u < 2 * s.n_ucol; u += blockDim.x) {
+      const int which = u >= s.n_ucol;
+      const UCol c = s.ucol[u - which * s.n_ucol];
+      const bool self = c.col == c.mcol;
+      if ((self && which) || !ucol_in_range(s, c)) continue;
+      // member of n1: fp/fn + sp/sn n1 for positive and negative n1; the sign
+      // is also that of the conjugation
+      const int sp = which ? -1 : 1, sn = self ? -1 : sp;
+      const int fp = self ? c.h0 - 1 : c.h0 + c.R1;
+      const float gp = (float)sp, gn = (float)sn;
+      cpx<float> v[N];
+#pragma unroll
+      for (int p = 0; p < N; ++p) {
+        v[p] = zero<float>();
+        if (!in_sphere_band(p, N)) continue;
+        const int n1 = freq_of(p, N);
+        if (n1 == 0) {
+          if (self) {
+            v[p] = mk(rt2 * xa[j0], xb ? rt2 * xb[j0] : 0.f);
+          } else {
+            const float4 f = st[fp];
+            v[p] = mk(f.x - gp * f.w, gp * f.y + f.z);
+          }
+        } else if (iabs(n1) <= c.R1) {
+          const float4 f = st[fp + (n1 > 0 ? sp : sn) * n1];
+          const float g = n1 > 0 ? gp : gn;
+          v[p] = mk(f.x - g * f.w, g * f.y + f.z);
+        }
+      }
+      LineDFT<float, N, +1, BAND>::run(v);
+      cpx<float>* o = B1 + (which ? c.mcol : c.col);
+#pragma unroll
+      for (int p = 0; p < N; ++p) o[(long long)p * s.n_col] = v[p];
+    }
+    __syncthreads();
+    // planes of this thread's group, PG at a time: y-lines (plane, n3), z-lines
+    // (plane, i2) with the potential, y-lines back, a line per thread.  A thread's
+    // y-lines there and back are the same.  One loop body for the three keeps
+    // the code of one transform each way in the instruction cache.
+#pragma unroll 1
+    for (int p0 = grp * PG; p0 < N; p0 += groups * PG) {
+#pragma unroll 1
+      for (int step = 0; step < 3; ++step) {
+        const bool z = step == 1;
+        const int i1 = min(p0 + (z ? zp : yp), N - 1);
+        const bool act = p0 + (z ? zp : yp) < N && (z ? zon : yact);
+        const int bound = act ? (z ? s.R3 : yR) : -1;
+        const int col = i1 * s.n_col;
+        // a y-line's columns, its (n3, i2) row, and a z-line's two parts
+        auto line = [&] { return B1 + (col + ymid); };
+        auto yt = [&] { return yin ? B1 + (col + ysl) : T2 + (yp * N * rows.out + ysl - rows.in); };
+        auto zin = [&] { return B1 + (col + i2 * rows.in + s.R3); };
+        auto zout = [&] { return T2 + ((zp * N + i2) * rows.out + s.R3 - rows.in); };
+        // OVER: a plane's y-lines overwrite what others read, so a barrier follows
+        // their loads.  The body is the warp's, with the lines' loads and stores
+        // predicated: a branch per line around the barrier spilled its registers.
+        if (__any_sync(0xffffffffu, act)) {
+          cpx<float> v[N];
+          if (step < 2) {
+            if (z) {
+              const cpx<float>*zi = zin(), *zo = zout();
+#pragma unroll
+              for (int p = 0; p < N; ++p) {
+                const int n = freq_of(p, N);
+                v[p] = in_sphere_band(p, N) && iabs(n) <= bound
+                           ? (OVER && n + s.R3 < rows.in ? zi : zo)[n]
+                           : zero<float>();
+              }
+            } else {
+              const cpx<float>* l = line();
+#pragma unroll
+              for (int p = 0; p < N; ++p) {
+                const int n = freq_of(p, N);
+                v[p] = in_sphere_band(p, N) && iabs(n) <= bound ? l[n] : zero<float>();
+              }
+            }
+            if (OVER && !z) group_sync();
+            LineDFT<float, N, +1, BAND>::run(v);
+          } else {
+            const cpx<float>* y = yt();
+            const int ys = yin ? rows.in : rows.out;
+#pragma unroll
+            for (int p = 0; p < N; ++p, y += ys) v[p] = *y;
+            if (OVER) group_sync();
+          }
+          if (step == 0) {
+            cpx<float>* y = yt();
+            const int ys = yin ? rows.in : rows.out;
+#pragma unroll
+            for (int p = 0; p < N; ++p, y += ys)
+              if (act) *y = v[p];
+          } else {
+            if (z) {
+              const float* vp = vt + i1 * (N * N) + i2;
+#pragma unroll
+              for (int p = 0; p < N; ++p) v[p] = scale(v[p], __ldg(vp + p * N));
+            }
+            LineDFT<float, N, -1, ALL>::run(v);
+            if (z) {
+              cpx<float>*zi = zin(), *zo = zout();
+#pragma unroll
+              for (int p = 0; p < N; ++p) {
+                const int n = freq_of(p, N);
+                if (in_sphere_band(p, N) && iabs(n) <= bound)
+                  (OVER && n + s.R3 < rows.in ? zi : zo)[n] = v[p];
+              }
+            } else {
+              cpx<float>* l = line();
+#pragma unroll
+              for (int p = 0; p < N; ++p) {
+                const int n = freq_of(p, N);
+                if (in_sphere_band(p, N) && iabs(n) <= bound) l[n] = v[p];
+              }
+            }
+          }
+        } else if (OVER && !z) {
+          group_sync();
+        }
+        if (step < 2) group_sync();
       }
     }
     __syncthreads();
+    // x-lines back.  With d the transform of a column and dm that of its
+    // mirror at -n1, 2 Va = d + conj(dm) and 2 i Vb = d - conj(dm): the line of
+    // a (which = 0) or b (1) is the transform of that combination of the columns
 #pragma unroll 1
-    for (int base = 0; base < s.n_ucol; base += lines) {
-      const int uc = base + threadIdx.x / TL;
-      xline_forward<float, N>(s, B1, map, nl, ep, item, uc, uc < s.n_ucol, rtw);
+    for (int u = tid; u < 2 * s.n_ucol; u += blockDim.x) {
+      const int which = u >= s.n_ucol;
+      const UCol c = s.ucol[u - which * s.n_ucol];
+      if (!ucol_in_range(s, c)) continue;
+      const bool self = c.col == c.mcol;
+      const float g = which ? -1.f : 1.f;
+      const cpx<float>* o = B1 + c.col;
+      const long long dm = c.mcol - c.col;
+      cpx<float> v[N];
+#pragma unroll
+      for (int p = 0; p < N; ++p) {
+        const cpx<float> a = o[(long long)p * s.n_col], b = o[(long long)p * s.n_col + dm];
+        v[p] = mk(a.x + g * b.x, a.y - g * b.y);
+      }
+      LineDFT<float, N, -1, ALL>::run(v);
+      // b's value is -i times the line's
+      float* d = stf + 4 * (self ? c.h0 - 1 : c.h0 + c.R1) + 2 * which;
+#pragma unroll
+      for (int p = 0; p < N; ++p) {
+        if (!in_sphere_band(p, N)) continue;
+        const int n1 = freq_of(p, N);
+        const float re = which ? v[p].y : v[p].x, im = which ? -v[p].x : v[p].y;
+        if (n1 == 0 && self)
+          stf[2 * j0 + 2 * which] = re;
+        else if (iabs(n1) <= c.R1 && (!self || n1 > 0))
+          *reinterpret_cast<float2*>(d + 4 * n1) = make_float2(re, im);
+      }
+    }
+    __syncthreads();
+    // four components at a time: their loads are in flight together (the
+    // outputs may alias the inputs, so the compiler keeps loads behind stores)
+    const OutRow<float> oa(ep, ia), ob(ep, ib);
+    const bool old = ep.beta != 0;
+#pragma unroll 1
+    for (int jb = tid; jb <= j0; jb += 4 * blockDim.x) {
+      float xi[4][2], yo[4][2], kin[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int j = jb + q * blockDim.x;
+        const bool on = j <= j0, two = on && ib >= 0;
+        xi[q][0] = on && oa.x_ ? oa.x_[j] : 0.f;
+        xi[q][1] = two && ob.x_ ? ob.x_[j] : 0.f;
+        yo[q][0] = on && old ? oa.y_[j] : 0.f;
+        yo[q][1] = two && old ? ob.y_[j] : 0.f;
+        kin[q] = j < j0 ? s.kin[j >> 1] : 0.f;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int j = jb + q * blockDim.x;
+        if (j > j0) break;
+        const bool g0 = j == j0;
+        const float* d = stf + (j >> 1) * 4 + (j & 1);
+        const float w = ep.scale * (g0 ? 0.25f * rt2 : 0.5f) *
+                        (g0 ? (ep.coef == COEF_ONE ? 1.f : 0.f) : coef_of<float>(ep.coef, s.g2, j >> 1));
+        const float dg = ep.kin * kin[q];
+        // the diagonal term is the large one: its product is the fused one.
+        // Without a diagonal term or an old output its value above is zero.
+        oa.y_[j] = fmaf(ep.beta, yo[q][0], fmaf(dg + oa.sh_, xi[q][0], w * d[0]));
+        if (ib >= 0) ob.y_[j] = fmaf(ep.beta, yo[q][1], fmaf(dg + ob.sh_, xi[q][1], w * d[2]));
+      }
     }
   }
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     const int mine = items > (int)blockIdx.x ? (items - 1 - (int)blockIdx.x) / gridDim.x + 1 : 0;
     dev_timer_block_end(timer, t0, mine * item_flops, mine * item_bytes);
   }
+}
+
+// out (i1, i3, i2) = scale in (i1, i2, i3) on a cubic grid: a z-line per thread
+// then reads the potential coalesced, and the transforms' 1 / (N1 N2 N3), which
+// rounded to FP32 would be a common error of all components, is in its rounding
+__global__ void k_fused_potential(const double* __restrict__ in, float* __restrict__ out, int N,
+                                  double scale) {
+  const int plane = blockIdx.x * N * N;
+  for (int j = threadIdx.x; j < N * N; j += blockDim.x)
+    out[plane + j] = (float)(scale * in[plane + (j % N) * N + j / N]);
 }
 
 // resident blocks per SM of a kernel at a block size and shared memory
@@ -853,66 +1038,64 @@ cudaError_t launch_slab(const SphereDev<float>& s, const SlabArgs<float>& a, cud
   return cudaErrorInvalidValue;
 }
 
-// planes per group of the fused kernel: the fewest planes whose thread
-// group (a power of two, at least a warp) covers every y-line slot at once
-static int fused_planes(int nslot, int tl) {
-  int vt = 32;
-  while (vt < nslot * tl && vt < FUSED_THREADS) vt *= 2;
-  return FUSED_THREADS / vt;
+struct FusedShape {
+  int planes, groups;
+  bool over;
+};
+static FusedShape fused_shape(int N) {
+  switch (N) {
+    case 24: return {Fused<24>::PLANES, Fused<24>::GROUPS, Fused<24>::OVER};
+    case 32: return {Fused<32>::PLANES, Fused<32>::GROUPS, Fused<32>::OVER};
+    case 40: return {Fused<40>::PLANES, Fused<40>::GROUPS, Fused<40>::OVER};
+    case 48: return {Fused<48>::PLANES, Fused<48>::GROUPS, Fused<48>::OVER};
+  }
+  return {0, 0, false};
 }
 
-// groups of more than one warp synchronise on named barriers 1..G, and the
-// hardware has barriers 0..15 only
-static bool fused_barriers_ok(int G) { return FUSED_THREADS / G == 32 || G <= 15; }
-
-static int fused_tl(int N) {
-  switch (N) {
-    case 24: return Tpl<float, 24>::v;
-    case 32: return Tpl<float, 32>::v;
-    case 40: return Tpl<float, 40>::v;
-    case 48: return Tpl<float, 48>::v;
-  }
-  return 0;
+// shared memory of a block of 'groups' groups
+static size_t fused_bytes(const SphereDev<float>& s, int groups) {
+  const FusedShape f = fused_shape(s.N1);
+  const size_t t2 = (size_t)groups * f.planes * s.N1 * fused_rows(f.over, s.n_col, s.R3, s.N1).out;
+  const size_t members = ((size_t)s.n_half + 1) * 2;  // (a, b) of a half index: two complex
+  return ((size_t)s.N1 * s.n_col + std::max(t2, members)) * sizeof(cpx<float>);
 }
 
 int hpsi_fused_planes(const SphereDev<float>& s, int planes) {
-  const int tl = fused_tl(s.N1);
-  if (!tl) return 0;
-  const int nslot = 2 * s.R3 + 1;
-  const int G0 = fused_planes(nslot, tl);
-  // a requested group must be a power of two whose thread groups (512/G
-  // threads) are at least a warp; fewer threads than a plane's y-lines take
-  // two rounds per pass
-  if (planes > 0 && FUSED_THREADS / planes >= 32 && (planes & (planes - 1)) == 0 &&
-      fused_barriers_ok(planes))
-    return planes;
-  return fused_barriers_ok(G0) ? G0 : 0;
+  if (s.N1 != s.N2 || s.N2 != s.N3) return 0;
+  const FusedShape f = fused_shape(s.N1);
+  if (!f.planes) return 0;
+  int groups = planes > 0 ? std::min(std::max(planes / f.planes, 1), f.groups) : f.groups;
+  while (groups > 0 && fused_bytes(s, groups) > 226 * 1024) --groups;
+  return groups * f.planes;
 }
 
 size_t hpsi_fused_smem(const SphereDev<float>& s, int planes) {
-  if (s.N1 != s.N2 || s.N2 != s.N3 || !fused_tl(s.N1)) return 0;
-  const int nslot = 2 * s.R3 + 1;
   const int G = hpsi_fused_planes(s, planes);
-  if (G <= 0) return 0;
-  const size_t bytes = ((size_t)s.N1 * s.n_col + (size_t)G * nslot * (s.N2 + 8)) * sizeof(cpx<float>);
-  return bytes <= 225 * 1024 ? bytes : 0;
+  return G > 0 ? fused_bytes(s, G / fused_shape(s.N1).planes) : 0;
+}
+
+cudaError_t fused_potential(const double* in, float* out, int N, double scale, cudaStream_t st) {
+  count_launch();
+  k_fused_potential<<<N, 256, 0, st>>>(in, out, N, scale);
+  return cudaGetLastError();
 }
 
 template <int N>
 static cudaError_t hpsi_fused_impl(const SphereDev<float>& s, const float* x, long long ldx,
-                                   ItemMap map, int n_items, const float* v,
+                                   ItemMap map, int n_items, const float* vt,
                                    const Epilogue<float>& ep, size_t smem, int G,
                                    cudaStream_t st) {
   auto kern = k_hpsi_fused<N>;
   static std::atomic<bool> attr_set{false};
   if (!attr_set.load()) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         225 * 1024);
+                                         226 * 1024);
     if (e != cudaSuccess) return e;
     attr_set.store(true);
   }
+  const int threads = G / Fused<N>::PLANES * FG_THREADS;
   const unsigned grid = (unsigned)std::min<long long>(
-      n_items, (long long)occupancy(kern, FUSED_THREADS, smem) * sm_count());
+      n_items, (long long)occupancy(kern, threads, smem) * sm_count());
   // algorithmic work: as the three launches it replaces (x-lines both ways,
   // y- and z-lines both ways, V products); bytes: the vectors only
   const double planes = (double)n_items * s.N1;
@@ -923,23 +1106,23 @@ static cudaError_t hpsi_fused_impl(const SphereDev<float>& s, const float* x, lo
   // timed on the device (this kernel also runs inside the CG graphs): the
   // work is counted per processed item
   count_launch();
-  kern<<<grid, FUSED_THREADS, smem, st>>>(s, x, ldx, map, n_items, v, ep, G,
-                                          dev_timer(PC_HPSI_FUSED), fl / n_items, by / n_items);
+  kern<<<grid, threads, smem, st>>>(s, x, ldx, map, n_items, vt, ep, dev_timer(PC_HPSI_FUSED),
+                                    fl / n_items, by / n_items);
   return cudaGetLastError();
 }
 
 cudaError_t launch_hpsi_fused(const SphereDev<float>& s, const float* x, long long ldx, ItemMap map,
-                              int n_items, const float* v, const Epilogue<float>& ep,
+                              int n_items, const float* vt, const Epilogue<float>& ep,
                               cudaStream_t st, int planes) {
   const size_t smem = hpsi_fused_smem(s, planes);
   if (smem == 0) return cudaErrorInvalidValue;
   if (n_items <= 0) return cudaSuccess;
   const int G = hpsi_fused_planes(s, planes);
   switch (s.N1) {
-    case 24: return hpsi_fused_impl<24>(s, x, ldx, map, n_items, v, ep, smem, G, st);
-    case 32: return hpsi_fused_impl<32>(s, x, ldx, map, n_items, v, ep, smem, G, st);
-    case 40: return hpsi_fused_impl<40>(s, x, ldx, map, n_items, v, ep, smem, G, st);
-    case 48: return hpsi_fused_impl<48>(s, x, ldx, map, n_items, v, ep, smem, G, st);
+    case 24: return hpsi_fused_impl<24>(s, x, ldx, map, n_items, vt, ep, smem, G, st);
+    case 32: return hpsi_fused_impl<32>(s, x, ldx, map, n_items, vt, ep, smem, G, st);
+    case 40: return hpsi_fused_impl<40>(s, x, ldx, map, n_items, vt, ep, smem, G, st);
+    case 48: return hpsi_fused_impl<48>(s, x, ldx, map, n_items, vt, ep, smem, G, st);
   }
   return cudaErrorInvalidValue;
 }

@@ -191,13 +191,15 @@ cudaError_t launch_cols_bwd(const SphereDev<double>& s, const cpx<double>* b1, I
 // cols_bwd with that epilogue.  hpsi_fused_smem returns its shared memory
 // per block, 0 where the fused form does not apply.
 // planes (0 = default) sets the x-planes transformed at once by a block (the
-// autotuner's FFT batch; a power of two from 1 to 16 whose thread groups
-// still cover a plane's y-lines, else the default is used).
+// autotuner's FFT batch), brought to a number of whole thread groups that fits.
+// vt: scale times the potential, each plane transposed (fused_potential); ep.scale
+// is what is left of the epilogue's.
 size_t hpsi_fused_smem(const SphereDev<float>& s, int planes = 0);
 int hpsi_fused_planes(const SphereDev<float>& s, int planes = 0);
 cudaError_t launch_hpsi_fused(const SphereDev<float>& s, const float* x, long long ldx, ItemMap map,
-                              int n_items, const float* v, const Epilogue<float>& ep,
+                              int n_items, const float* vt, const Epilogue<float>& ep,
                               cudaStream_t st, int planes = 0);
+cudaError_t fused_potential(const double* in, float* out, int N, double scale, cudaStream_t st);
 
 // Digit tables of the FP64 transforms for lines of N points (empty for other
 // lengths), and the potential v [n] as 63-bit integers scaled by the exponent
