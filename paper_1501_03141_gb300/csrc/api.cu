@@ -1127,13 +1127,14 @@ int setup_states(pdep_ctx* c, SysData& s, cudaStream_t st) {
 // The CG step's launch shape and the FP32 projection kernel are fixed once
 // the autotuner has timed them (or autotuning is off); only then is the loop
 // captured in a graph.
-bool tuned(const pdep_ctx* c, const SysData& s, int pi) {
+bool tuned(const pdep_ctx* c, const SysData& s, int pi, int n) {
   if (!c->opt.autotune) return true;
   const bool pv_ok = pi == 1 || c->opt.proj_variant >= 0 || c->proj_variant >= 0 ||
                      c->opt.precision == PDEP_MIXED_BF16;
   const bool fused_ok = pi == 1 || !c->opt.fused_hpsi || hpsi_fused_smem(s.sf) == 0 ||
                         tune_done(c, "fused_planes:" + std::to_string(s.N[0]));
-  return c->cg_variant[pi] >= 0 && pv_ok && fused_ok;
+  const bool cg_ok = c->cg_variant[pi] >= 0 || cg_streams(n, s.n_pw, pi == 1 ? 8 : 4);
+  return cg_ok && pv_ok && fused_ok;
 }
 int cg_variant_of(const pdep_ctx* c, int pi) {
   return c->cg_variant[pi] >= 0 ? c->cg_variant[pi] : 0;
@@ -1331,7 +1332,7 @@ int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int ma
   a.tolv = tolv;
   // loops under 256 RHS are never timed by the autotuner: they run the
   // current (or default) shapes and are captured right away
-  const bool graph = c->opt.use_graph && (tuned(c, s, pi) || n < 256);
+  const bool graph = c->opt.use_graph && (tuned(c, s, pi, n) || n < 256);
   if (!graph) {
     // eager: host loop, one 16-byte read of the loop state per step
     const bool tail = n <= CG_TAIL_MAX, fuse = tail && few_projection<R>(c, s, n);
@@ -1356,7 +1357,8 @@ int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int ma
       // Autotuner: while untuned, each large step tries the next launch shape
       // (all shapes compute the same update) and its time per RHS is kept;
       // afterwards the fastest shape is used.
-      const bool tuning = c->opt.autotune && c->cg_variant[pi] < 0 && n_act >= 256;
+      const bool tuning = c->opt.autotune && c->cg_variant[pi] < 0 && n_act >= 256 &&
+                          !cg_streams(n, s.n_pw, sizeof(R));
       a.variant = tuning ? c->cg_tune_next[pi] : cg_variant_of(c, pi);
       if (tail && n < 256) a.variant = CG_FEW;
       a.list_count = nullptr;

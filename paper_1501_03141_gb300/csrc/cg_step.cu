@@ -8,8 +8,8 @@
 //
 // Why clusters: with a handful of RHS a step's time is the latency of one
 // block walking one vector.  Against the streaming block per RHS this replaced:
-// 84 RHS of 16 375 coefficients (FP32) 131 -> 7 us, 8 RHS of 799 14.5 -> 7 us;
-// 8192 RHS of 6859 at HBM speed (the autotuner picks the block shape).
+// three RHS of 64^3 one CG application 13.4 -> 9.9 ms, eight of 24^3 2.19 -> 1.61 ms.
+// More than CG_TAIL_MAX RHS are streamed (k_cg_stream below).
 //
 // Two forms for few RHS: PROJ adds the projection term sum_w sigma_w |w><w| p
 // to A p first (the RHS's cluster has p in registers, the states come from L2),
@@ -18,6 +18,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "linalg.cuh"
 #include "profile.cuh"
@@ -324,6 +325,222 @@ __global__ void __launch_bounds__(T)
   }
 }
 
+// --- many RHS -----------------------------------------------------------------
+// One block per RHS leaves the memory idle while the block reduces, and what its
+// registers hold in flight is too little to begin with (8192 RHS of 6859 FP32 at
+// 2.8 TB/s).  Here persistent blocks stream the RHS: p, A p, r and x of the next
+// two come by bulk copies into two shared-memory stages while one is worked on,
+// some 110 KB in flight per SM whatever the row length (short rows: several
+// blocks per SM).  K comes from L2, outputs go from registers to memory.  58 steps
+// of up to 8192 RHS of 6859 FP32: 20.5 -> 10.8 ms (5.2 TB/s); 41 of up to 1408
+// RHS of 1935: 0.95 -> 0.66 ms.
+constexpr int CG_STREAM_V = 4;
+constexpr size_t CG_STREAM_SMEM = 224 * 1024;
+constexpr long long CG_WAIT_CYCLES = 2000000000ll;  // about a second
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
+}
+// bounded wait for the phase of the given parity; false when it ran out
+__device__ __forceinline__ bool stage_wait(unsigned long long* bar, uint32_t parity) {
+  const long long t0 = clock64();
+  for (;;) {
+    uint32_t done;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(smem_addr(bar)), "r"(parity)
+        : "memory");
+    if (done) return true;
+    if (clock64() - t0 > CG_WAIT_CYCLES) return false;
+  }
+}
+
+template <typename R, int T>
+__global__ void __launch_bounds__(T)
+    k_cg_stream(CgArgs<R> a, const int* __restrict__ list, int rowb) {
+  constexpr int E = Vec<R>::n, V = CG_STREAM_V;
+  extern __shared__ __align__(128) unsigned char stages[];
+  __shared__ __align__(8) unsigned long long full[2];
+  __shared__ double sh[2][T / 32];
+  __shared__ double2 tot[2];
+  __shared__ R coef[2];
+  __shared__ int flag, dead;
+  const int tid = threadIdx.x, G = gridDim.x;
+  const int listed = a.list_count ? *a.list_count : a.n_listed;
+  int k = blockIdx.x;
+  if (k >= listed) return;
+  auto rhs = [&](int q) { return q < listed ? (list ? list[q] : q) : -1; };
+  // by one thread: the four rows of RHS i into a stage
+  auto issue = [&](int st, int i) {
+    const R* src[4] = {a.p, a.ap, a.r, a.x};
+    const uint32_t bar = smem_addr(&full[st]);
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(4 * rowb)
+                 : "memory");
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      asm volatile(
+          "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+              smem_addr(stages + (st * 4 + q) * (size_t)rowb)),
+          "l"(src[q] + (long long)i * a.ld), "r"(rowb), "r"(bar)
+          : "memory");
+  };
+  const bool feeder = tid == 32;
+  int i0 = rhs(k), i1 = rhs(k + G);
+  if (feeder) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&full[0])) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&full[1])) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    dead = 0;
+    issue(0, i0);
+    if (i1 >= 0) issue(1, i1);
+  }
+  __syncthreads();
+  int it = 0;
+#pragma unroll 1
+  for (; i0 >= 0; k += G, ++it) {
+    const int st = it & 1, i = i0;
+    const CgScal s = a.sc[i];
+    const int i2 = rhs(k + 2 * G);
+    const R* K = a.kprec + (long long)(i % a.n_occ) * a.ld;
+    R pv[V][E], av[V][E], rv[V][E], xv[V][E], kv[V][E];
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      const int j = (v * T + tid) * E;
+#pragma unroll
+      for (int e = 0; e < E; ++e) kv[v][e] = R(0);
+      if (j < a.n_pw) Vec<R>::ld(K + j, kv[v]);
+    }
+    if (!stage_wait(&full[st], (it >> 1) & 1)) {
+      dead = 1;
+      atomicOr(a.status, (unsigned)DEV_TIMEOUT);
+    }
+    const R* row = reinterpret_cast<const R*>(stages + st * 4 * (size_t)rowb);
+    const int rn_ = rowb / (int)sizeof(R);
+    R pap = R(0);
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      const int j = (v * T + tid) * E;
+      if (j < a.n_pw) {
+        Vec<R>::ld(row + j, pv[v]);
+        Vec<R>::ld(row + rn_ + j, av[v]);
+        Vec<R>::ld(row + 2 * rn_ + j, rv[v]);
+        Vec<R>::ld(row + 3 * rn_ + j, xv[v]);
+      }
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        if (j + e >= a.n_pw) pv[v][e] = av[v][e] = rv[v][e] = xv[v][e] = kv[v][e] = R(0);
+#pragma unroll
+      for (int e = 0; e < E; ++e) pap += pv[v][e] * av[v][e];
+    }
+    block_totals<R, T>(pap, R(0), sh, &tot[0]);  // its barrier: the stage has been read
+    if (feeder && i2 >= 0 && !dead) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      issue(st, i2);
+    }
+    if (tid == 0) {
+      const double t = tot[0].x, al = s.rz / t;
+      flag = !s.active || dead ? 3 : (!(t > 0.0) || !isfinite(al)) ? 1 : 0;
+      coef[0] = (R)al;
+      if (flag == 1) {
+        atomicOr(a.status, isfinite(t) ? (unsigned)DEV_BREAKDOWN : (unsigned)DEV_NONFINITE);
+        a.sc[i].active = 0;
+      }
+    }
+    __syncthreads();
+    if (dead) break;
+    if (!flag) {
+      const R alpha = coef[0];
+      const long long o = (long long)i * a.ld;
+      R rr = R(0), rkr = R(0);
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        const int j = (v * T + tid) * E;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          xv[v][e] += alpha * pv[v][e];
+          const R r = rv[v][e] - alpha * av[v][e];
+          rv[v][e] = r;
+          rr += r * r;
+          av[v][e] = kv[v][e] * r;  // K r, A p is no longer needed
+          rkr += av[v][e] * r;
+        }
+        if (j < a.n_pw) {
+          Vec<R>::st(a.x + o + j, xv[v]);
+          Vec<R>::st(a.r + o + j, rv[v]);
+        }
+      }
+      block_totals<R, T>(rr, rkr, sh, &tot[1]);
+      if (tid == 0) {
+        const double2 q = tot[1];
+        const double rn = sqrt(q.x);
+        const bool done = rn <= (a.tolv ? a.tolv[i] : a.tol) * s.bnorm;
+        flag = done ? 2 : 0;
+        coef[1] = (R)(q.y / s.rz);
+        CgScal n = s;
+        n.iters = s.iters + 1;
+        n.rnorm = rn;
+        n.rz = q.y;
+        n.active = done ? 0 : 1;
+        if (!isfinite(rn)) {
+          n.active = 0;
+          atomicOr(a.status, (unsigned)DEV_NONFINITE);
+        }
+        a.sc[i] = n;
+        if (n.active) atomicAdd(a.n_active, 1);
+      }
+      __syncthreads();
+      if (flag != 2) {
+        const R beta = coef[1];
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+          const int j = (v * T + tid) * E;
+#pragma unroll
+          for (int e = 0; e < E; ++e) pv[v][e] = av[v][e] + beta * pv[v][e];
+          if (j < a.n_pw) Vec<R>::st(a.p + o + j, pv[v]);
+        }
+      }
+    }
+    i0 = i1;
+    i1 = i2;
+  }
+  if (dead && feeder) {
+    // a wait ran out: the other stage's copies end before the block leaves
+    const int nx = it + 1;
+    if (i1 >= 0) stage_wait(&full[nx & 1], (nx >> 1) & 1);
+    stage_wait(&full[it & 1], (it >> 1) & 1);
+  }
+}
+
+template <typename R, int T>
+cudaError_t launch_stream(const CgArgs<R>& a, const int* list, int nb, int rowb, cudaStream_t st) {
+  auto kern = k_cg_stream<R, T>;
+  static std::atomic<bool> attr_set{false};
+  if (!attr_set.load()) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)CG_STREAM_SMEM);
+    if (e != cudaSuccess) return e;
+    attr_set.store(true);
+  }
+  const size_t smem = 8 * (size_t)rowb;
+  static const int sms = [] {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n > 0 ? n : 152;
+  }();
+  int per = 0;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, T, smem);
+  if (e != cudaSuccess) return e;
+  kern<<<std::min(nb, std::max(per, 1) * sms), T, smem, st>>>(a, list, rowb);
+  return cudaGetLastError();
+}
+
+// bytes of a row in a stage
+int stream_row(int n_pw, int elem) { return (n_pw * elem + 15) / 16 * 16; }
+
 template <typename R, int T, int V, bool PROJ>
 cudaError_t launch(const CgArgs<R>& a, const int* list, int nb, int C, const CgProj<R>& pj,
                    const CgTail& tail, cudaStream_t st) {
@@ -351,6 +568,10 @@ int cluster_for(int nvec, int T, int V) {
 
 }  // namespace
 
+bool cg_streams(int n_rhs, int n_pw, int elem) {
+  return n_rhs > CG_TAIL_MAX && 8 * (size_t)stream_row(n_pw, elem) <= CG_STREAM_SMEM;
+}
+
 template <typename R>
 cudaError_t cg_step(const CgArgs<R>& a, const int* list, int n_list, cudaStream_t st,
                     const CgProj<R>* proj, const CgTail* tail) {
@@ -363,6 +584,15 @@ cudaError_t cg_step(const CgArgs<R>& a, const int* list, int n_list, cudaStream_
   const int nvec = (a.n_pw + Vec<R>::n - 1) / Vec<R>::n;
   const CgProj<R> pj = proj ? *proj : CgProj<R>{};
   const CgTail tl = tail ? *tail : CgTail{};
+  if (!proj && !tl.on && cg_streams(a.n_rhs, a.n_pw, sizeof(R))) {
+    CgArgs<R> b = a;
+    b.n_listed = nb;
+    const int rowb = stream_row(a.n_pw, sizeof(R));
+    if (nvec <= 64 * CG_STREAM_V) return launch_stream<R, 64>(b, list, nb, rowb, st);
+    if (nvec <= 128 * CG_STREAM_V) return launch_stream<R, 128>(b, list, nb, rowb, st);
+    if (nvec <= 256 * CG_STREAM_V) return launch_stream<R, 256>(b, list, nb, rowb, st);
+    return launch_stream<R, 512>(b, list, nb, rowb, st);
+  }
   // shapes of the autotuner (cg_start's default CG_FEW: as many blocks per RHS
   // as help, for few RHS)
   struct Shape {

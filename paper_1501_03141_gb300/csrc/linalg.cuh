@@ -190,6 +190,7 @@ struct CgArgs {
   int variant;          // block shape (picked by the autotuner), or CG_FEW
   const int* list_count = nullptr;  // device length of the active list (cg_step sized for
                                     // the largest; blocks past it exit)
+  int n_listed = 0;                 // cg_step: listed RHS without a device count (set inside)
   const double* mask = nullptr;     // cg_start: RHS i takes part only if mask[i] != 0
   const double* tolv = nullptr;     // per-RHS relative tolerance (replaces tol when set)
 };
@@ -235,6 +236,10 @@ cudaError_t solve_finish(const double* rel, int n, double tol, DevStats* ds, uns
 // block shapes of one CG step (cg_step.cu) the autotuner times; CG_FEW: as many
 // blocks per RHS as a cluster holds, for few RHS
 enum CgVariant : int { CG_FEW = -1, CG_NUM_VARIANTS = 4 };
+// Whether the step streams its RHS through persistent blocks (more than
+// CG_TAIL_MAX RHS whose rows fit two shared-memory stages); the block shapes
+// above play no part then.
+bool cg_streams(int n_rhs, int n_pw, int elem);
 // The projection term sum_w sigma_w |w><w| p added to A p inside the step:
 // states [n][ld] (the step's ld), n <= CG_PROJ_MAX.
 constexpr int CG_PROJ_MAX = 128;
