@@ -132,6 +132,16 @@ struct CgGraph {
   cudaGraphExec_t exec;
 };
 
+// The refinement rounds after the first, captured as a while node over rounds
+// (each with the CG loop's node inside), valid for what it was captured with.
+struct RoundsGraph {
+  int prec, sys, n, cg_variant, proj_variant, tune_gen;
+  int check, round, body;  // kernels before the first round, per round, per CG step
+  const void *b, *x, *dn, *its, *rel, *r64, *ad;
+  unsigned long long ws_gen, budget_ns;
+  cudaGraphExec_t exec;
+};
+
 struct pdep_ctx {
   int device = 0;
   pdep_options opt{};
@@ -149,6 +159,8 @@ struct pdep_ctx {
   unsigned long long ws_gen = 0;  // bumped whenever a workspace buffer is reallocated
   unsigned long long budget_ns = 0;   // clock_budget_cycles in ns of %globaltimer
   std::vector<CgGraph> cg_graphs;     // executable CG-loop graphs, released in pdep_destroy
+  std::vector<RoundsGraph> rounds_graphs;  // likewise
+  int round_launches = 0;             // kernels per round of the last rounds graph
   int body_launches[2] = {0, 0};      // kernels per CG step of the last graph (FP32, FP64)
   long long graph_launches = 0;       // CG graphs launched
   long long prologue_launches = 0;    // kernels before their loops
@@ -1206,89 +1218,106 @@ CgTail step_tail(const pdep_ctx* c, int* list, int max_iter, int prec,
 // a step is then the transform's launches and one more.
 // Launches inside are sized for n; the kernels read the list length from
 // the device loop state.  All workspace is allocated beforehand (cg_workspace).
+// captures what fn enqueues on the capture stream as a child graph of g behind
+// 'after' (may be null); launches counts its kernels
+template <typename F>
+int add_captured(pdep_ctx* c, cudaGraph_t g, cudaGraphNode_t after, cudaGraphNode_t* node,
+                 int* launches, F fn) {
+  cudaStream_t cs = c->cap_stream;
+  cudaGraph_t part = nullptr;
+  CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeRelaxed));
+  capture_begin();
+  const int status = fn(cs);
+  *launches += capture_end();
+  const cudaError_t e = cudaStreamEndCapture(cs, &part);
+  if (status != PDEP_OK || e != cudaSuccess) {
+    if (part) cudaGraphDestroy(part);
+    cudaGetLastError();
+    if (status != PDEP_OK) return status;
+    CK(e);
+  }
+  const cudaError_t add = cudaGraphAddChildGraphNode(node, g, after ? &after : nullptr,
+                                                     after ? 1 : 0, part);
+  cudaGraphDestroy(part);
+  CK(add);
+  return PDEP_OK;
+}
+
+// adds a while node behind 'after' whose condition is h; its body graph
+int add_while(cudaGraph_t g, cudaGraphNode_t after, cudaGraphConditionalHandle h,
+              cudaGraphNode_t* node, cudaGraph_t* body) {
+  cudaGraphNodeParams cp{};
+  cp.type = cudaGraphNodeTypeConditional;
+  cp.conditional.handle = h;
+  cp.conditional.type = cudaGraphCondTypeWhile;
+  cp.conditional.size = 1;
+  CK(cudaGraphAddNode(node, g, &after, nullptr, 1, &cp));
+  *body = cp.conditional.phGraph_out[0];
+  return PDEP_OK;
+}
+
+// The CG loop's nodes in graph g, behind 'after' (may be null).
 template <typename R>
-int capture_cg_graph(pdep_ctx* c, SysData& s, CgArgs<R> a, const R* b, int n, int max_iter,
-                     int* list, CgGraph* gr) {
-  cudaGraphExec_t* out = &gr->exec;
+int add_cg_loop(pdep_ctx* c, SysData& s, CgArgs<R> a, const R* b, int n, int max_iter, int* list,
+                cudaGraph_t g, cudaGraphNode_t after, cudaGraphNode_t* node, int* prologue,
+                int* per_step) {
   const bool tail = n <= CG_TAIL_MAX, fuse = tail && few_projection<R>(c, s, n);
   if (tail) a.variant = n < 256 ? (int)CG_FEW : a.variant;
   const int pi = sizeof(R) == 8 ? 1 : 0;
-  cudaStream_t cs = c->cap_stream;
-  const unsigned long long gen = c->ws_gen;
-  cudaGraph_t g = nullptr, pro = nullptr, body = nullptr;
   cudaGraphConditionalHandle h = 0;
-  int status = PDEP_OK, launches = 0;
-  auto abort_capture = [&]() {
-    cudaGraph_t junk = nullptr;
-    cudaStreamEndCapture(cs, &junk);
-    if (junk && junk != body) cudaGraphDestroy(junk);
-    cudaGetLastError();
-  };
-  auto chk = [&](cudaError_t e) {
-    if (e != cudaSuccess && status == PDEP_OK) {
-      set_last_error(__FILE__, __LINE__, cudaGetErrorString(e));
-      status = PDEP_ERR_CUDA;
-    }
-    return e == cudaSuccess;
-  };
-  if (!chk(cudaGraphCreate(&g, 0))) return status;
-  if (chk(cudaGraphConditionalHandleCreate(&h, g, 0, 0)) &&
-      chk(cudaStreamBeginCapture(cs, cudaStreamCaptureModeRelaxed))) {
-    capture_begin();
-    bool ok = chk(cudaMemsetAsync(&c->d_loop->active, 0, sizeof(int), cs)) &&
-              chk(cudaMemsetAsync(c->d_counter, 0, sizeof(int), cs)) &&
-              chk(cg_start<R>(a, b, s.ld, cs)) &&
-              (!tail || chk(active_list(a.sc, n, list, &c->d_loop->listed, cs))) &&
-              chk(loop_begin(c->d_loop, max_iter, h, 1, cs));
-    gr->prologue = capture_end();
-    if (ok) {
-      chk(cudaStreamEndCapture(cs, &pro));
-    } else {
-      abort_capture();
-    }
-  }
-  cudaGraphNode_t pn = nullptr, wn = nullptr;
-  cudaGraphNodeParams cp{};
-  if (status == PDEP_OK && chk(cudaGraphAddChildGraphNode(&pn, g, nullptr, 0, pro))) {
-    cp.type = cudaGraphNodeTypeConditional;
-    cp.conditional.handle = h;
-    cp.conditional.type = cudaGraphCondTypeWhile;
-    cp.conditional.size = 1;
-    if (chk(cudaGraphAddNode(&wn, g, &pn, nullptr, 1, &cp))) body = cp.conditional.phGraph_out[0];
-  }
-  if (status == PDEP_OK &&
-      chk(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed))) {
-    capture_begin();
-    bool ok = tail || chk(active_list_reset(a.sc, n, list, &c->d_loop->listed, &c->d_loop->active, cs));
-    if (ok) {
-      const int r = apply_h<R>(c, s, a.p, (R*)a.ap, n, list, n, true, !fuse, cs, nullptr,
-                               &c->d_loop->listed);
-      if (r != PDEP_OK) {
-        status = r;
-        ok = false;
-      }
-    }
+  CK(cudaGraphConditionalHandleCreate(&h, g, 0, 0));
+  cudaGraphNode_t pn = nullptr, bn = nullptr;
+  RET(add_captured(c, g, after, &pn, prologue, [&](cudaStream_t cs) -> int {
+    CK(cudaMemsetAsync(&c->d_loop->active, 0, sizeof(int), cs));
+    CK(cudaMemsetAsync(c->d_counter, 0, sizeof(int), cs));
+    CK(cg_start<R>(a, b, s.ld, cs));
+    if (tail) CK(active_list(a.sc, n, list, &c->d_loop->listed, cs));
+    CK(loop_begin(c->d_loop, max_iter, h, 1, cs));
+    return PDEP_OK;
+  }));
+  cudaGraph_t body = nullptr;
+  RET(add_while(g, pn, h, node, &body));
+  return add_captured(c, body, nullptr, &bn, per_step, [&](cudaStream_t cs) -> int {
+    if (!tail) CK(active_list_reset(a.sc, n, list, &c->d_loop->listed, &c->d_loop->active, cs));
+    RET(apply_h<R>(c, s, a.p, (R*)a.ap, n, list, n, true, !fuse, cs, nullptr, &c->d_loop->listed));
     a.list_count = &c->d_loop->listed;
     const CgProj<R> pj = step_projection<R>(s);
     const CgTail tl = step_tail(c, list, max_iter, pi, h, 1);
-    ok = ok && chk(cg_step<R>(a, list, n, cs, fuse ? &pj : nullptr, tail ? &tl : nullptr)) &&
-         (tail ||
-          chk(loop_next(c->d_loop, max_iter, c->budget_ns, c->d_status, pi, h, 1, cs)));
-    launches = capture_end();
-    if (ok) {
-      cudaGraph_t got = body;
-      chk(cudaStreamEndCapture(cs, &got));
-    } else {
-      abort_capture();
-    }
-  }
+    CK(cg_step<R>(a, list, n, cs, fuse ? &pj : nullptr, tail ? &tl : nullptr));
+    if (!tail) CK(loop_next(c->d_loop, max_iter, c->budget_ns, c->d_status, pi, h, 1, cs));
+    return PDEP_OK;
+  });
+}
+
+// fn(g) adds the nodes of a new graph; instantiates it
+template <typename F>
+int build_graph(pdep_ctx* c, cudaGraphExec_t* out, F fn) {
+  const unsigned long long gen = c->ws_gen;
+  cudaGraph_t g = nullptr;
+  CK(cudaGraphCreate(&g, 0));
+  int status = fn(g);
   if (status == PDEP_OK && c->ws_gen != gen)
     status = fail(PDEP_ERR_CUDA, "workspace moved while capturing a CG graph");
-  if (status == PDEP_OK) chk(cudaGraphInstantiate(out, g, 0));
-  if (pro) cudaGraphDestroy(pro);
+  if (status == PDEP_OK) {
+    const cudaError_t e = cudaGraphInstantiate(out, g, 0);
+    if (e != cudaSuccess) {
+      set_last_error(__FILE__, __LINE__, cudaGetErrorString(e));
+      status = PDEP_ERR_CUDA;
+    }
+  }
   cudaGraphDestroy(g);
-  gr->body = launches;
   return status;
+}
+
+template <typename R>
+int capture_cg_graph(pdep_ctx* c, SysData& s, const CgArgs<R>& a, const R* b, int n, int max_iter,
+                     int* list, CgGraph* gr) {
+  gr->prologue = gr->body = 0;
+  return build_graph(c, &gr->exec, [&](cudaGraph_t g) -> int {
+    cudaGraphNode_t node = nullptr;
+    return add_cg_loop<R>(c, s, a, b, n, max_iter, list, g, nullptr, &node, &gr->prologue,
+                          &gr->body);
+  });
 }
 
 // Sternheimer PCG on (H - eps_v + sum_w sigma_w |w><w|) x = b for n RHS
@@ -1298,22 +1327,19 @@ int capture_cg_graph(pdep_ctx* c, SysData& s, CgArgs<R> a, const R* b, int n, in
 // control kernel (no host round trip per step).  While the autotuner is
 // still timing launch shapes (or use_graph is 0) the same steps are launched
 // from a host loop that reads the control flag after each step.
+// H x inside the loop is the inner CG's (restored on every return)
+struct InnerFlag {
+  bool& f;
+  bool old;
+  InnerFlag(bool& ff, bool v) : f(ff), old(ff) { f = v; }
+  ~InnerFlag() { f = old; }
+};
 template <typename R>
-int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int max_iter,
-            CgScal* sc, const double* mask, cudaStream_t st, const double* tolv) {
-  const int si = (int)(&s - c->sys.data());
-  // H x inside this loop is the inner CG's (restored on every return)
-  struct InnerFlag {
-    bool& f;
-    bool old;
-    InnerFlag(bool& ff, bool v) : f(ff), old(ff) { f = v; }
-    ~InnerFlag() { f = old; }
-  } inner_flag(c->cg_inner, sizeof(R) == 4);
+int cg_setup(pdep_ctx* c, SysData& s, R* x, int n, double tol, CgScal* sc, const double* mask,
+             const double* tolv, CgArgs<R>* out, int** list) {
   R *r, *p, *ap;
-  int* list;
-  RET(cg_workspace<R>(c, s, n, &r, &p, &ap, &list));
-  const int pi = sizeof(R) == 8 ? 1 : 0;
-  CgArgs<R> a{};
+  RET(cg_workspace<R>(c, s, n, &r, &p, &ap, list));
+  CgArgs<R>& a = *out;
   a.x = x;
   a.r = r;
   a.p = p;
@@ -1330,6 +1356,24 @@ int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int ma
   a.n_active = &c->d_loop->active;
   a.mask = mask;
   a.tolv = tolv;
+  return PDEP_OK;
+}
+// the projection kernel apply_h uses inside a captured loop
+int captured_proj(const pdep_ctx* c) {
+  const int pv = c->opt.proj_variant >= 0 ? c->opt.proj_variant : c->proj_variant;
+  return pv < 0 ? 1 : pv;
+}
+
+template <typename R>
+int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int max_iter,
+            CgScal* sc, const double* mask, cudaStream_t st, const double* tolv) {
+  const int si = (int)(&s - c->sys.data());
+  InnerFlag inner_flag(c->cg_inner, sizeof(R) == 4);
+  const int pi = sizeof(R) == 8 ? 1 : 0;
+  CgArgs<R> a{};
+  int* list;
+  RET(cg_setup<R>(c, s, x, n, tol, sc, mask, tolv, &a, &list));
+  R *p = a.p, *ap = (R*)a.ap;
   // loops under 256 RHS are never timed by the autotuner: they run the
   // current (or default) shapes and are captured right away
   const bool graph = c->opt.use_graph && (tuned(c, s, pi, n) || n < 256);
@@ -1383,8 +1427,7 @@ int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int ma
     return PDEP_OK;
   }
   a.variant = cg_variant_of(c, pi);
-  int pv = c->opt.proj_variant >= 0 ? c->opt.proj_variant : c->proj_variant;
-  if (pv < 0) pv = 1;  // what apply_h uses while the projection kernel is untimed
+  const int pv = captured_proj(c);
   CgGraph* g = nullptr;
   for (CgGraph& e : c->cg_graphs)
     if (e.prec == pi && e.sys == si && e.n == n && e.max_iter == max_iter && e.tol == tol &&
@@ -1441,8 +1484,8 @@ int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int ma
 // recomputed residual drifted above the recursion's; the mixed modes run
 // each FP32 inner solve to inner_tol.  d_refine[0] holds a round's
 // unconverged count: the A delta and the residual update run on that many
-// listed RHS (launches sized for n).  Rounds whose list is empty cost only
-// their launches.
+// listed RHS (launches sized for n).  The rounds after the first run inside a
+// graph (use_graph) as long as RHS need them.
 // Relative reduction each FP32 inner solve aims for.  With BF16
 // coefficients the CG operator is perturbed at about 2^-9 of the projection
 // term, so a round gains little more than ~3e-3 however long the inner CG
@@ -1484,31 +1527,111 @@ int refine_rounds(pdep_ctx* c, SysData& s, const double* b, const double* xd, do
   CK(cudaMemsetAsync(x, 0, sizeof(double) * (size_t)n * s.ld, st));
   CK(fill_value(rel, n, 1.0, st));
   int* n_un = c->d_refine;
-  for (int round = 0; round < c->opt.max_refine; ++round) {
-    NvtxRange nv("refinement_round");
-    CK(unconverged_list(rel, tol, n, list, n_un, st, &c->d_dstats->rounds_cur));
-    CK(refine_prepare<Ri>(r64, s.ld, s.n_pw, n, rel, tol, ri, s.ld, rn, st, tolv,
+  const int pi = fp64 ? 1 : 0;
+  const double inner = fp64 ? 0.0 : inner_tol_of(c);
+  const int max_iter = fp64 ? c->opt.cg_max_iter : c->opt.inner_max_iter;
+  auto prepare = [&](int round, cudaStream_t q) -> int {
+    CK(refine_prepare<Ri>(r64, s.ld, s.n_pw, n, rel, tol, ri, s.ld, rn, q, tolv,
                           (round == 0 ? 0.9 : 0.5) * tol, 0.5));
-    if (fp64)
-      RET(cg_loop<Ri>(c, s, ri, di, n, 0.0, c->opt.cg_max_iter, sc, rn, st, tolv));
-    else
-      RET(cg_loop<Ri>(c, s, ri, di, n, inner_tol_of(c), c->opt.inner_max_iter, sc, rn, st,
-                      nullptr));
-    CK(cg_collect(sc, n, its_total, c->d_dstats, st));
+    return PDEP_OK;
+  };
+  auto update = [&](int round, cudaStream_t q) -> int {
+    CK(cg_collect(sc, n, its_total, c->d_dstats, q));
     // delta = rn d (+ xd in the first round, when every RHS is listed)
     const double* xr = round == 0 ? xd : nullptr;
     const bool f32_round = f32_later && round > 0;
-    CK(refine_delta<Ri>(x, dl, s.ld, di, s.ld, s.n_pw, n, rn, xr, st, f32_round ? dlf : nullptr));
+    CK(refine_delta<Ri>(x, dl, s.ld, di, s.ld, s.n_pw, n, rn, xr, q, f32_round ? dlf : nullptr));
     if (f32_round) {
-      RET(apply_h<float>(c, s, dlf, adf, n, list, n, true, true, st, dn, n_un));
-      CK(residual_update(r64, adf, b, s.ld, s.n_pw, n, rel, list, xr, s.d_sigma64, s.n_occ, st,
+      RET(apply_h<float>(c, s, dlf, adf, n, list, n, true, true, q, dn, n_un));
+      CK(residual_update(r64, adf, b, s.ld, s.n_pw, n, rel, list, xr, s.d_sigma64, s.n_occ, q,
                          n_un));
-      continue;
+      return PDEP_OK;
     }
-    RET(apply_h<double>(c, s, dl, ad, n, list, n, true, true, st, dn, n_un,
+    RET(apply_h<double>(c, s, dl, ad, n, list, n, true, true, q, dn, n_un,
                         !fp64 && c->opt.df_refine));
-    CK(residual_update(r64, ad, b, s.ld, s.n_pw, n, rel, list, xr, s.d_sigma64, s.n_occ, st,
-                       n_un));
+    CK(residual_update(r64, ad, b, s.ld, s.n_pw, n, rel, list, xr, s.d_sigma64, s.n_occ, q, n_un));
+    return PDEP_OK;
+  };
+  for (int round = 0; round < c->opt.max_refine; ++round) {
+    NvtxRange nv("refinement_round");
+    if (round == 1 && c->opt.use_graph && (tuned(c, s, pi, n) || n < 256)) {
+      // The rounds after the first are the same launches: one graph whose while
+      // node runs a round only if an RHS needs it.  (Enqueued one by one, each
+      // empty round cost its launches, some 58 us, and most solves need one or
+      // two of the six.)
+      const int si = (int)(&s - c->sys.data()), variant = cg_variant_of(c, pi), pv = captured_proj(c);
+      CgArgs<Ri> a{};
+      int* cgl;
+      RET(cg_setup<Ri>(c, s, di, n, inner, sc, rn, tolv, &a, &cgl));
+      a.variant = variant;
+      if (f32_later) {
+        cpx<float>* b1;
+        float* S;
+        RET(ws(c, "b1_32", b1_count(s, (n + 1) / 2), &b1));
+        RET(ws(c, "pv_32", (size_t)((s.n_ext + 3) & ~3) * std::max(n, 1), &S));
+      }
+      RoundsGraph* g = nullptr;
+      for (RoundsGraph& e : c->rounds_graphs)
+        if (e.prec == pi && e.sys == si && e.n == n && e.b == b && e.x == x && e.dn == dn &&
+            e.its == its_total && e.rel == rel && e.r64 == r64 && e.ad == ad &&
+            e.ws_gen == c->ws_gen && e.budget_ns == c->budget_ns && e.cg_variant == variant &&
+            e.proj_variant == pv && e.tune_gen == c->tune_gen)
+          g = &e;
+      if (!g) {
+        RoundsGraph e{pi, si, n, variant, pv, c->tune_gen, 0, 0, 0, b, x, dn, its_total, rel,
+                      r64, ad, c->ws_gen, c->budget_ns, nullptr};
+        RET(build_graph(c, &e.exec, [&](cudaGraph_t top) -> int {
+          cudaGraphConditionalHandle h = 0;
+          CK(cudaGraphConditionalHandleCreate(&h, top, 0, 0));
+          auto check = [&](int first, cudaStream_t q) -> int {
+            CK(unconverged_list(rel, tol, n, list, n_un, q, nullptr));
+            CK(rounds_next(c->d_loop, n_un, first, 1, c->opt.max_refine,
+                           &c->d_dstats->rounds_cur, h, q));
+            return PDEP_OK;
+          };
+          cudaGraphNode_t first = nullptr, loop = nullptr, pre = nullptr, cg = nullptr, up = nullptr;
+          cudaGraph_t body = nullptr;
+          RET(add_captured(c, top, nullptr, &first, &e.check,
+                           [&](cudaStream_t q) { return check(1, q); }));
+          RET(add_while(top, first, h, &loop, &body));
+          RET(add_captured(c, body, nullptr, &pre, &e.round,
+                           [&](cudaStream_t q) { return prepare(1, q); }));
+          {
+            InnerFlag inner_flag(c->cg_inner, !fp64);
+            RET(add_cg_loop<Ri>(c, s, a, ri, n, max_iter, cgl, body, pre, &cg, &e.round, &e.body));
+          }
+          return add_captured(c, body, cg, &up, &e.round, [&](cudaStream_t q) -> int {
+            RET(update(1, q));
+            return check(0, q);
+          });
+        }));
+        if (c->rounds_graphs.size() >= 16) {
+          cudaGraphExecDestroy(c->rounds_graphs.front().exec);
+          c->rounds_graphs.erase(c->rounds_graphs.begin());
+        }
+        c->rounds_graphs.push_back(e);
+        g = &c->rounds_graphs.back();
+      }
+      {
+        ProfScope ps(fp64 ? PC_CG_GRAPH_F64 : PC_CG_GRAPH_F32, st, 0.0, 0.0);
+        CK(cudaGraphLaunch(g->exec, st));
+      }
+      ++c->graph_launches;
+      c->prologue_launches += g->check;
+      c->round_launches = g->round;
+      c->body_launches[pi] = g->body;
+      break;
+    }
+    CK(unconverged_list(rel, tol, n, list, n_un, st, &c->d_dstats->rounds_cur));
+    if (round > 0 && !c->opt.use_graph) {
+      // the host loop reads its control words anyway
+      CK(cudaMemcpyAsync(c->h_pin, n_un, sizeof(int), cudaMemcpyDeviceToHost, st));
+      CK(cudaStreamSynchronize(st));
+      if (c->h_pin[0] == 0) break;
+    }
+    RET(prepare(round, st));
+    RET(cg_loop<Ri>(c, s, ri, di, n, inner, max_iter, sc, rn, st, tolv));
+    RET(update(round, st));
   }
   return PDEP_OK;
 }
@@ -1697,7 +1820,7 @@ int reset_stats(pdep_ctx* c, cudaStream_t st) {
 // Synchronises st and fills the solve statistics (device counters included).
 int read_stats(pdep_ctx* c, pdep_stats* out, cudaStream_t st) {
   DevStats d;
-  unsigned long long steps[2];
+  unsigned long long steps[3];
   CK(cudaMemcpyAsync(&d, c->d_dstats, sizeof(DevStats), cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(steps, c->d_loop->steps, sizeof(steps), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
@@ -1716,6 +1839,7 @@ int read_stats(pdep_ctx* c, pdep_stats* out, cudaStream_t st) {
   // launches outside graphs are counted on the host; a graph contributes its
   // prologue per launch and its body per step, the steps counted on the device (loop_next counts eager steps too: those are subtracted)
   long long in_graphs = c->prologue_launches;
+  in_graphs += (long long)steps[2] * c->round_launches;
   for (int pi = 0; pi < 2; ++pi)
     in_graphs += ((long long)steps[pi] - c->eager_steps[pi]) * c->body_launches[pi];
   out->kernel_launches = (launch_count() - c->st_launch0) + in_graphs;
@@ -1898,6 +2022,8 @@ void pdep_destroy(pdep_ctx* c) {
   c->eig_graphs.release();
   for (CgGraph& g : c->cg_graphs) cudaGraphExecDestroy(g.exec);
   c->cg_graphs.clear();
+  for (RoundsGraph& g : c->rounds_graphs) cudaGraphExecDestroy(g.exec);
+  c->rounds_graphs.clear();
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   if (c->d_loop) cudaFree(c->d_loop);
   if (c->d_dstats) cudaFree(c->d_dstats);

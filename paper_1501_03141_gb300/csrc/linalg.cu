@@ -1367,6 +1367,26 @@ cudaError_t loop_next(CgLoopState* ls, int max_iter, unsigned long long budget_n
   return cudaGetLastError();
 }
 
+__global__ void k_rounds_next(CgLoopState* ls, const int* n_un, int first, int done, int max_rounds,
+                              int* rounds, cudaGraphConditionalHandle h) {
+  if (first)
+    ls->round = done;
+  else
+    ls->steps[2] += 1;
+  const bool go = *n_un > 0 && ls->round < max_rounds;
+  if (go) {
+    ls->round += 1;
+    *rounds += 1;
+  }
+  cudaGraphSetConditional(h, go ? 1u : 0u);
+}
+cudaError_t rounds_next(CgLoopState* ls, const int* n_un, int first, int done, int max_rounds,
+                        int* rounds, cudaGraphConditionalHandle h, cudaStream_t st) {
+  count_launch();
+  k_rounds_next<<<1, 1, 0, st>>>(ls, n_un, first, done, max_rounds, rounds, h);
+  return cudaGetLastError();
+}
+
 __global__ void k_cg_collect(const CgScal* __restrict__ sc, int n, int* its_total, DevStats* ds) {
   unsigned long long sum = 0;
   int mx = 0;

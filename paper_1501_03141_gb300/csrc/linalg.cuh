@@ -205,7 +205,9 @@ struct CgLoopState {
   int iter;                       // steps done in this loop
   int go;                         // 1 while another step is due
   unsigned long long t0;          // %globaltimer (ns) at the loop start
-  unsigned long long steps[2];    // steps over all loops (FP32, FP64), for launch counts
+  unsigned long long steps[3];    // steps over all loops (FP32, FP64), and refinement rounds
+                                  // run inside graphs, for launch counts
+  int round;                      // refinement round of the enclosing graph
 };
 // Device statistics of the Sternheimer solves since the last reset.
 struct DevStats {
@@ -226,6 +228,12 @@ cudaError_t loop_begin(CgLoopState* ls, int max_iter, cudaGraphConditionalHandle
 cudaError_t loop_next(CgLoopState* ls, int max_iter, unsigned long long budget_ns,
                       unsigned* status, int prec, cudaGraphConditionalHandle h, int has_handle,
                       cudaStream_t st);
+// Loop control of the refinement rounds inside a graph: another round runs while
+// *n_un RHS are unconverged and fewer than max_rounds have run (first: the check
+// before them, with 'done' rounds run already); a round that starts is counted
+// in *rounds.
+cudaError_t rounds_next(CgLoopState* ls, const int* n_un, int first, int done, int max_rounds,
+                        int* rounds, cudaGraphConditionalHandle h, cudaStream_t st);
 // After a CG loop: its_total[i] += sc[i].iters (its_total may be null), and
 // the sum / largest count into ds.
 cudaError_t cg_collect(const CgScal* sc, int n, int* its_total, DevStats* ds, cudaStream_t st);
