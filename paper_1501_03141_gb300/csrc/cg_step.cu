@@ -310,7 +310,6 @@ __global__ void __launch_bounds__(T)
   if (tid == 0) {
     CgLoopState* ls = tail.loop;
     *tail.ticket = 0;
-    ls->listed = total;
     ls->active = total;
     const int it = ls->iter + 1;
     ls->iter = it;
@@ -320,6 +319,7 @@ __global__ void __launch_bounds__(T)
       go = false;
       atomicOr(a.status, (unsigned)DEV_TIMEOUT);
     }
+    ls->listed = go ? total : 0;  // a further step of the same graph pass is empty
     ls->go = go ? 1 : 0;
     if (tail.has_handle) cudaGraphSetConditional(tail.handle, go ? 1u : 0u);
   }
