@@ -44,13 +44,11 @@ WORKLOAD = ("cube48: 48^3 grid, L=20 bohr, 64 Gaussian wells (seed 1501031411), 
             "N_pdep=128, 6 Davidson iterations, Sternheimer tol 1e-10")
 # Nominal units x clocks of a GB300 (152 SMs, 128 FP32 lanes each, 2070 MHz):
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12     # 80.5 TFLOP/s FFMA
-FP64_PEAK_TFLOPS = 1.25                                # nominal FP64 rate of GB300
-# Double-float arithmetic (pairs of FP32 numbers) on the FP32 pipe: a line-FFT
-# flop costs about 9.4 FP32 instructions on average (a double-float add is
-# 11 instructions, a multiply 7; a radix-2 butterfly with twiddle is 4
-# multiplies and 6 adds for 10 algorithmic flops), against the pipe's
-# 152 x 128 instructions per clock
-DF64_PEAK_TFLOPS = 152 * 128 * 2.070e9 / 9.4 / 1e12     # 4.28 TFLOP/s FP64-equivalent
+# FP64 products run as exact digit products on the FP16 tensor cores: 36 FP16
+# products each (28 in the mixed refinement), mma.sync at the 1018 multiply-adds
+# per SM and clock it was measured to retire.  (The FP64 pipe: 1.25 TFLOP/s.)
+FP64_PEAK_TFLOPS = 152 * 1018 * 2 * 2.070e9 / 36 / 1e12    # 17.8 TFLOP/s FP64-equivalent
+DF64_PEAK_TFLOPS = 152 * 1018 * 2 * 2.070e9 / 28 / 1e12    # 22.9 TFLOP/s FP64-equivalent
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic.json")
 CSRC = os.path.join(ROOT, "paper_1501_03141_gb300", "csrc")
@@ -270,9 +268,10 @@ def roofline(prof):
         r = {"bound": "alu", "achieved": round(tfl, 3), "peak": round(alu_peak, 3),
              "unit": "TFLOP/s", "frac": round(f_alu, 4),
              "peak_source": "derived from unit counts x 2070 MHz (" +
-                            ("152 SM x 128 FP32 lanes / 9.4 instructions per double-float "
-                             "flop" if name.endswith("df64") else
-                             "FP64 nominal 1.25 TFLOP/s" if name.endswith("f64") else
+                            ("152 SM x 1018 FP16 multiply-adds x 2 / 28 digit products"
+                             if name.endswith("df64") else
+                             "152 SM x 1018 FP16 multiply-adds x 2 / 36 digit products"
+                             if name.endswith("f64") else
                              "152 SM x 128 FP32 lanes x 2") + ")",
              "hbm_frac_of_" + src: round(f_hbm, 4)}
     else:

@@ -165,21 +165,24 @@ typedef struct {
                                 keep the fastest; 0: fixed defaults */
   int use_graph;             /* 1 (default): each Sternheimer CG loop runs as one CUDA
                                 graph with a device-driven while node (no host round trip
-                                per step) once the autotuner has fixed the launch shapes;
+                                per step) once the autotuner has fixed the launch shapes,
+                                and the refinement rounds after the first as one more;
                                 0: a host loop that reads the loop state after every step */
   int df_refine;             /* mixed modes, precision of the refinement's A delta (and of
                                 the density response accumulated with it); vectors,
                                 residuals and the density stay FP64 throughout.
-                                2 (default): transforms in double-float arithmetic (pairs
-                                of FP32 numbers, about 48 significant bits; the FP32 pipe
-                                runs 64x the FP64 rate) in the first round, FP32 in later
+                                2 (default): transforms as exact products of seven base-256
+                                digits on the tensor cores (below 2e-15 of the result; the
+                                FP64 path takes eight) in the first round, FP32 in later
                                 rounds, whose correction is about inner_tol of the
                                 solution, so that FP32 errs by ~1e-7 inner_tol ||b||;
-                                1: double-float in every round; 0: FP64 transforms */
+                                1: seven digits in every round; 0: eight */
   int fused_hpsi;            /* 1 (default): the FP32 H x of the inner CG on the cubic grids
                                 24^3 .. 48^3 in one launch that keeps each item's column
-                                scratch in shared memory; 0: three launches through a
-                                global-memory scratch (always used for other grids) */
+                                scratch in shared memory (for few vectors on 32^3 .. 48^3,
+                                where a block per pair leaves SMs idle, in three); 0: three
+                                launches through a global-memory scratch (always used for
+                                other grids) */
 } pdep_options;
 
 typedef struct {
@@ -192,15 +195,16 @@ typedef struct {
   double max_cg_residual;       /* largest final ||b - A x|| / ||b||, recomputed in FP64 */
   double max_dav_residual;      /* largest final ||chi0bar x - theta x|| / |theta_1| */
   double seconds;               /* wall time of the call */
-  int cg_variant;               /* CG-step launch shape the autotuner chose (-1: untuned) */
+  int cg_variant;               /* CG-step launch shape the autotuner chose (-1: untuned; loops
+                                   of more than 1024 RHS have a shape of their own) */
   int proj_variant;             /* FP32 projection kernel in use (-1: untuned, 0, 1, 2;
                                    3: PDEP_MIXED_BF16, BF16 coefficients in the inner CG) */
   int chi0_chunks;              /* perturbation chunks of the last chi0bar application */
   long long kernel_launches;    /* library kernels the call ran, those inside CUDA graphs
                                    included (graph steps counted on the device) */
-  long long graph_launches;     /* CG-loop graphs launched */
-  int fused_planes;             /* x-planes per group of the fused FP32 transform the
-                                   autotuner chose (-1: untuned or not used) */
+  long long graph_launches;     /* CG-loop and refinement graphs launched */
+  int fused_planes;             /* x-planes a block of the fused FP32 transform works on at
+                                   once, as the autotuner chose (-1: untuned or not used) */
   int gemm_shape;               /* split-K of the FP64 projection GEMMs the autotuner chose: 0 the
                                    default, 1 half of it, 2 twice, 3 four times (-1 untuned) */
 } pdep_stats;
@@ -334,7 +338,7 @@ int pdep_lanczos(pdep_ctx* ctx, int sys, const double* R, int n, int n_steps, co
 /* y = H x for n sphere vectors x [n][n_pw] -> y [n][n_pw], H = -nabla^2/2 + V
  * (the local-potential Hamiltonian of the setup), evaluated with the pruned
  * sphere <-> grid transforms; precision PDEP_FP64, PDEP_MIXED (FP32
- * transforms) or PDEP_APPLY_DF64 (double-float transforms on FP64 vectors,
+ * transforms) or PDEP_APPLY_DF64 (seven-digit transforms on FP64 vectors,
  * those of the mixed modes' refinement).  This is the H*psi kernel the
  * Sternheimer CG applies. */
 #define PDEP_APPLY_DF64 3

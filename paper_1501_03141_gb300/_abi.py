@@ -31,7 +31,7 @@ PDEP_FP64 = 0
 PDEP_MIXED_TF32 = 1
 PDEP_MIXED_BF16 = 2
 PDEP_MIXED = PDEP_MIXED_TF32
-PDEP_APPLY_DF64 = 3   # pdep_apply_hamiltonian: double-float transforms
+PDEP_APPLY_DF64 = 3   # pdep_apply_hamiltonian: seven-digit transforms
 
 PDEP_SCREEN_CHIBAR = 0
 PDEP_SCREEN_EPSINV = 1

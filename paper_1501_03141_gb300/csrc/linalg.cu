@@ -311,7 +311,9 @@ __global__ void k_jacobi_sweep_start(double* A, int n, double* __restrict__ wt,
 // orthogonal rotation a = W_q k, b = W_p k, W' = W / (1 + a b), and one that is
 // right to 1e-7 leaves the pair 1e-7 of its product for the next sweep.  With
 // the squares and square root, two dot products and c, s rotation in FP64 a
-// round of 64 columns took 4.6 us and a 768-column eigenproblem's sweep 3.5 ms.
+// round of 64 columns took 4.6 us and a 768-column eigenproblem's sweep 3.5 ms;
+// all eigenproblems of a 128-vector solve on 48^3 (up to 768) 120 -> 84 ms, of a
+// 16-vector solve on 24^3 28.6 -> 22.5 ms.
 template <int E, int T>
 __global__ void __launch_bounds__(T) k_jacobi_pair(double* A, int n, int nn, int round,
                                                    double* __restrict__ wt,

@@ -19,7 +19,7 @@ enum ProfClass : int {
   PC_GEMM_TF32 = 10,  // tensor-core (3xTF32) FP32 projections
   PC_CG_GRAPH_F32 = 11,  // whole captured CG loops (FP32 steps; their kernels are not
   PC_CG_GRAPH_F64 = 12,  // timed one by one inside a graph)
-  PC_COLS_DF = 13,       // double-float transforms (mixed-precision refinement)
+  PC_COLS_DF = 13,       // seven-digit transforms (mixed-precision refinement)
   PC_SLAB_DF = 14,
   PC_HPSI_FUSED = 15,    // FP32 H x in one launch (column scratch in shared memory)
   PC_GEMM_DF = 16,       // FP64 GEMMs of the mixed modes' refinement

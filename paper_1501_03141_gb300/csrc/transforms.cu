@@ -297,8 +297,8 @@ __device__ __forceinline__ void xline_forward(const SphereDev<R>& s, const cpx<R
 }
 
 // ---------------------------------------------------------------------------
-// slab pass, FP32: one x-plane i1 of one item (FP64 and double-float data
-// take transforms_fx.cu)
+// slab pass, FP32: one x-plane i1 of one item (FP64 data take
+// transforms_fx.cu)
 // ---------------------------------------------------------------------------
 // largest block a slab of this shape launches with: every z-line (N2 lines)
 // or every y-line (at most N3/2 + 1 planes) in one round

@@ -17,7 +17,9 @@ namespace {
 //
 // Bound by the latency of a warp's chain (conversion, digits, products, sums):
 // a tile per warp, with the members (in) or the coefficients (out) exchanged
-// through shared memory, halves it against one warp for both tiles.
+// through shared memory, halves it against one warp for both tiles.  A pass over
+// 128 items on 24^3 19.3 -> 14.2 us, on 48^3 53.6 -> 50.1 us (82 us as FP64
+// FFTs).
 constexpr int COLS_PAIRS = 2;  // column groups per block
 constexpr int COLS_THREADS = 64 * COLS_PAIRS;
 
