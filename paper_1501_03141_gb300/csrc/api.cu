@@ -539,10 +539,9 @@ std::string shape_key(const char* what, const SysData& s) {
 // 3854 against 4145; 48^3, 64 items 6267 against 6961, 128 items 10032 against 7904.
 int few_items(int N) { return N <= 24 ? 0 : N <= 32 ? 38 : 76; }
 
-
 // R: FP32 or FP64.  refine (FP64): the product of a mixed-mode refinement, whose
-// transforms take seven digits (far below the FP32 inner solve's needs and
-// above double-float).
+// transforms take seven digits (errors below 2e-15 of the product, far below the
+// FP32 inner solve's needs).
 template <typename R>
 int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list, int n_list,
             bool with_shift, bool with_pv, cudaStream_t st, double* dn = nullptr,
@@ -651,7 +650,7 @@ int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list,
         return PDEP_OK;
       }
       int pv = c->opt.proj_variant >= 0 ? c->opt.proj_variant : c->proj_variant;
-      const bool tuning = c->opt.autotune && pv < 0 && m >= 256;
+      const bool tuning = c->opt.autotune && pv < 0 && m >= 256 && !capturing(st);
       if (pv < 0) pv = tuning ? c->proj_tune_next : 2;
       if (tuning) CK(cudaEventRecord(c->ev[0], st));
       if (pv == 1 || pv == 2) {
@@ -1177,8 +1176,9 @@ int cg_workspace(pdep_ctx* c, SysData& s, int n, R** r, R** p, R** ap, int** lis
 
 // Whether the CG step adds the projection itself: the states pass through L2
 // twice per RHS, which up to about 64 MB (some 8 us) costs less than the
-// coefficient and update launches (on 24^3 with 8 RHS 18 us against 3; on 64^3
-// with 84 RHS of 44 states 26 us against some 60).
+// coefficient and update launches (18 us on 24^3 with 8 RHS; together with the
+// step as a cluster and its loop control one application there fell from 2186 to
+// 1614 us, and on 64^3 with 84 RHS from 13.4 to 9.9 ms).
 template <typename R>
 bool few_projection(const pdep_ctx* c, const SysData& s, int n) {
   if (sizeof(R) == 4 && (c->opt.proj_variant >= 0 || s.d_psib16)) return false;
@@ -1485,7 +1485,7 @@ int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int ma
 // Refinement rounds (iterative refinement written in solution updates):
 // round k solves A delta = r for every RHS still above cg_tol, with an inner
 // CG in precision Ri on the residual scaled to unit norm, then x += delta
-// and r -= A delta with A delta in FP64 arithmetic (or double-float, mixed
+// and r -= A delta with A delta in FP64 arithmetic (or seven digits, mixed
 // modes) and the density response of delta accumulated by that same
 // transform (dn is linear in x).  The FP64 path runs its inner solve to
 // 0.9 cg_tol (round 0) or 0.5 cg_tol (later rounds) of ||b_i|| through

@@ -37,3 +37,22 @@ def test_rounds_graph_equals_host_loop(prec, kw, n):
         assert rel(b, a) < 1e-7 and rel(a2, a) < 1e-7 and rel(b2, b) < 1e-7
     else:  # stopped after the first round(s): one FP32 solve's accuracy
         assert sb["max_cg_residual"] > 1e-10 and rel(b, a) < 1e-2
+
+
+# PDEP_MIXED_BF16 never times the FP32 projection kernels in its CG loops, so its
+# refinement rounds are captured while those are untimed; accurate to the same
+# residual as above
+def test_rounds_graph_bf16_untimed():
+    need_gpu()
+    lib_ready()
+    import paper_1501_03141_gb300 as pg
+    s = synthetic.make_system("tiny")
+    got = []
+    for use_graph in (0, 1):
+        with pg.Context(s, precision=pg.PDEP_MIXED_BF16, use_graph=use_graph) as ctx:
+            phi = np.random.default_rng(6).standard_normal((160, ctx.sizes()["n_pdep_dim"]))
+            for _ in range(3):
+                w = ctx.chi0_apply(phi)
+            got.append(w)
+            assert ctx.stats()["max_cg_residual"] <= 1e-10
+    assert rel(got[1], got[0]) < 1e-7
