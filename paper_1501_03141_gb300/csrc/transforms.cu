@@ -589,7 +589,7 @@ __global__ void __launch_bounds__(SlabThreads<N2, N3>::v, (SlabMinBlocks<N2, N3>
 // planes as its lanes cover z-lines (4, 3, 2, 2 planes of 24, 32, 40, 48 lines);
 // the groups share nothing but B1 and synchronise by named barriers.  168
 // registers (96 hold a line of 48) leave 12 warps.  Measured against four lanes
-// per line: 245 thousand instructions per item; 56 launches of up to 4096 items on
+// per line: 264 thousand instructions per item; 56 launches of up to 4096 items on
 // 48^3 87.0 -> 55.6 ms (68.1 ms with a group's planes beside the whole column
 // scratch, three groups; 74.3 ms with the three steps' code apart), 37 launches
 // on 32^3 3.22 -> 2.24 ms.  Error of H x against FP64 5.4e-8 -> 5.1e-8 on 48^3.
