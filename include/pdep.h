@@ -414,6 +414,11 @@ int pdep_sync_status(pdep_ctx* ctx, void* stream);
  * last pdep_solve. */
 int pdep_get_stats(pdep_ctx* ctx, pdep_stats* stats, void* stream);
 
+/* CG-loop and refinement graphs captured on this context since pdep_setup (host
+ * work of the first call of a shape; calls like an earlier one capture none,
+ * whatever arrays they are given).  0 for a null context. */
+int pdep_graph_captures(const pdep_ctx* ctx);
+
 /* 1 if this library was compiled with -DPDEP_BOUNDS_CHECK (every index read
  * from the host-built sphere tables is tested before use in the transform
  * kernels), else 0. */

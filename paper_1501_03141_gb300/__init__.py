@@ -159,6 +159,10 @@ class Context:
         _abi.check(r, "pdep_get_stats", (_abi.PDEP_OK, _abi.PDEP_ERR_NOT_CONVERGED))
         return {k: getattr(st, k) for k, _ in _abi.pdep_stats._fields_}
 
+    def graph_captures(self):
+        """CG-loop and refinement graphs captured on this context so far."""
+        return self._lib.pdep_graph_captures(self._h)
+
     def _finish(self, status, where, allow, bufs, sync):
         """With device buffers only the library call just enqueued the work:
         unless sync is False, wait and read the device status word here."""

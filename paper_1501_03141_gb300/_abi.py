@@ -44,6 +44,7 @@ EXPORTS = (
     "pdep_profile", "pdep_destroy", "pdep_status_string", "pdep_last_error",
     "pdep_apply_hamiltonian_noalloc", "pdep_screening_apply", "pdep_lanczos", "pdep_chi0_imag",
     "pdep_chibar_apply", "pdep_sync_status", "pdep_bounds_checked", "pdep_get_stats",
+    "pdep_graph_captures",
 )
 
 PDEP_PROFILE_CLASSES = 17
@@ -167,10 +168,12 @@ def load(path: str = LIB_PATH):
     lib.pdep_sync_status.argtypes = [vp, vp]
     lib.pdep_get_stats.argtypes = [vp, ctypes.POINTER(pdep_stats), vp]
     lib.pdep_bounds_checked.argtypes = []
+    lib.pdep_graph_captures.argtypes = [vp]
     for name in ("pdep_setup", "pdep_get_sizes", "pdep_get_occupied", "chi0_apply",
                  "sternheimer_solve", "pdep_solve", "pdep_apply_hamiltonian", "pdep_to_grid",
                  "pdep_screening_apply", "pdep_lanczos", "pdep_chi0_imag",
-                 "pdep_chibar_apply", "pdep_sync_status", "pdep_bounds_checked", "pdep_get_stats"):
+                 "pdep_chibar_apply", "pdep_sync_status", "pdep_bounds_checked", "pdep_get_stats",
+                 "pdep_graph_captures"):
         getattr(lib, name).restype = ip
     del dp
     _lib = lib

@@ -137,7 +137,8 @@ struct CgGraph {
 struct RoundsGraph {
   int prec, sys, n, cg_variant, proj_variant, tune_gen;
   int check, round, body;  // kernels before the first round, per round, per CG step
-  const void *b, *x, *dn, *its, *rel, *r64, *ad;
+  bool dn;               // with the density response (its array: pdep_ctx::d_dn)
+  const void *b, *x, *its, *rel, *r64, *ad;
   unsigned long long ws_gen, budget_ns;
   cudaGraphExec_t exec;
 };
@@ -155,6 +156,7 @@ struct pdep_ctx {
   CgLoopState* d_loop = nullptr;
   DevStats* d_dstats = nullptr;
   int* d_refine = nullptr;        // [0]: unconverged count of the current refinement round
+  double** d_dn = nullptr;        // the density response being accumulated (SlabArgs::dn)
   cudaStream_t cap_stream = nullptr;  // private stream the CG graphs are captured on
   unsigned long long ws_gen = 0;  // bumped whenever a workspace buffer is reallocated
   unsigned long long budget_ns = 0;   // clock_budget_cycles in ns of %globaltimer
@@ -163,6 +165,7 @@ struct pdep_ctx {
   int round_launches = 0;             // kernels per round of the last rounds graph
   int body_launches[2] = {0, 0};      // kernels per CG step of the last graph (FP32, FP64)
   long long graph_launches = 0;       // CG graphs launched
+  int graph_captures = 0;             // CG and refinement graphs captured since pdep_setup
   long long prologue_launches = 0;    // kernels before their loops
   long long eager_steps[2] = {0, 0};  // CG steps launched from the host loop (FP32, FP64)
   long long st_launch0 = 0;           // launch counter at the last statistics reset
@@ -476,9 +479,10 @@ size_t b1_count(const SysData& s, int n_items) {
 // uses occupied state i % n_occ; without with_shift Y = H X.  Then, if
 // with_pv, the occupied and deflated states are shifted:
 // Y += Psi_ext diag(sigma) (Psi_ext^T X) on the same columns.
-// dn (FP64 only, may be null): the transform also accumulates the density
-// response dn_j(r) += (4/Omega) u_v(r) x_i(r) of every vector i = j n_occ + v
-// it transforms (Eq. deltani); dn must hold the (i / n_occ) perturbations.
+// dn (may be null): the transform also accumulates the density response
+// dn_j(r) += (4/Omega) u_v(r) x_i(r) of every vector i = j n_occ + v it
+// transforms (Eq. deltani) to the array whose address the device word *dn
+// holds; it must hold the (i / n_occ) perturbations.
 bool capturing(cudaStream_t st) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
@@ -544,7 +548,7 @@ int few_items(int N) { return N <= 24 ? 0 : N <= 32 ? 38 : 76; }
 // FP32 inner solve's needs).
 template <typename R>
 int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list, int n_list,
-            bool with_shift, bool with_pv, cudaStream_t st, double* dn = nullptr,
+            bool with_shift, bool with_pv, cudaStream_t st, double* const* dn = nullptr,
             const int* d_count = nullptr, bool refine = false, long long ldx = 0,
             long long ldy = 0) {
   const int digits = refine ? 7 : 8;
@@ -1315,6 +1319,7 @@ int build_graph(pdep_ctx* c, cudaGraphExec_t* out, F fn) {
     }
   }
   cudaGraphDestroy(g);
+  if (status == PDEP_OK) ++c->graph_captures;
   return status;
 }
 
@@ -1507,7 +1512,7 @@ inline double inner_tol_of(const pdep_ctx* c) {
 
 template <typename Ri>
 int refine_rounds(pdep_ctx* c, SysData& s, const double* b, const double* xd, double* x, int n,
-                  double* dn, int* its_total, double* rel, double* r64, double* ad,
+                  double* const* dn, int* its_total, double* rel, double* r64, double* ad,
                   cudaStream_t st) {
   const bool fp64 = sizeof(Ri) == 8;
   const double tol = c->opt.cg_tol;
@@ -1581,14 +1586,14 @@ int refine_rounds(pdep_ctx* c, SysData& s, const double* b, const double* xd, do
       }
       RoundsGraph* g = nullptr;
       for (RoundsGraph& e : c->rounds_graphs)
-        if (e.prec == pi && e.sys == si && e.n == n && e.b == b && e.x == x && e.dn == dn &&
-            e.its == its_total && e.rel == rel && e.r64 == r64 && e.ad == ad &&
+        if (e.prec == pi && e.sys == si && e.n == n && e.b == b && e.x == x &&
+            e.dn == (dn != nullptr) && e.its == its_total && e.rel == rel && e.r64 == r64 && e.ad == ad &&
             e.ws_gen == c->ws_gen && e.budget_ns == c->budget_ns && e.cg_variant == variant &&
             e.proj_variant == pv && e.tune_gen == c->tune_gen)
           g = &e;
       if (!g) {
-        RoundsGraph e{pi, si, n, variant, pv, c->tune_gen, 0, 0, 0, b, x, dn, its_total, rel,
-                      r64, ad, c->ws_gen, c->budget_ns, nullptr};
+        RoundsGraph e{pi, si, n, variant, pv, c->tune_gen, 0, 0, 0, dn != nullptr, b, x, its_total,
+                      rel, r64, ad, c->ws_gen, c->budget_ns, nullptr};
         RET(build_graph(c, &e.exec, [&](cudaGraph_t top) -> int {
           cudaGraphConditionalHandle h = 0;
           CK(cudaGraphConditionalHandleCreate(&h, top, 0, 0));
@@ -1662,11 +1667,16 @@ int solve_rhs(pdep_ctx* c, SysData& s, const double* b, const double* xd, double
   // r64 = b: the FP64 residual, updated as r -= A delta for every update
   // delta of x (and checked against b's norm)
   CK(cudaMemcpyAsync(r64, b, sizeof(double) * (size_t)n * s.ld, cudaMemcpyDeviceToDevice, st));
-  if (dn) CK(cudaMemsetAsync(dn, 0, sizeof(double) * (size_t)(n / s.n_occ) * s.n_r, st));
+  // The kernels find the density's array, the caller's own for chi0_apply on the
+  // device, through a device word, so that it is no part of a captured graph: a
+  // new array with every call, or one per chunk of perturbations, would be a
+  // capture each.
+  if (dn) CK(density_start(dn, (size_t)(n / s.n_occ) * s.n_r, c->d_dn, st));
+  double* const* slot = dn ? c->d_dn : nullptr;
   if (c->opt.precision == PDEP_FP64)
-    RET(refine_rounds<double>(c, s, b, xd, x, n, dn, its_total, rel, r64, ad, st));
+    RET(refine_rounds<double>(c, s, b, xd, x, n, slot, its_total, rel, r64, ad, st));
   else
-    RET(refine_rounds<float>(c, s, b, xd, x, n, dn, its_total, rel, r64, ad, st));
+    RET(refine_rounds<float>(c, s, b, xd, x, n, slot, its_total, rel, r64, ad, st));
   // rel holds the FP64 residual of every RHS from its last update.  No final
   // P_c projection is needed: the shifted operator lifts occupied state w to
   // eps_{n_ext} - eps_v > 0, so the occupied component of x is at most
@@ -2014,6 +2024,8 @@ int pdep_sync_status(pdep_ctx* c, void* stream) {
   return r;
 }
 
+int pdep_graph_captures(const pdep_ctx* c) { return c ? c->graph_captures : 0; }
+
 int pdep_bounds_checked(void) {
 #ifdef PDEP_BOUNDS_CHECK
   return 1;
@@ -2037,6 +2049,7 @@ void pdep_destroy(pdep_ctx* c) {
   if (c->d_loop) cudaFree(c->d_loop);
   if (c->d_dstats) cudaFree(c->d_dstats);
   if (c->d_refine) cudaFree(c->d_refine);
+  if (c->d_dn) cudaFree(c->d_dn);
   for (auto& kv : c->bufs)
     if (kv.second.p) cudaFree(kv.second.p);
   for (void* p : c->owned) cudaFree(p);
@@ -2080,6 +2093,7 @@ int pdep_setup(const pdep_system_desc* sys, int n_sys, const pdep_options* opt, 
       cudaMalloc(&c->d_loop, sizeof(CgLoopState)) != cudaSuccess ||
       cudaMalloc(&c->d_dstats, sizeof(DevStats)) != cudaSuccess ||
       cudaMalloc(&c->d_refine, 4 * sizeof(int)) != cudaSuccess ||
+      cudaMalloc(&c->d_dn, sizeof(double*)) != cudaSuccess ||
       cudaMallocHost(&c->h_pin, 16 * sizeof(int)) != cudaSuccess)
     return bail(fail(PDEP_ERR_OOM, "context allocation"));
   cudaMemset(c->d_status, 0, sizeof(unsigned));

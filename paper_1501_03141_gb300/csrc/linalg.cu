@@ -1187,9 +1187,16 @@ cudaError_t block_cg_p(double* p, const double* r, long long ld, int rows, int n
   return cudaGetLastError();
 }
 
-cudaError_t fill_zero(void* p, size_t bytes, cudaStream_t st) {
-  if (bytes == 0) return cudaSuccess;
-  return cudaMemsetAsync(p, 0, bytes, st);
+__global__ void k_density_start(double* dn, long long count, double** slot) {
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (t == 0) *slot = dn;
+  for (long long i = t; i < count; i += (long long)gridDim.x * blockDim.x) dn[i] = 0.0;
+}
+cudaError_t density_start(double* dn, size_t count, double** slot, cudaStream_t st) {
+  const int blocks = (int)std::min<size_t>((count + 1023) / 1024, 8 * (size_t)num_sms());
+  count_launch();
+  k_density_start<<<std::max(blocks, 1), 256, 0, st>>>(dn, (long long)count, slot);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------

@@ -126,7 +126,8 @@ cudaError_t cholesky_winv(const double* G, int m, double rel_thr, double* W, int
                           cudaStream_t st);
 cudaError_t scale_by_isqrt_clamped(double* Q, long long ldq, int n, const double* d, double dmin,
                                    int* keep, cudaStream_t st);
-cudaError_t fill_zero(void* p, size_t bytes, cudaStream_t st);
+// dn [count] = 0, and its address into the device word *slot (SlabArgs::dn)
+cudaError_t density_start(double* dn, size_t count, double** slot, cudaStream_t st);
 
 // Tensor-core (3xTF32, mma.sync) FP32 projections, all matrices column-major:
 // S (M x N, lds) = diag(sigma) P^T X(:, bmap)      (K = rows of P and X)

@@ -486,7 +486,7 @@ __device__ __forceinline__ void slab_unit(const SphereDev<float>& s, const SlabA
           if (same)
             acc[i] = fma(xb, ub[i3], acc[i]);
           else if (ib >= 0)
-            atomicAdd(a.dn + (long long)jb * a.dn_stride + off + i3, a.dn_scale * (xb * ub[i3]));
+            atomicAdd(*a.dn + (long long)jb * a.dn_stride + off + i3, a.dn_scale * (xb * ub[i3]));
         }
       }
       // SLAB_HPSI: multiply by the local potential on the grid
@@ -546,7 +546,7 @@ __global__ void __launch_bounds__(SlabThreads<N2, N3>::v, (SlabMinBlocks<N2, N3>
       const int g0 = w / s.N1 * group, i1 = w % s.N1;
       auto flush = [&](int j) {
         if (i2 >= N2) return;
-        double* dn = a.dn + (long long)j * a.dn_stride + ((long long)i1 * N2 + i2) * N3;
+        double* dn = *a.dn + (long long)j * a.dn_stride + ((long long)i1 * N2 + i2) * N3;
 #pragma unroll
         for (int i = 0; i < M3; ++i) {
           atomicAdd(dn + pos_b<N3, TL3>(t3, i), a.dn_scale * acc[i]);

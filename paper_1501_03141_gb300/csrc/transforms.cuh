@@ -161,8 +161,10 @@ struct SlabArgs {
   GridSrc<R> src;        // FROM_GRID (f: one grid per group, g: per-vector grids)
   ItemMap map;
   // HPSI: also accumulate dn_j(r) += dn_scale u_v(r) x_vj(r) for
-  // every vector i = j * dn_nocc + v of the item (atomically; dn may be null)
-  double* dn = nullptr;
+  // every vector i = j * dn_nocc + v of the item (atomically; dn may be null).
+  // *dn, in device memory, is the array's address: a graph captured with it
+  // serves whatever array the caller of a later solve brings
+  double* const* dn = nullptr;
   const double* u = nullptr;  // occupied grids [dn_nocc][dn_stride]
   int dn_nocc = 1;
   long long dn_stride = 0;

@@ -151,8 +151,9 @@ __device__ __forceinline__ void z_chunk(const SphereDev<double>& s, const SlabAr
       const int ja = ia / a.dn_nocc, jb = ib >= 0 ? ib / a.dn_nocc : -1;
       const double* ua = a.u + (long long)(ia - ja * a.dn_nocc) * a.dn_stride + line;
       const double* ub = ib >= 0 ? a.u + (long long)(ib - jb * a.dn_nocc) * a.dn_stride + line : ua;
-      double* da = a.dn + (long long)ja * a.dn_stride + line;
-      double* db = ib >= 0 ? a.dn + (long long)jb * a.dn_stride + line : da;
+      double* const dn = *a.dn;
+      double* da = dn + (long long)ja * a.dn_stride + line;
+      double* db = ib >= 0 ? dn + (long long)jb * a.dn_stride + line : da;
       const double sc = a.dn_scale * fx_unit(e3);
       const bool same = jb == ja;
 #pragma unroll
@@ -219,8 +220,8 @@ __device__ void slab_nan(const SphereDev<double>& s, const SlabArgs<double>& a, 
       if (ia >= 0) a.out[(long long)ia * a.out_stride + plane + p] = nan;
       if (ib >= 0) a.out[(long long)ib * a.out_stride + plane + p] = nan;
     } else if (a.mode == SLAB_HPSI && a.dn) {
-      atomicAdd(a.dn + (long long)(ia / a.dn_nocc) * a.dn_stride + plane + p, nan);
-      if (ib >= 0) atomicAdd(a.dn + (long long)(ib / a.dn_nocc) * a.dn_stride + plane + p, nan);
+      atomicAdd(*a.dn + (long long)(ia / a.dn_nocc) * a.dn_stride + plane + p, nan);
+      if (ib >= 0) atomicAdd(*a.dn + (long long)(ib / a.dn_nocc) * a.dn_stride + plane + p, nan);
     }
   }
   if (a.mode == SLAB_TO_GRID) return;
