@@ -7,7 +7,6 @@
 #include <cmath>
 #include <cstring>
 #include <functional>
-#include <initializer_list>
 #include <map>
 #include <string>
 #include <type_traits>
@@ -16,6 +15,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "common.cuh"
+#include "direct_io.cuh"
 #include "linalg.cuh"
 #include "profile.cuh"
 #include "transforms.cuh"
@@ -255,22 +255,15 @@ cudaMemcpyKind kind_from_dev(const void* dst) {
   return is_device_ptr(dst) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
 }
 
-// Whether a call can work on the caller's arrays in place of staged copies: all
-// on the device, aligned for FP64 loads, and the written one apart from the read
-// ones (vectors that overlap were always accepted, through the copies).
-struct Span {
-  const void* p;
-  size_t bytes;
-};
-bool direct_io(const Span& out, std::initializer_list<Span> in) {
-  const char* o = (const char*)out.p;
-  if (!is_device_ptr(out.p) || ((uintptr_t)o & 7)) return false;
-  for (const Span& x : in) {
-    const char* q = (const char*)x.p;
-    if (!is_device_ptr(q) || ((uintptr_t)q & 7)) return false;
-    if (q < o + out.bytes && o < q + x.bytes) return false;
+// an array of the caller's for direct_io
+Span span(const void* p, size_t bytes) {
+  cudaPointerAttributes at;
+  if (!p || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return {p, bytes, false, false, -1};
   }
-  return true;
+  const bool managed = at.type == cudaMemoryTypeManaged;
+  return {p, bytes, managed || at.type == cudaMemoryTypeDevice, managed, at.device};
 }
 
 // host source -> host or device destination
@@ -2258,7 +2251,7 @@ int pdep_screening_apply(pdep_ctx* c, int sys, int kind, const double* eigvals,
     g[i] = lam[i] / (1.0 - lam[i]);
   }
   const size_t vb = sizeof(double) * (size_t)dim;
-  const bool direct = direct_io({out, vb * n}, {{f, vb * n}, {eigvecs, vb * n_pdep}});
+  const bool direct = direct_io(c->device, span(out, vb * n), {span(f, vb * n), span(eigvecs, vb * n_pdep)});
   double *S, *dg;
   RET(ws(c, "sc_s", (size_t)n_pdep * n, &S));
   RET(ws(c, "sc_g", (size_t)n_pdep, &dg));
@@ -2609,7 +2602,7 @@ int pdep_apply_hamiltonian(pdep_ctx* c, int sys, const double* x, int n, double*
   cudaStream_t st = (cudaStream_t)stream;
   SysData& s = c->sys[sys];
   const size_t bytes = sizeof(double) * (size_t)n * s.n_pw;
-  const bool direct = direct_io({y, bytes}, {{x, bytes}});
+  const bool direct = direct_io(c->device, span(y, bytes), {span(x, bytes)});
   // rows n_pw apart in the caller's arrays, s.ld apart in staged ones
   const double* in = x;
   double* outv = y;
@@ -2647,8 +2640,8 @@ int pdep_to_grid(pdep_ctx* c, int sys, const double* x, int n, double* u, void* 
   if (n == 0) return PDEP_OK;
   cudaStream_t st = (cudaStream_t)stream;
   SysData& s = c->sys[sys];
-  const bool direct = direct_io({u, sizeof(double) * (size_t)n * s.n_r},
-                                {{x, sizeof(double) * (size_t)n * s.n_pw}});
+  const bool direct = direct_io(c->device, span(u, sizeof(double) * (size_t)n * s.n_r),
+                                {span(x, sizeof(double) * (size_t)n * s.n_pw)});
   const double* in = x;
   double* grid = u;
   long long ld = s.n_pw;
