@@ -18,7 +18,6 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
-#include <atomic>
 
 #include "linalg.cuh"
 #include "profile.cuh"
@@ -517,13 +516,8 @@ __global__ void __launch_bounds__(T)
 template <typename R, int T>
 cudaError_t launch_stream(const CgArgs<R>& a, const int* list, int nb, int rowb, cudaStream_t st) {
   auto kern = k_cg_stream<R, T>;
-  static std::atomic<bool> attr_set{false};
-  if (!attr_set.load()) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)CG_STREAM_SMEM);
-    if (e != cudaSuccess) return e;
-    attr_set.store(true);
-  }
+  static OncePerDevice limit;  // per instantiation
+  if (const cudaError_t e = raise_smem_limit(limit, kern, (int)CG_STREAM_SMEM)) return e;
   const size_t smem = 8 * (size_t)rowb;
   static const int sms = [] {
     int dev = 0, n = 0;

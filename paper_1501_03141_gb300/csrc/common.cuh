@@ -8,6 +8,7 @@
 #include <algorithm>
 
 #include "../../include/pdep.h"
+#include "per_device.cuh"
 
 namespace pdep {
 
@@ -47,6 +48,18 @@ __device__ __forceinline__ cpx<R> shfl_xor(cpx<R> a, int m) {
 template <typename R>
 __device__ __forceinline__ cpx<R> shfl_idx(cpx<R> a, int lane) {
   return mk(__shfl_sync(0xffffffffu, a.x, lane), __shfl_sync(0xffffffffu, a.y, lane));
+}
+
+// Raises the dynamic shared memory a kernel may be launched with on the current
+// device, once per device.
+template <typename K>
+cudaError_t raise_smem_limit(OncePerDevice& once, K kern, int bytes) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  return once(dev, [&] {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  });
 }
 
 // Device-side status word bits (OR-ed by kernels, read by the host after a sync).

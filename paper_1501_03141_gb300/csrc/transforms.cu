@@ -1,5 +1,4 @@
 // Plane-wave sphere <-> grid transforms (see transforms.cuh for the scheme).
-#include <atomic>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -971,12 +970,8 @@ static cudaError_t slab_impl_dn(const SphereDev<float>& s, const SlabArgs<float>
   if (nt > SlabThreads<N2, N3>::v) return cudaErrorInvalidConfiguration;
   const size_t smem = slab_smem_bytes(s.n_col, s.R3, N2, sizeof(float));
   auto kern = k_slab<N2, N3, DN>;
-  static std::atomic<bool> attr_set{false};  // per instantiation; raised once
-  if (!attr_set.load()) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e != cudaSuccess) return e;
-    attr_set.store(true);
-  }
+  static OncePerDevice limit;  // per instantiation
+  if (const cudaError_t e = raise_smem_limit(limit, kern, 200 * 1024)) return e;
   const int gx = a.n_items;
   if (gx == 0) return cudaSuccess;
   const long long resident = (long long)occupancy(kern, nt, smem) * sm_count();
@@ -1086,13 +1081,8 @@ static cudaError_t hpsi_fused_impl(const SphereDev<float>& s, const float* x, lo
                                    const Epilogue<float>& ep, size_t smem, int G,
                                    cudaStream_t st) {
   auto kern = k_hpsi_fused<N>;
-  static std::atomic<bool> attr_set{false};
-  if (!attr_set.load()) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         226 * 1024);
-    if (e != cudaSuccess) return e;
-    attr_set.store(true);
-  }
+  static OncePerDevice limit;  // per instantiation
+  if (const cudaError_t e = raise_smem_limit(limit, kern, 226 * 1024)) return e;
   const int threads = G / Fused<N>::PLANES * FG_THREADS;
   const unsigned grid = (unsigned)std::min<long long>(
       n_items, (long long)occupancy(kern, threads, smem) * sm_count());

@@ -7,7 +7,6 @@
 // refinement's passes (seven digits, before in double-float) over 4096 items,
 // there and back with the density and from the grid, 35.9 -> 25.3 ms.
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <vector>
 
@@ -477,12 +476,8 @@ cudaError_t slab_fx_mode(const SphereDev<double>& s, const SlabArgs<double>& a, 
   if (a.n_items <= 0) return cudaSuccess;
   const size_t smem = slab_smem_bytes(s.n_col, s.R3, N2, 8);
   auto kern = k_slab_fx<MODE, S, N2, N3>;
-  static std::atomic<bool> attr_set{false};  // per instantiation; raised once
-  if (!attr_set.load()) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e != cudaSuccess) return e;
-    attr_set.store(true);
-  }
+  static OncePerDevice limit;  // per instantiation
+  if (const cudaError_t e = raise_smem_limit(limit, kern, 200 * 1024)) return e;
   double fl = 0, by = 0;
   slab_work(s, a, fl, by);
   ProfScope ps(S < FX_S ? PC_SLAB_DF : PC_SLAB_F64, st, fl, by,

@@ -1,7 +1,6 @@
 // The FP64 column passes on the tensor cores (fx_line.cuh): x-lines between the
 // sphere and the column scratch.
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <vector>
 
