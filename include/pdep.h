@@ -91,7 +91,13 @@ typedef enum {
 } pdep_status;
 
 typedef enum {
-  PDEP_FP64 = 0,       /* every step in FP64 */
+  PDEP_FP64 = 0,       /* every step in FP64.  Transforms and matrix products are sums
+                          of exact digit products whose error, below that of FP64
+                          multiply-adds, is relative to the largest entries that meet
+                          (of a plane of the transform, of a row and a column of a
+                          product), not to each result; pdep_screening_apply keeps
+                          the component-wise accuracy of multiply-adds for whatever
+                          vectors it is given */
   PDEP_MIXED_TF32 = 1, /* FP32 FFTs, H*psi and vector updates inside the
                           Sternheimer CG, its projection term on the tensor
                           cores (TF32 operands split in three for FP32

@@ -2279,14 +2279,16 @@ int pdep_screening_apply(pdep_ctx* c, int sys, int kind, const double* eigvals,
   }
   // S = Phi^T f, scaled per row by lambda/(1-lambda); out = Phi S (+ f)
   const long long ldf = kind == PDEP_SCREEN_WP ? s.ld : ld;
-  CK(gemm<double>(true, n_pdep, n, dim, 1.0, phi, ld, fx, ldf, 0.0, S, n_pdep, st));
+  CK(gemm<double>(true, n_pdep, n, dim, 1.0, phi, ld, fx, ldf, 0.0, S, n_pdep, st, nullptr, nullptr,
+                  nullptr, 0, false, true));
   CK(scale_rows<double>(S, n_pdep, n_pdep, n, dg, st));
   double beta = 0.0;
   if (kind == PDEP_SCREEN_EPSINV) {
     CK(cudaMemcpyAsync(o, fx, sizeof(double) * (size_t)n * ld, cudaMemcpyDeviceToDevice, st));
     beta = 1.0;
   }
-  CK(gemm<double>(false, dim, n, n_pdep, 1.0, phi, ld, S, n_pdep, beta, o, ld, st));
+  CK(gemm<double>(false, dim, n, n_pdep, 1.0, phi, ld, S, n_pdep, beta, o, ld, st, nullptr, nullptr,
+                  nullptr, 0, false, true));
   if (kind == PDEP_SCREEN_WP) CK(scale_sqrt_coulomb(o, ld, o, ld, s.n_half, n, s.sd.g2, st));
   if (!direct)
     CK(cudaMemcpy2DAsync(out, vb, o, s.ld * sizeof(double), vb, n, kind_from_dev(out), st));

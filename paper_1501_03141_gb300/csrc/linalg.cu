@@ -186,11 +186,11 @@ template <typename R>
 cudaError_t gemm(bool transA, int m, int n, int k, double alpha, const R* A,
                  long long lda, const R* B, long long ldb, double beta,
                  R* C, long long ldc, cudaStream_t st, const int* bmap,
-                 const int* cmap, const int* ndev, int split_x8, bool mixed) {
+                 const int* cmap, const int* ndev, int split_x8, bool mixed, bool graded) {
   if (m <= 0 || n <= 0) return cudaSuccess;
   if constexpr (sizeof(R) == 8) {
     return gemm_fx(transA, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, num_sms(), st, bmap, cmap,
-                   ndev, split_x8, mixed);
+                   ndev, split_x8, mixed, graded);
   } else {
     // 80-row tiles when they pad m less than 64-row tiles do
     const bool t80 = ((m + 79) / 80) * 80 < ((m + 63) / 64) * 64;
@@ -234,10 +234,10 @@ cudaError_t gemm(bool transA, int m, int n, int k, double alpha, const R* A,
 
 template cudaError_t gemm<double>(bool, int, int, int, double, const double*, long long,
                                   const double*, long long, double, double*, long long,
-                                  cudaStream_t, const int*, const int*, const int*, int, bool);
+                                  cudaStream_t, const int*, const int*, const int*, int, bool, bool);
 template cudaError_t gemm<float>(bool, int, int, int, double, const float*, long long, const float*,
                                  long long, double, float*, long long, cudaStream_t, const int*,
-                                 const int*, const int*, int, bool);
+                                 const int*, const int*, int, bool, bool);
 
 // ---------------------------------------------------------------------------
 // one-sided Jacobi eigensolver

@@ -18,17 +18,20 @@ namespace pdep {
 // double by exact integer products on the FP16 tensor cores (fx_gemm.cu).
 // split_x8 (FP64; optional): split-K multiplier of the default split
 // (split_x8 / 8, 0 = default); the autotuner picks it per GEMM shape.  mixed:
-// profiled with the mixed modes' refinement.
+// profiled with the mixed modes' refinement.  FP64 results are accurate relative
+// to the largest magnitudes of the row of op(A) and the column of B; graded
+// (FP64): relative to the sum of the magnitudes of the products, as a chain of
+// multiply-adds is, for operands whose entries the caller chose.
 template <typename R>
 cudaError_t gemm(bool transA, int m, int n, int k, double alpha, const R* A,
                  long long lda, const R* B, long long ldb, double beta,
                  R* C, long long ldc, cudaStream_t st, const int* bmap = nullptr,
                  const int* cmap = nullptr, const int* ndev = nullptr, int split_x8 = 0,
-                 bool mixed = false);
+                 bool mixed = false, bool graded = false);
 cudaError_t gemm_fx(bool transA, int m, int n, int k, double alpha, const double* A, long long lda,
                     const double* B, long long ldb, double beta, double* C, long long ldc, int sms,
                     cudaStream_t st, const int* bmap, const int* cmap, const int* ndev,
-                    int split_x8, bool mixed);
+                    int split_x8, bool mixed, bool graded);
 
 // Symmetric eigendecomposition of the n x n matrix M (lda), FP64:
 // one-sided (Hestenes) Jacobi on M - sigma I (sigma = twice the Gershgorin
