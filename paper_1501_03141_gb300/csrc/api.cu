@@ -647,7 +647,8 @@ int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list,
         return PDEP_OK;
       }
       int pv = c->opt.proj_variant >= 0 ? c->opt.proj_variant : c->proj_variant;
-      const bool tuning = c->opt.autotune && pv < 0 && m >= 256 && !capturing(st);
+      // (a device count: how many columns the launch works on is not known here)
+      const bool tuning = c->opt.autotune && pv < 0 && m >= 256 && !d_count && !capturing(st);
       if (pv < 0) pv = tuning ? c->proj_tune_next : 2;
       if (tuning) CK(cudaEventRecord(c->ev[0], st));
       if (pv == 1 || pv == 2) {
@@ -1132,16 +1133,34 @@ int setup_states(pdep_ctx* c, SysData& s, cudaStream_t st) {
 // on that subspace: H commutes with the projector, so x has no component
 // along any w; the deflated states' share is added exactly, see split_rhs)
 // ---------------------------------------------------------------------------
+// Whether the CG step adds the projection itself: the states pass through L2
+// twice per RHS, which up to about 64 MB (some 8 us) costs less than the
+// coefficient and update launches (18 us on 24^3 with 8 RHS; together with the
+// step as a cluster and its loop control one application there fell from 2186 to
+// 1614 us, and on 64^3 with 84 RHS from 13.4 to 9.9 ms).
+template <typename R>
+bool few_projection(const pdep_ctx* c, const SysData& s, int n) {
+  if (sizeof(R) == 4 && (c->opt.proj_variant >= 0 || s.d_psib16)) return false;
+  return cg_proj_fits(s.n_pw, (int)sizeof(R), s.n_ext) &&
+         2.0 * n * s.n_ext * s.n_pw * sizeof(R) <= 64e6;
+}
+// (only up to CG_TAIL_MAX RHS does the step take it)
+bool step_projects(const pdep_ctx* c, const SysData& s, int pi, int n) {
+  return n <= CG_TAIL_MAX && (pi == 1 ? few_projection<double>(c, s, n) : few_projection<float>(c, s, n));
+}
+
 // The CG step's launch shape and the FP32 projection kernel are fixed once
 // the autotuner has timed them (or autotuning is off); only then is the loop
-// captured in a graph.
+// captured in a graph.  A step that adds the projection itself uses neither of
+// the two, and its loop never times them.
 bool tuned(const pdep_ctx* c, const SysData& s, int pi, int n) {
   if (!c->opt.autotune) return true;
-  const bool pv_ok = pi == 1 || c->opt.proj_variant >= 0 || c->proj_variant >= 0 ||
+  const bool fuse = step_projects(c, s, pi, n);
+  const bool pv_ok = pi == 1 || fuse || c->opt.proj_variant >= 0 || c->proj_variant >= 0 ||
                      c->opt.precision == PDEP_MIXED_BF16;
   const bool fused_ok = pi == 1 || !c->opt.fused_hpsi || hpsi_fused_smem(s.sf) == 0 ||
                         tune_done(c, "fused_planes:" + std::to_string(s.N[0]));
-  const bool cg_ok = c->cg_variant[pi] >= 0 || cg_streams(n, s.n_pw, pi == 1 ? 8 : 4);
+  const bool cg_ok = fuse || c->cg_variant[pi] >= 0 || cg_streams(n, s.n_pw, pi == 1 ? 8 : 4);
   return cg_ok && pv_ok && fused_ok;
 }
 int cg_variant_of(const pdep_ctx* c, int pi) {
@@ -1169,18 +1188,6 @@ int cg_workspace(pdep_ctx* c, SysData& s, int n, R** r, R** p, R** ap, int** lis
     RET(ws(c, sizeof(R) == 8 ? "pv_64" : "pv_32", (size_t)s.n_ext * std::max(n, 1), &S));
   }
   return PDEP_OK;
-}
-
-// Whether the CG step adds the projection itself: the states pass through L2
-// twice per RHS, which up to about 64 MB (some 8 us) costs less than the
-// coefficient and update launches (18 us on 24^3 with 8 RHS; together with the
-// step as a cluster and its loop control one application there fell from 2186 to
-// 1614 us, and on 64^3 with 84 RHS from 13.4 to 9.9 ms).
-template <typename R>
-bool few_projection(const pdep_ctx* c, const SysData& s, int n) {
-  if (sizeof(R) == 4 && (c->opt.proj_variant >= 0 || s.d_psib16)) return false;
-  return cg_proj_fits(s.n_pw, (int)sizeof(R), s.n_ext) &&
-         2.0 * n * s.n_ext * s.n_pw * sizeof(R) <= 64e6;
 }
 
 template <typename R>
@@ -1258,9 +1265,9 @@ template <typename R>
 int add_cg_loop(pdep_ctx* c, SysData& s, CgArgs<R> a, const R* b, int n, int max_iter, int* list,
                 cudaGraph_t g, cudaGraphNode_t after, cudaGraphNode_t* node, int* prologue,
                 int* per_step) {
-  const bool tail = n <= CG_TAIL_MAX, fuse = tail && few_projection<R>(c, s, n);
-  if (tail) a.variant = n < 256 ? (int)CG_FEW : a.variant;
   const int pi = sizeof(R) == 8 ? 1 : 0;
+  const bool tail = n <= CG_TAIL_MAX, fuse = step_projects(c, s, pi, n);
+  if (tail) a.variant = n < 256 ? (int)CG_FEW : a.variant;
   cudaGraphConditionalHandle h = 0;
   CK(cudaGraphConditionalHandleCreate(&h, g, 0, 0));
   cudaGraphNode_t pn = nullptr, bn = nullptr;
@@ -1386,7 +1393,7 @@ int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int ma
   const bool graph = c->opt.use_graph && (tuned(c, s, pi, n) || n < 256);
   if (!graph) {
     // eager: host loop, one 16-byte read of the loop state per step
-    const bool tail = n <= CG_TAIL_MAX, fuse = tail && few_projection<R>(c, s, n);
+    const bool tail = n <= CG_TAIL_MAX, fuse = step_projects(c, s, pi, n);
     const CgProj<R> pj = step_projection<R>(s);
     const CgTail tl = step_tail(c, list, max_iter, pi, 0, 0);
     CK(cudaMemsetAsync(&c->d_loop->active, 0, sizeof(int), st));
@@ -1408,7 +1415,7 @@ int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int ma
       // Autotuner: while untuned, each large step tries the next launch shape
       // (all shapes compute the same update) and its time per RHS is kept;
       // afterwards the fastest shape is used.
-      const bool tuning = c->opt.autotune && c->cg_variant[pi] < 0 && n_act >= 256 &&
+      const bool tuning = c->opt.autotune && c->cg_variant[pi] < 0 && n_act >= 256 && !fuse &&
                           !cg_streams(n, s.n_pw, sizeof(R));
       a.variant = tuning ? c->cg_tune_next[pi] : cg_variant_of(c, pi);
       if (tail && n < 256) a.variant = CG_FEW;
