@@ -519,6 +519,13 @@ bool tune_done(const pdep_ctx* c, const std::string& key) {
   return it != c->tunes.end() && it->second.best >= 0;
 }
 
+// The FP32 projection kernel in use: the option's, the timed choice, or before
+// that the default.  Graphs are keyed by it.
+int proj_kernel(const pdep_ctx* c) {
+  if (c->opt.proj_variant >= 0) return c->opt.proj_variant;
+  return c->proj_variant >= 0 ? c->proj_variant : 2;
+}
+
 // split-K candidates of the FP64 projection GEMMs, in eighths of the default
 const int kGemmSplits[4] = {8, 4, 16, 32};
 std::string shape_key(const char* what, const SysData& s) {
@@ -646,10 +653,10 @@ int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list,
                           d_count));
         return PDEP_OK;
       }
-      int pv = c->opt.proj_variant >= 0 ? c->opt.proj_variant : c->proj_variant;
       // (a device count: how many columns the launch works on is not known here)
-      const bool tuning = c->opt.autotune && pv < 0 && m >= 256 && !d_count && !capturing(st);
-      if (pv < 0) pv = tuning ? c->proj_tune_next : 2;
+      const bool tuning = c->opt.autotune && c->opt.proj_variant < 0 && c->proj_variant < 0 &&
+                          m >= 256 && !d_count && !capturing(st);
+      const int pv = tuning ? c->proj_tune_next : proj_kernel(c);
       if (tuning) CK(cudaEventRecord(c->ev[0], st));
       if (pv == 1 || pv == 2) {
         const long long lds = (s.n_ext + 3) & ~3;
@@ -1180,9 +1187,8 @@ int cg_workspace(pdep_ctx* c, SysData& s, int n, R** r, R** p, R** ap, int** lis
   RET(ws(c, "cg_list", (size_t)n, list));
   cpx<R>* b1;
   RET(ws(c, sizeof(R) == 8 ? "b1_64" : "b1_32", b1_count(s, (n + 1) / 2), &b1));
-  const int pv = c->opt.proj_variant >= 0 ? c->opt.proj_variant : c->proj_variant;
   R* S;
-  if (sizeof(R) == 4 && pv != 0) {
+  if (sizeof(R) == 4 && proj_kernel(c) != 0) {
     RET(ws(c, "pv_32", (size_t)((s.n_ext + 3) & ~3) * std::max(n, 1), &S));
   } else {
     RET(ws(c, sizeof(R) == 8 ? "pv_64" : "pv_32", (size_t)s.n_ext * std::max(n, 1), &S));
@@ -1372,12 +1378,6 @@ int cg_setup(pdep_ctx* c, SysData& s, R* x, int n, double tol, CgScal* sc, const
   a.tolv = tolv;
   return PDEP_OK;
 }
-// the projection kernel apply_h uses inside a captured loop
-int captured_proj(const pdep_ctx* c) {
-  const int pv = c->opt.proj_variant >= 0 ? c->opt.proj_variant : c->proj_variant;
-  return pv < 0 ? 1 : pv;
-}
-
 template <typename R>
 int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int max_iter,
             CgScal* sc, const double* mask, cudaStream_t st, const double* tolv) {
@@ -1441,7 +1441,7 @@ int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int ma
     return PDEP_OK;
   }
   a.variant = cg_variant_of(c, pi);
-  const int pv = captured_proj(c);
+  const int pv = proj_kernel(c);
   CgGraph* g = nullptr;
   for (CgGraph& e : c->cg_graphs)
     if (e.prec == pi && e.sys == si && e.n == n && e.max_iter == max_iter && e.tol == tol &&
@@ -1573,7 +1573,7 @@ int refine_rounds(pdep_ctx* c, SysData& s, const double* b, const double* xd, do
       // node runs a round only if an RHS needs it.  (Enqueued one by one, each
       // empty round cost its launches, some 58 us, and most solves need one or
       // two of the six.)
-      const int si = (int)(&s - c->sys.data()), variant = cg_variant_of(c, pi), pv = captured_proj(c);
+      const int si = (int)(&s - c->sys.data()), variant = cg_variant_of(c, pi), pv = proj_kernel(c);
       CgArgs<Ri> a{};
       int* cgl;
       RET(cg_setup<Ri>(c, s, di, n, inner, sc, rn, tolv, &a, &cgl));
