@@ -125,7 +125,7 @@ struct Tune {
 // valid for the buffers and settings it was captured with.
 struct CgGraph {
   int prec, sys, n, max_iter, cg_variant, proj_variant, tune_gen;
-  int prologue, body;  // kernels before the loop, and per step
+  int prologue;  // kernels before the loop
   double tol;
   const void *b, *x, *sc, *mask, *tolv;
   unsigned long long ws_gen, budget_ns;
@@ -136,7 +136,7 @@ struct CgGraph {
 // (each with the CG loop's node inside), valid for what it was captured with.
 struct RoundsGraph {
   int prec, sys, n, cg_variant, proj_variant, tune_gen;
-  int check, round, body;  // kernels before the first round, per round, per CG step
+  int check;  // kernels before the first round
   bool dn;               // with the density response (its array: pdep_ctx::d_dn)
   const void *b, *x, *its, *rel, *r64, *ad;
   unsigned long long ws_gen, budget_ns;
@@ -162,12 +162,9 @@ struct pdep_ctx {
   unsigned long long budget_ns = 0;   // clock_budget_cycles in ns of %globaltimer
   std::vector<CgGraph> cg_graphs;     // executable CG-loop graphs, released in pdep_destroy
   std::vector<RoundsGraph> rounds_graphs;  // likewise
-  int round_launches = 0;             // kernels per round of the last rounds graph
-  int body_launches[2] = {0, 0};      // kernels per CG step of the last graph (FP32, FP64)
   long long graph_launches = 0;       // CG graphs launched
   int graph_captures = 0;             // CG and refinement graphs captured since pdep_setup
   long long prologue_launches = 0;    // kernels before their loops
-  long long eager_steps[2] = {0, 0};  // CG steps launched from the host loop (FP32, FP64)
   long long st_launch0 = 0;           // launch counter at the last statistics reset
   pdep_stats last_dav{};              // statistics of the last pdep_solve
   cudaEvent_t ev[2] = {nullptr, nullptr};
@@ -1204,15 +1201,14 @@ CgProj<R> step_projection(const SysData& s) {
   pj.n = s.n_ext;
   return pj;
 }
-CgTail step_tail(const pdep_ctx* c, int* list, int max_iter, int prec,
-                 cudaGraphConditionalHandle h, int has_handle) {
+CgTail step_tail(const pdep_ctx* c, int* list, int max_iter, cudaGraphConditionalHandle h,
+                 int has_handle) {
   CgTail t;
   t.on = 1;
   t.ticket = c->d_counter;
   t.list = list;
   t.loop = c->d_loop;
   t.max_iter = max_iter;
-  t.prec = prec;
   t.budget_ns = c->budget_ns;
   t.handle = h;
   t.has_handle = has_handle;
@@ -1269,8 +1265,7 @@ int add_while(cudaGraph_t g, cudaGraphNode_t after, cudaGraphConditionalHandle h
 // The CG loop's nodes in graph g, behind 'after' (may be null).
 template <typename R>
 int add_cg_loop(pdep_ctx* c, SysData& s, CgArgs<R> a, const R* b, int n, int max_iter, int* list,
-                cudaGraph_t g, cudaGraphNode_t after, cudaGraphNode_t* node, int* prologue,
-                int* per_step) {
+                cudaGraph_t g, cudaGraphNode_t after, cudaGraphNode_t* node, int* prologue) {
   const int pi = sizeof(R) == 8 ? 1 : 0;
   const bool tail = n <= CG_TAIL_MAX, fuse = step_projects(c, s, pi, n);
   if (tail) a.variant = n < 256 ? (int)CG_FEW : a.variant;
@@ -1292,19 +1287,22 @@ int add_cg_loop(pdep_ctx* c, SysData& s, CgArgs<R> a, const R* b, int n, int max
   // application on 24^3, 8 RHS, 1295 -> 1230 us, 48^3, 64 RHS, 4605 -> 4454.
   // An empty FP64 step, four launches over all planes, costs more than it saves.
   const int steps = tail && pi == 0 ? 4 : 1;
-  RET(add_captured(c, body, nullptr, &bn, per_step, [&](cudaStream_t cs) -> int {
+  int pass = 0;
+  RET(add_captured(c, body, nullptr, &bn, &pass, [&](cudaStream_t cs) -> int {
     a.list_count = &c->d_loop->listed;
     const CgProj<R> pj = step_projection<R>(s);
-    const CgTail tl = step_tail(c, list, max_iter, pi, h, 1);
+    CgTail tl = step_tail(c, list, max_iter, h, 1);
     for (int k = 0; k < steps; ++k) {
       if (!tail) CK(active_list_reset(a.sc, n, list, &c->d_loop->listed, &c->d_loop->active, cs));
       RET(apply_h<R>(c, s, a.p, (R*)a.ap, n, list, n, true, !fuse, cs, nullptr, &c->d_loop->listed));
+      // the first step, which always has RHS, counts the whole pass
+      tl.launches = k == 0 ? steps * (capture_count() + 1) : 0;
       CK(cg_step<R>(a, list, n, cs, fuse ? &pj : nullptr, tail ? &tl : nullptr));
-      if (!tail) CK(loop_next(c->d_loop, max_iter, c->budget_ns, c->d_status, pi, h, 1, cs));
+      if (!tail)
+        CK(loop_next(c->d_loop, max_iter, c->budget_ns, c->d_status, capture_count() + 1, h, 1, cs));
     }
     return PDEP_OK;
   }));
-  *per_step /= steps;
   return PDEP_OK;
 }
 
@@ -1332,11 +1330,10 @@ int build_graph(pdep_ctx* c, cudaGraphExec_t* out, F fn) {
 template <typename R>
 int capture_cg_graph(pdep_ctx* c, SysData& s, const CgArgs<R>& a, const R* b, int n, int max_iter,
                      int* list, CgGraph* gr) {
-  gr->prologue = gr->body = 0;
+  gr->prologue = 0;
   return build_graph(c, &gr->exec, [&](cudaGraph_t g) -> int {
     cudaGraphNode_t node = nullptr;
-    return add_cg_loop<R>(c, s, a, b, n, max_iter, list, g, nullptr, &node, &gr->prologue,
-                          &gr->body);
+    return add_cg_loop<R>(c, s, a, b, n, max_iter, list, g, nullptr, &node, &gr->prologue);
   });
 }
 
@@ -1395,7 +1392,7 @@ int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int ma
     // eager: host loop, one 16-byte read of the loop state per step
     const bool tail = n <= CG_TAIL_MAX, fuse = step_projects(c, s, pi, n);
     const CgProj<R> pj = step_projection<R>(s);
-    const CgTail tl = step_tail(c, list, max_iter, pi, 0, 0);
+    const CgTail tl = step_tail(c, list, max_iter, 0, 0);
     CK(cudaMemsetAsync(&c->d_loop->active, 0, sizeof(int), st));
     CK(cudaMemsetAsync(c->d_counter, 0, sizeof(int), st));
     CK(cg_start<R>(a, b, s.ld, st));
@@ -1435,8 +1432,7 @@ int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int ma
           c->cg_variant[pi] = best;
         }
       }
-      if (!tail) CK(loop_next(c->d_loop, max_iter, c->budget_ns, c->d_status, pi, 0, 0, st));
-      ++c->eager_steps[pi];
+      if (!tail) CK(loop_next(c->d_loop, max_iter, c->budget_ns, c->d_status, 0, 0, 0, st));
     }
     return PDEP_OK;
   }
@@ -1483,7 +1479,6 @@ int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int ma
   }
   ++c->graph_launches;
   c->prologue_launches += g->prologue;
-  c->body_launches[pi] = g->body;
   return PDEP_OK;
 }
 
@@ -1592,15 +1587,16 @@ int refine_rounds(pdep_ctx* c, SysData& s, const double* b, const double* xd, do
             e.proj_variant == pv && e.tune_gen == c->tune_gen)
           g = &e;
       if (!g) {
-        RoundsGraph e{pi, si, n, variant, pv, c->tune_gen, 0, 0, 0, dn != nullptr, b, x, its_total,
+        RoundsGraph e{pi, si, n, variant, pv, c->tune_gen, 0, dn != nullptr, b, x, its_total,
                       rel, r64, ad, c->ws_gen, c->budget_ns, nullptr};
         RET(build_graph(c, &e.exec, [&](cudaGraph_t top) -> int {
           cudaGraphConditionalHandle h = 0;
           CK(cudaGraphConditionalHandleCreate(&h, top, 0, 0));
+          int round_launches = 0;  // of the round's parts before the one being captured
           auto check = [&](int first, cudaStream_t q) -> int {
             CK(unconverged_list(rel, tol, n, list, n_un, q, nullptr));
             CK(rounds_next(c->d_loop, n_un, first, 1, c->opt.max_refine,
-                           &c->d_dstats->rounds_cur, h, q));
+                           &c->d_dstats->rounds_cur, round_launches + capture_count() + 1, h, q));
             return PDEP_OK;
           };
           cudaGraphNode_t first = nullptr, loop = nullptr, pre = nullptr, cg = nullptr, up = nullptr;
@@ -1608,13 +1604,14 @@ int refine_rounds(pdep_ctx* c, SysData& s, const double* b, const double* xd, do
           RET(add_captured(c, top, nullptr, &first, &e.check,
                            [&](cudaStream_t q) { return check(1, q); }));
           RET(add_while(top, first, h, &loop, &body));
-          RET(add_captured(c, body, nullptr, &pre, &e.round,
+          RET(add_captured(c, body, nullptr, &pre, &round_launches,
                            [&](cudaStream_t q) { return prepare(1, q); }));
           {
             InnerFlag inner_flag(c->cg_inner, !fp64);
-            RET(add_cg_loop<Ri>(c, s, a, ri, n, max_iter, cgl, body, pre, &cg, &e.round, &e.body));
+            RET(add_cg_loop<Ri>(c, s, a, ri, n, max_iter, cgl, body, pre, &cg, &round_launches));
           }
-          return add_captured(c, body, cg, &up, &e.round, [&](cudaStream_t q) -> int {
+          int last = 0;
+          return add_captured(c, body, cg, &up, &last, [&](cudaStream_t q) -> int {
             RET(update(1, q));
             return check(0, q);
           });
@@ -1632,8 +1629,6 @@ int refine_rounds(pdep_ctx* c, SysData& s, const double* b, const double* xd, do
       }
       ++c->graph_launches;
       c->prologue_launches += g->check;
-      c->round_launches = g->round;
-      c->body_launches[pi] = g->body;
       break;
     }
     CK(unconverged_list(rel, tol, n, list, n_un, st, &c->d_dstats->rounds_cur));
@@ -1829,19 +1824,19 @@ int reset_stats(pdep_ctx* c, cudaStream_t st) {
   c->st_chunks = 0;
   c->graph_launches = 0;
   c->prologue_launches = 0;
-  c->eager_steps[0] = c->eager_steps[1] = 0;
   c->st_launch0 = launch_count();
   CK(cudaMemsetAsync(c->d_dstats, 0, sizeof(DevStats), st));
-  CK(cudaMemsetAsync(c->d_loop->steps, 0, sizeof(c->d_loop->steps), st));
+  CK(cudaMemsetAsync(&c->d_loop->launches, 0, sizeof(c->d_loop->launches), st));
   return PDEP_OK;
 }
 
 // Synchronises st and fills the solve statistics (device counters included).
 int read_stats(pdep_ctx* c, pdep_stats* out, cudaStream_t st) {
   DevStats d;
-  unsigned long long steps[3];
+  unsigned long long in_graphs;
   CK(cudaMemcpyAsync(&d, c->d_dstats, sizeof(DevStats), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(steps, c->d_loop->steps, sizeof(steps), cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(&in_graphs, &c->d_loop->launches, sizeof(in_graphs), cudaMemcpyDeviceToHost,
+                     st));
   CK(cudaStreamSynchronize(st));
   out->sternheimer_solves = c->st_solves;
   out->cg_iterations = (long long)d.cg_iters;
@@ -1855,13 +1850,10 @@ int read_stats(pdep_ctx* c, pdep_stats* out, cudaStream_t st) {
                           ? 3
                           : (c->opt.proj_variant >= 0 ? c->opt.proj_variant : c->proj_variant);
   out->chi0_chunks = c->st_chunks;
-  // launches outside graphs are counted on the host; a graph contributes its
-  // prologue per launch and its body per step, the steps counted on the device (loop_next counts eager steps too: those are subtracted)
-  long long in_graphs = c->prologue_launches;
-  in_graphs += (long long)steps[2] * c->round_launches;
-  for (int pi = 0; pi < 2; ++pi)
-    in_graphs += ((long long)steps[pi] - c->eager_steps[pi]) * c->body_launches[pi];
-  out->kernel_launches = (launch_count() - c->st_launch0) + in_graphs;
+  // launches outside graphs and those before a graph's loop are counted on the
+  // host, those of its passes on the device
+  out->kernel_launches =
+      (launch_count() - c->st_launch0) + c->prologue_launches + (long long)in_graphs;
   out->graph_launches = c->graph_launches;
   out->fused_planes = -1;
   out->gemm_shape = -1;

@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(T)
     ls->active = total;
     const int it = ls->iter + 1;
     ls->iter = it;
-    ls->steps[tail.prec] += 1;
+    ls->launches += tail.launches;
     bool go = total > 0 && it < tail.max_iter;
     if (go && tail.budget_ns > 0 && global_ns() - ls->t0 > tail.budget_ns) {
       go = false;

@@ -1348,11 +1348,11 @@ __global__ void k_loop_begin(CgLoopState* ls, int max_iter, cudaGraphConditional
   if (has_handle) cudaGraphSetConditional(h, go);
 }
 __global__ void k_loop_next(CgLoopState* ls, int max_iter, unsigned long long budget_ns,
-                            unsigned* status, int prec, cudaGraphConditionalHandle h,
+                            unsigned* status, int launches, cudaGraphConditionalHandle h,
                             int has_handle) {
   const int it = ls->iter + 1;
   ls->iter = it;
-  ls->steps[prec] += 1;
+  ls->launches += launches;
   const bool active = ls->active > 0;
   bool go = active && it < max_iter;
   if (go && budget_ns > 0 && global_ns() - ls->t0 > budget_ns) {
@@ -1369,19 +1369,19 @@ cudaError_t loop_begin(CgLoopState* ls, int max_iter, cudaGraphConditionalHandle
   return cudaGetLastError();
 }
 cudaError_t loop_next(CgLoopState* ls, int max_iter, unsigned long long budget_ns,
-                      unsigned* status, int prec, cudaGraphConditionalHandle h, int has_handle,
+                      unsigned* status, int launches, cudaGraphConditionalHandle h, int has_handle,
                       cudaStream_t st) {
   count_launch();
-  k_loop_next<<<1, 1, 0, st>>>(ls, max_iter, budget_ns, status, prec, h, has_handle);
+  k_loop_next<<<1, 1, 0, st>>>(ls, max_iter, budget_ns, status, launches, h, has_handle);
   return cudaGetLastError();
 }
 
 __global__ void k_rounds_next(CgLoopState* ls, const int* n_un, int first, int done, int max_rounds,
-                              int* rounds, cudaGraphConditionalHandle h) {
+                              int* rounds, int launches, cudaGraphConditionalHandle h) {
   if (first)
     ls->round = done;
   else
-    ls->steps[2] += 1;
+    ls->launches += launches;
   const bool go = *n_un > 0 && ls->round < max_rounds;
   if (go) {
     ls->round += 1;
@@ -1390,9 +1390,9 @@ __global__ void k_rounds_next(CgLoopState* ls, const int* n_un, int first, int d
   cudaGraphSetConditional(h, go ? 1u : 0u);
 }
 cudaError_t rounds_next(CgLoopState* ls, const int* n_un, int first, int done, int max_rounds,
-                        int* rounds, cudaGraphConditionalHandle h, cudaStream_t st) {
+                        int* rounds, int launches, cudaGraphConditionalHandle h, cudaStream_t st) {
   count_launch();
-  k_rounds_next<<<1, 1, 0, st>>>(ls, n_un, first, done, max_rounds, rounds, h);
+  k_rounds_next<<<1, 1, 0, st>>>(ls, n_un, first, done, max_rounds, rounds, launches, h);
   return cudaGetLastError();
 }
 

@@ -209,8 +209,7 @@ struct CgLoopState {
   int iter;                       // steps done in this loop
   int go;                         // 1 while another step is due
   unsigned long long t0;          // %globaltimer (ns) at the loop start
-  unsigned long long steps[3];    // steps over all loops (FP32, FP64), and refinement rounds
-                                  // run inside graphs, for launch counts
+  unsigned long long launches;    // kernels run inside graphs, but those before their loops
   int round;                      // refinement round of the enclosing graph
 };
 // Device statistics of the Sternheimer solves since the last reset.
@@ -226,18 +225,20 @@ struct DevStats {
 // step after each CG step (iter += 1; go = active > 0 && iter < max_iter &&
 // elapsed <= budget_ns; a spent budget with RHS still active sets
 // DEV_TIMEOUT).  With a graph handle (has_handle) the decision also drives
-// the enclosing while node.  prec selects the launch-count slot (0 FP32, 1 FP64).
+// the enclosing while node.  launches: kernels of a pass of that node, counted in
+// the loop state (0 from the host loop, whose launches the host counts).
 cudaError_t loop_begin(CgLoopState* ls, int max_iter, cudaGraphConditionalHandle h, int has_handle,
                        cudaStream_t st);
 cudaError_t loop_next(CgLoopState* ls, int max_iter, unsigned long long budget_ns,
-                      unsigned* status, int prec, cudaGraphConditionalHandle h, int has_handle,
+                      unsigned* status, int launches, cudaGraphConditionalHandle h, int has_handle,
                       cudaStream_t st);
 // Loop control of the refinement rounds inside a graph: another round runs while
 // *n_un RHS are unconverged and fewer than max_rounds have run (first: the check
 // before them, with 'done' rounds run already); a round that starts is counted
-// in *rounds.
+// in *rounds, and one that ends adds its launches (but those of its CG loop's
+// passes) to the loop state's count.
 cudaError_t rounds_next(CgLoopState* ls, const int* n_un, int first, int done, int max_rounds,
-                        int* rounds, cudaGraphConditionalHandle h, cudaStream_t st);
+                        int* rounds, int launches, cudaGraphConditionalHandle h, cudaStream_t st);
 // After a CG loop: its_total[i] += sc[i].iters (its_total may be null), and
 // the sum / largest count into ds.
 cudaError_t cg_collect(const CgScal* sc, int n, int* its_total, DevStats* ds, cudaStream_t st);
@@ -270,7 +271,8 @@ struct CgTail {
   int* ticket = nullptr;
   int* list = nullptr;
   CgLoopState* loop = nullptr;
-  int max_iter = 0, prec = 0;
+  int max_iter = 0;
+  int launches = 0;    // kernels this step adds to the loop state's count
   unsigned long long budget_ns = 0;
   cudaGraphConditionalHandle handle = 0;
   int has_handle = 0;  // the decision also drives the enclosing while node

@@ -127,6 +127,8 @@ int capture_end() {
   return t_capture_launches;
 }
 
+int capture_count() { return t_capture_launches; }
+
 long long launch_count() { return g_launches.load(std::memory_order_relaxed); }
 
 namespace {

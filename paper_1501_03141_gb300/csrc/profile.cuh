@@ -31,6 +31,7 @@ enum ProfClass : int {
 void count_launch();
 void capture_begin();
 int capture_end();
+int capture_count();  // launches counted so far
 // kernels launched by this process outside graph captures (always counted)
 long long launch_count();
 
