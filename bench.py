@@ -323,7 +323,6 @@ def run_ours(args):
     barrier()
     clocks = ClockSampler(local)
     clocks.start()
-    pg.profile_start()
     e0 = torch.cuda.Event(enable_timing=True)
     e1 = torch.cuda.Event(enable_timing=True)
     torch.cuda.synchronize(dev)
@@ -344,9 +343,14 @@ def run_ours(args):
     torch.cuda.synchronize(dev)
     if nvtx is not None:
         nvtx.range_pop()
-    prof = pg.profile_stop()
     clk = clocks.stop()
     barrier()
+    mixed_vals = ev.cpu().numpy()
+    # the kernel profile of one more step: the timers' code and events stay out
+    # of the timed ones
+    pg.profile_start()
+    ctx.pdep_solve(phi0=phi0_dev, eigvals=ev, eigvecs=evec)
+    prof = pg.profile_stop()
     t_local = e0.elapsed_time(e1) / 1e3
     bounds = [e0] + marks + [e1]
     step_ms = step_spread([a.elapsed_time(b) for a, b in zip(bounds[:-1], bounds[1:])])
@@ -354,7 +358,6 @@ def run_ours(args):
     total_solves = reduce_scalar(solves, "sum", dev if world > 1 else None)
     value = total_solves / t
     eigpairs = world * npd * args.steps / t
-    mixed_vals = ev.cpu().numpy()
 
     # e2e: the same step through the public API with pinned host buffers
     phi0 = torch.from_numpy(phi0_np).pin_memory()

@@ -126,6 +126,7 @@ struct Tune {
 struct CgGraph {
   int prec, sys, n, max_iter, cg_variant, proj_variant, tune_gen;
   int prologue;  // kernels before the loop
+  bool prof;     // with timers in its kernels
   double tol;
   const void *b, *x, *sc, *mask, *tolv;
   unsigned long long ws_gen, budget_ns;
@@ -137,6 +138,7 @@ struct CgGraph {
 struct RoundsGraph {
   int prec, sys, n, cg_variant, proj_variant, tune_gen;
   int check;  // kernels before the first round
+  bool prof;  // with timers in its kernels
   bool dn;               // with the density response (its array: pdep_ctx::d_dn)
   const void *b, *x, *its, *rel, *r64, *ad;
   unsigned long long ws_gen, budget_ns;
@@ -1444,7 +1446,7 @@ int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int ma
         e.b == b && e.x == x && e.sc == sc && e.mask == mask && e.tolv == tolv &&
         e.ws_gen == c->ws_gen &&
         e.cg_variant == a.variant && e.proj_variant == pv && e.budget_ns == c->budget_ns &&
-        e.tune_gen == c->tune_gen) {
+        e.tune_gen == c->tune_gen && e.prof == profiling()) {
       g = &e;
       break;
     }
@@ -1465,6 +1467,7 @@ int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int ma
     e.proj_variant = pv;
     e.budget_ns = c->budget_ns;
     e.tune_gen = c->tune_gen;
+    e.prof = profiling();
     RET(capture_cg_graph<R>(c, s, a, b, n, max_iter, list, &e));
     if (c->cg_graphs.size() >= 16) {
       cudaGraphExecDestroy(c->cg_graphs.front().exec);
@@ -1584,11 +1587,11 @@ int refine_rounds(pdep_ctx* c, SysData& s, const double* b, const double* xd, do
         if (e.prec == pi && e.sys == si && e.n == n && e.b == b && e.x == x &&
             e.dn == (dn != nullptr) && e.its == its_total && e.rel == rel && e.r64 == r64 && e.ad == ad &&
             e.ws_gen == c->ws_gen && e.budget_ns == c->budget_ns && e.cg_variant == variant &&
-            e.proj_variant == pv && e.tune_gen == c->tune_gen)
+            e.proj_variant == pv && e.tune_gen == c->tune_gen && e.prof == profiling())
           g = &e;
       if (!g) {
-        RoundsGraph e{pi, si, n, variant, pv, c->tune_gen, 0, dn != nullptr, b, x, its_total,
-                      rel, r64, ad, c->ws_gen, c->budget_ns, nullptr};
+        RoundsGraph e{pi, si, n, variant, pv, c->tune_gen, 0, profiling(), dn != nullptr, b, x,
+                      its_total, rel, r64, ad, c->ws_gen, c->budget_ns, nullptr};
         RET(build_graph(c, &e.exec, [&](cudaGraph_t top) -> int {
           cudaGraphConditionalHandle h = 0;
           CK(cudaGraphConditionalHandleCreate(&h, top, 0, 0));

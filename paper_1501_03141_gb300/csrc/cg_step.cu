@@ -356,9 +356,10 @@ __device__ __forceinline__ bool stage_wait(unsigned long long* bar, uint32_t par
   }
 }
 
-template <typename R, int T>
+// TIMED: the form inside graphs captured while profiling
+template <typename R, int T, bool TIMED>
 __global__ void __launch_bounds__(T)
-    k_cg_stream(CgArgs<R> a, const int* __restrict__ list, int rowb) {
+    k_cg_stream(CgArgs<R> a, const int* __restrict__ list, int rowb, DevTimer* timer) {
   constexpr int E = Vec<R>::n, V = CG_STREAM_V;
   extern __shared__ __align__(128) unsigned char stages[];
   __shared__ __align__(8) unsigned long long full[2];
@@ -370,6 +371,7 @@ __global__ void __launch_bounds__(T)
   const int listed = a.list_count ? *a.list_count : a.n_listed;
   int k = blockIdx.x;
   if (k >= listed) return;
+  if (TIMED && k == 0 && tid == 0) dev_timer_first(timer);
   auto rhs = [&](int q) { return q < listed ? (list ? list[q] : q) : -1; };
   // by one thread: the four rows of RHS i into a stage
   auto issue = [&](int st, int i) {
@@ -511,11 +513,15 @@ __global__ void __launch_bounds__(T)
     if (i1 >= 0) stage_wait(&full[nx & 1], (nx >> 1) & 1);
     stage_wait(&full[it & 1], (it >> 1) & 1);
   }
+  if (TIMED && tid == 0)
+    dev_timer_done(timer, min(listed, G), blockIdx.x == 0, 12.0 * listed * (double)a.n_pw,
+                   7.0 * listed * (double)a.n_pw * sizeof(R));
 }
 
-template <typename R, int T>
-cudaError_t launch_stream(const CgArgs<R>& a, const int* list, int nb, int rowb, cudaStream_t st) {
-  auto kern = k_cg_stream<R, T>;
+template <typename R, int T, bool TIMED>
+cudaError_t launch_stream_form(const CgArgs<R>& a, const int* list, int nb, int rowb, DevTimer* timer,
+                               cudaStream_t st) {
+  auto kern = k_cg_stream<R, T, TIMED>;
   static OncePerDevice limit;  // per instantiation
   if (const cudaError_t e = raise_smem_limit(limit, kern, (int)CG_STREAM_SMEM)) return e;
   const size_t smem = 8 * (size_t)rowb;
@@ -528,8 +534,14 @@ cudaError_t launch_stream(const CgArgs<R>& a, const int* list, int nb, int rowb,
   int per = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, T, smem);
   if (e != cudaSuccess) return e;
-  kern<<<std::min(nb, std::max(per, 1) * sms), T, smem, st>>>(a, list, rowb);
+  kern<<<std::min(nb, std::max(per, 1) * sms), T, smem, st>>>(a, list, rowb, timer);
   return cudaGetLastError();
+}
+template <typename R, int T>
+cudaError_t launch_stream(const CgArgs<R>& a, const int* list, int nb, int rowb, cudaStream_t st) {
+  DevTimer* timer = capture_timer(sizeof(R) == 8 ? PC_CG_F64 : PC_CG_F32);
+  return timer ? launch_stream_form<R, T, true>(a, list, nb, rowb, timer, st)
+               : launch_stream_form<R, T, false>(a, list, nb, rowb, nullptr, st);
 }
 
 // bytes of a row in a stage

@@ -158,6 +158,8 @@ int dev_timers_init() {
 }
 
 DevTimer* dev_timer(int cls) { return g_timers ? g_timers + cls : nullptr; }
+bool profiling() { return prof().on; }
+DevTimer* capture_timer(int cls) { return t_capturing && profiling() ? dev_timer(cls) : nullptr; }
 
 // records nothing while the stream is being captured (events cannot time a
 // kernel inside a graph, and resolving records waits on events, which a

@@ -50,6 +50,13 @@ struct DevTimer {
 };
 int dev_timers_init();
 DevTimer* dev_timer(int cls);
+// The timer of a kernel that ProfScope times when it is launched on its own and
+// that is timed on the device inside a graph captured while profiling (a null
+// timer times nothing, so other graphs pay nothing; graphs are keyed by
+// profiling()): the FP32 projections on the tensor cores and the streamed CG step.
+// The step of few RHS, all latency, has none.
+DevTimer* capture_timer(int cls);
+bool profiling();
 
 __device__ __forceinline__ unsigned long long dev_clock_ns() {
   unsigned long long t;
@@ -72,6 +79,30 @@ __device__ __forceinline__ void dev_timer_block_end(DevTimer* t, unsigned long l
     t->launches += 1;
     t->t_min = ~0ull;
     t->t_max = 0ull;
+    t->done = 0u;
+  }
+}
+
+// For kernels of many blocks: one atomic per block.  By thread 0 of the launch's
+// first block at its start, and of every block that works at its end ('blocks' of
+// them; first: this is the first one, which adds the launch's work).
+__device__ __forceinline__ void dev_timer_first(DevTimer* t) {
+  if (t) atomicMin(&t->t_min, dev_clock_ns());
+}
+__device__ __forceinline__ void dev_timer_done(DevTimer* t, unsigned blocks, bool first,
+                                               double flops, double bytes) {
+  if (!t) return;
+  if (first) {
+    atomicAdd(&t->flops, flops);
+    atomicAdd(&t->bytes, bytes);
+  }
+  __threadfence();
+  if (atomicAdd(&t->done, 1u) == blocks - 1) {
+    __threadfence();
+    const unsigned long long lo = atomicOr(&t->t_min, 0ull), hi = dev_clock_ns();
+    t->total_ns += hi > lo ? hi - lo : 0ull;
+    t->launches += 1;
+    t->t_min = ~0ull;
     t->done = 0u;
   }
 }

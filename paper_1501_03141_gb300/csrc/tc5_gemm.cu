@@ -240,12 +240,13 @@ struct C5Pos {
   }
 };
 
-template <int BF>
+// TIMED: the form inside graphs captured while profiling
+template <int BF, bool TIMED>
 __global__ void __launch_bounds__(C5_THREADS, 1)
     k_tc5_coeffs(int n_ext, int N, int K, C5Geom g, const unsigned char* __restrict__ Pt,
                  const float* __restrict__ X, long long ldx, const int* __restrict__ bmap,
                  const float* __restrict__ sigma, float* __restrict__ S, long long lds,
-                 const int* __restrict__ ndev, unsigned* status) {
+                 const int* __restrict__ ndev, unsigned* status, DevTimer* timer) {
   extern __shared__ unsigned char c5_dyn[];
   // conv_full / conv_empty: converted buffer c holds unit i / is free again;
   // acc_full / acc_empty: accumulator a holds unit i / has been read;
@@ -261,6 +262,7 @@ __global__ void __launch_bounds__(C5_THREADS, 1)
   const int u0 = (int)((long long)U * blockIdx.x / gridDim.x);
   const int n = (int)((long long)U * (blockIdx.x + 1) / gridDim.x) - u0;
   if (n <= 0) return;
+  if (TIMED && threadIdx.x == 0) dev_timer_first(timer);  // (one block per SM: all of them)
   unsigned char* base = (unsigned char*)(((uintptr_t)c5_dyn + 1023) & ~(uintptr_t)1023);
   const uint32_t sbase = su32(base);
   const int R = c5_ring(g.nt);
@@ -502,6 +504,9 @@ __global__ void __launch_bounds__(C5_THREADS, 1)
   }
   __syncthreads();
   if (abort_flag && tid == 0) atomicOr(status, (unsigned)DEV_TIMEOUT);
+  if (TIMED && tid == 0)
+    dev_timer_done(timer, min(U, (int)gridDim.x), u0 == 0, 2.0 * n_ext * N * (double)K,
+                   ((double)n_ext * K + (double)K * N + (double)n_ext * N) * sizeof(float));
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -599,12 +604,17 @@ cudaError_t tc5_proj_coeffs(int n_ext, int N, int K, const void* Pt, const float
   if (K <= 0) return cudaMemsetAsync(S, 0, sizeof(float) * (size_t)lds * N, st);
   const C5Geom g = c5_geom(n_ext, K);
   const int smem = c5_smem(g.nt);
-  static int attr[2] = {0, 0};
-  if (smem > attr[bf16]) {
-    cudaError_t e = cudaFuncSetAttribute(bf16 ? k_tc5_coeffs<1> : k_tc5_coeffs<0>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  DevTimer* timer = capture_timer(PC_GEMM_TF32);
+  const int form = 2 * (bf16 ? 1 : 0) + (timer ? 1 : 0);
+  auto kern = form == 0   ? k_tc5_coeffs<0, false>
+              : form == 1 ? k_tc5_coeffs<0, true>
+              : form == 2 ? k_tc5_coeffs<1, false>
+                          : k_tc5_coeffs<1, true>;
+  static int attr[4] = {0, 0, 0, 0};
+  if (smem > attr[form]) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    attr[bf16] = smem;
+    attr[form] = smem;
   }
   cudaError_t e = cudaMemsetAsync(S, 0, sizeof(float) * (size_t)lds * N, st);
   if (e != cudaSuccess) return e;
@@ -616,12 +626,8 @@ cudaError_t tc5_proj_coeffs(int n_ext, int N, int K, const void* Pt, const float
                ((double)n_ext * K + (double)K * N + (double)n_ext * N) * sizeof(float), ndev, N);
   count_launch();
   const unsigned char* pt = (const unsigned char*)Pt;
-  if (bf16)
-    k_tc5_coeffs<1><<<grid, C5_THREADS, smem, st>>>(n_ext, N, K, g, pt, X, ldx, bmap, sigma, S,
-                                                    lds, ndev, status);
-  else
-    k_tc5_coeffs<0><<<grid, C5_THREADS, smem, st>>>(n_ext, N, K, g, pt, X, ldx, bmap, sigma, S,
-                                                    lds, ndev, status);
+  kern<<<grid, C5_THREADS, smem, st>>>(n_ext, N, K, g, pt, X, ldx, bmap, sigma, S, lds, ndev, status,
+                                       timer);
   return cudaGetLastError();
 }
 

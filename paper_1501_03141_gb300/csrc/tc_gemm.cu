@@ -65,11 +65,14 @@ __device__ __forceinline__ void cp_wait() {
 // ---------------------------------------------------------------------------
 constexpr int C_BM = 32, C_BN = 64, C_BK = 32, C_PAD = 36;
 
+// TIMED: the form inside graphs captured while profiling (the timer's code in the
+// other would change its schedule: k_tc_update lost 6%)
+template <bool TIMED>
 __global__ void __launch_bounds__(128)
     k_tc_coeffs(int M, int N, int K, const float* __restrict__ P, long long ldp,
                 const float* __restrict__ X, long long ldx, const int* __restrict__ bmap,
                 const float* __restrict__ sigma, float* __restrict__ S, long long lds,
-                int kchunk, const int* __restrict__ ndev) {
+                int kchunk, const int* __restrict__ ndev, DevTimer* timer) {
   __shared__ __align__(16) float As[2][C_BM][C_PAD];
   __shared__ __align__(16) float Bs[2][C_BN][C_PAD];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -77,6 +80,8 @@ __global__ void __launch_bounds__(128)
   const int row0 = blockIdx.x * C_BM, col0 = blockIdx.y * C_BN;
   if (ndev) N = min(N, *ndev);  // device count of the mapped columns
   if (col0 >= N) return;
+  const bool first = TIMED && tid == 0 && blockIdx.x + blockIdx.y + blockIdx.z == 0;
+  if (first) dev_timer_first(timer);
   const int kbeg = blockIdx.z * kchunk;
   const int kend = min(K, kbeg + kchunk);
 
@@ -179,6 +184,9 @@ __global__ void __launch_bounds__(128)
         const int j = col0 + warp * 16 + ni * 8 + 2 * t + (e & 1);
         if (r < M && j < N && nk > 0) atomicAdd(S + r + (long long)j * lds, sigma[r] * acc[mi][ni][e]);
       }
+  if (TIMED && tid == 0)
+    dev_timer_done(timer, gridDim.x * ((N + C_BN - 1) / C_BN) * gridDim.z, first, 2.0 * M * N * (double)K,
+                   ((double)M * K + (double)K * N + (double)M * N) * sizeof(float));
 }
 
 // ---------------------------------------------------------------------------
@@ -187,10 +195,11 @@ __global__ void __launch_bounds__(128)
 // ---------------------------------------------------------------------------
 constexpr int U_BM = 64, U_BN = 64, U_BK = 16, U_APAD = 72, U_BPAD = 20;
 
+template <bool TIMED>
 __global__ void __launch_bounds__(128)
     k_tc_update(int M, int N, int K, const float* __restrict__ P, long long ldp,
                 const float* __restrict__ S, long long lds, float* __restrict__ Y, long long ldy,
-                const int* __restrict__ cmap, const int* __restrict__ ndev) {
+                const int* __restrict__ cmap, const int* __restrict__ ndev, DevTimer* timer) {
   __shared__ __align__(16) float As[2][U_BK][U_APAD];  // A(r, w) at As[w][r]
   __shared__ __align__(16) float Bs[2][U_BN][U_BPAD];  // B(w, j) at Bs[j][w]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -199,6 +208,8 @@ __global__ void __launch_bounds__(128)
   const int row0 = blockIdx.x * U_BM, col0 = blockIdx.y * U_BN;
   if (ndev) N = min(N, *ndev);
   if (col0 >= N) return;
+  const bool first = TIMED && tid == 0 && blockIdx.x + blockIdx.y == 0;
+  if (first) dev_timer_first(timer);
 
   auto load = [&](int stage, int k0) {
     // A: 16 state columns x 16 chunks of 4 rows
@@ -301,6 +312,9 @@ __global__ void __launch_bounds__(128)
         const int j = col0 + wn * 32 + ni * 8 + 2 * t + (e & 1);
         if (r < M && j < N) Y[r + (long long)(cmap ? cmap[j] : j) * ldy] = acc[mi][ni][e];
       }
+  if (TIMED && tid == 0)
+    dev_timer_done(timer, gridDim.x * ((N + U_BN - 1) / U_BN), first, 2.0 * M * N * (double)K,
+                   ((double)M * K + (double)K * N + 2.0 * M * N) * sizeof(float));
 }
 
 }  // namespace
@@ -326,7 +340,9 @@ cudaError_t tc_proj_coeffs(int M, int N, int K, const float* P, long long ldp, c
   ProfScope ps(PC_GEMM_TF32, st, 2.0 * M * N * (double)K,
                ((double)M * K + (double)K * N + (double)M * N) * sizeof(float), ndev, N);
   count_launch();
-  k_tc_coeffs<<<grid, 128, 0, st>>>(M, N, K, P, ldp, X, ldx, bmap, sigma, S, lds, kchunk, ndev);
+  DevTimer* timer = capture_timer(PC_GEMM_TF32);
+  auto kern = timer ? k_tc_coeffs<true> : k_tc_coeffs<false>;
+  kern<<<grid, 128, 0, st>>>(M, N, K, P, ldp, X, ldx, bmap, sigma, S, lds, kchunk, ndev, timer);
   return cudaGetLastError();
 }
 
@@ -339,7 +355,9 @@ cudaError_t tc_proj_update(int M, int N, int K, const float* P, long long ldp, c
   ProfScope ps(PC_GEMM_TF32, st, 2.0 * M * N * (double)K,
                ((double)M * K + (double)K * N + 2.0 * M * N) * sizeof(float), ndev, N);
   count_launch();
-  k_tc_update<<<grid, 128, 0, st>>>(M, N, K, P, ldp, S, lds, Y, ldy, cmap, ndev);
+  DevTimer* timer = capture_timer(PC_GEMM_TF32);
+  auto kern = timer ? k_tc_update<true> : k_tc_update<false>;
+  kern<<<grid, 128, 0, st>>>(M, N, K, P, ldp, S, lds, Y, ldy, cmap, ndev, timer);
   return cudaGetLastError();
 }
 
