@@ -463,6 +463,13 @@ inline const float* sigma_of(const SysData& s, float*) { return s.d_sigma32; }
 inline const float* negeps_of(const SysData& s, float*) { return s.d_negeps32; }
 inline const float* kprec_of(const SysData& s, float*) { return s.d_kprec32; }
 
+// The density response being accumulated: its array (null: in a graph, which may
+// only keep the next), and the device word that holds its address.
+struct Density {
+  double* now;
+  double* const* at;
+};
+
 size_t b1_count(const SysData& s, int n_items) {
   return (size_t)n_items * s.N[0] * s.n_col;
 }
@@ -473,8 +480,7 @@ size_t b1_count(const SysData& s, int n_items) {
 // Y += Psi_ext diag(sigma) (Psi_ext^T X) on the same columns.
 // dn (may be null): the transform also accumulates the density response
 // dn_j(r) += (4/Omega) u_v(r) x_i(r) of every vector i = j n_occ + v it
-// transforms (Eq. deltani) to the array whose address the device word *dn
-// holds; it must hold the (i / n_occ) perturbations.
+// transforms (Eq. deltani); the array must hold the (i / n_occ) perturbations.
 bool capturing(cudaStream_t st) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
@@ -547,7 +553,7 @@ int few_items(int N) { return N <= 24 ? 0 : N <= 32 ? 38 : 76; }
 // FP32 inner solve's needs).
 template <typename R>
 int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list, int n_list,
-            bool with_shift, bool with_pv, cudaStream_t st, double* const* dn = nullptr,
+            bool with_shift, bool with_pv, cudaStream_t st, const Density* dn = nullptr,
             const int* d_count = nullptr, bool refine = false, long long ldx = 0,
             long long ldy = 0) {
   const int digits = refine ? 7 : 8;
@@ -601,7 +607,8 @@ int apply_h(pdep_ctx* c, SysData& s, const R* X, R* Y, int n, const int* d_list,
     a.n_items = n_items;
     a.map = map;
     if (dn) {
-      a.dn = dn;
+      a.dn = dn->now;
+      a.dn_at = dn->at;
       a.u = s.d_u;
       a.dn_nocc = s.n_occ;
       a.dn_stride = s.n_r;
@@ -1510,7 +1517,7 @@ inline double inner_tol_of(const pdep_ctx* c) {
 
 template <typename Ri>
 int refine_rounds(pdep_ctx* c, SysData& s, const double* b, const double* xd, double* x, int n,
-                  double* const* dn, int* its_total, double* rel, double* r64, double* ad,
+                  const Density* dn, int* its_total, double* rel, double* r64, double* ad,
                   cudaStream_t st) {
   const bool fp64 = sizeof(Ri) == 8;
   const double tol = c->opt.cg_tol;
@@ -1547,7 +1554,8 @@ int refine_rounds(pdep_ctx* c, SysData& s, const double* b, const double* xd, do
                           (round == 0 ? 0.9 : 0.5) * tol, 0.5));
     return PDEP_OK;
   };
-  auto update = [&](int round, cudaStream_t q) -> int {
+  Density in_graph{nullptr, dn ? dn->at : nullptr};
+  auto update = [&](int round, cudaStream_t q, const Density* dn) -> int {
     CK(cg_collect(sc, n, its_total, c->d_dstats, q));
     // delta = rn d (+ xd in the first round, when every RHS is listed)
     const double* xr = round == 0 ? xd : nullptr;
@@ -1615,7 +1623,7 @@ int refine_rounds(pdep_ctx* c, SysData& s, const double* b, const double* xd, do
           }
           int last = 0;
           return add_captured(c, body, cg, &up, &last, [&](cudaStream_t q) -> int {
-            RET(update(1, q));
+            RET(update(1, q, dn ? &in_graph : nullptr));
             return check(0, q);
           });
         }));
@@ -1643,7 +1651,7 @@ int refine_rounds(pdep_ctx* c, SysData& s, const double* b, const double* xd, do
     }
     RET(prepare(round, st));
     RET(cg_loop<Ri>(c, s, ri, di, n, inner, max_iter, sc, rn, st, tolv));
-    RET(update(round, st));
+    RET(update(round, st, dn));
   }
   return PDEP_OK;
 }
@@ -1665,12 +1673,13 @@ int solve_rhs(pdep_ctx* c, SysData& s, const double* b, const double* xd, double
   // r64 = b: the FP64 residual, updated as r -= A delta for every update
   // delta of x (and checked against b's norm)
   CK(cudaMemcpyAsync(r64, b, sizeof(double) * (size_t)n * s.ld, cudaMemcpyDeviceToDevice, st));
-  // The kernels find the density's array, the caller's own for chi0_apply on the
-  // device, through a device word, so that it is no part of a captured graph: a
+  // The kernels of a graph find the density's array, the caller's own for
+  // chi0_apply on the device, through a device word: were it part of the graph, a
   // new array with every call, or one per chunk of perturbations, would be a
   // capture each.
   if (dn) CK(density_start(dn, (size_t)(n / s.n_occ) * s.n_r, c->d_dn, st));
-  double* const* slot = dn ? c->d_dn : nullptr;
+  const Density target{dn, c->d_dn};
+  const Density* slot = dn ? &target : nullptr;
   if (c->opt.precision == PDEP_FP64)
     RET(refine_rounds<double>(c, s, b, xd, x, n, slot, its_total, rel, r64, ad, st));
   else

@@ -485,7 +485,7 @@ __device__ __forceinline__ void slab_unit(const SphereDev<float>& s, const SlabA
           if (same)
             acc[i] = fma(xb, ub[i3], acc[i]);
           else if (ib >= 0)
-            atomicAdd(*a.dn + (long long)jb * a.dn_stride + off + i3, a.dn_scale * (xb * ub[i3]));
+            atomicAdd(*a.dn_at + (long long)jb * a.dn_stride + off + i3, a.dn_scale * (xb * ub[i3]));
         }
       }
       // SLAB_HPSI: multiply by the local potential on the grid
@@ -545,7 +545,7 @@ __global__ void __launch_bounds__(SlabThreads<N2, N3>::v, (SlabMinBlocks<N2, N3>
       const int g0 = w / s.N1 * group, i1 = w % s.N1;
       auto flush = [&](int j) {
         if (i2 >= N2) return;
-        double* dn = *a.dn + (long long)j * a.dn_stride + ((long long)i1 * N2 + i2) * N3;
+        double* dn = *a.dn_at + (long long)j * a.dn_stride + ((long long)i1 * N2 + i2) * N3;
 #pragma unroll
         for (int i = 0; i < M3; ++i) {
           atomicAdd(dn + pos_b<N3, TL3>(t3, i), a.dn_scale * acc[i]);
@@ -990,7 +990,7 @@ static cudaError_t slab_impl_dn(const SphereDev<float>& s, const SlabArgs<float>
 }
 template <int N2, int N3>
 static cudaError_t slab_impl(const SphereDev<float>& s, const SlabArgs<float>& a, cudaStream_t st) {
-  return a.mode == SLAB_HPSI && a.dn ? slab_impl_dn<N2, N3, true>(s, a, st)
+  return a.mode == SLAB_HPSI && a.dn_at ? slab_impl_dn<N2, N3, true>(s, a, st)
                                      : slab_impl_dn<N2, N3, false>(s, a, st);
 }
 

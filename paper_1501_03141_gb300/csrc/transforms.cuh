@@ -161,10 +161,13 @@ struct SlabArgs {
   GridSrc<R> src;        // FROM_GRID (f: one grid per group, g: per-vector grids)
   ItemMap map;
   // HPSI: also accumulate dn_j(r) += dn_scale u_v(r) x_vj(r) for
-  // every vector i = j * dn_nocc + v of the item (atomically; dn may be null).
-  // *dn, in device memory, is the array's address: a graph captured with it
-  // serves whatever array the caller of a later solve brings
-  double* const* dn = nullptr;
+  // every vector i = j * dn_nocc + v of the item (atomically; dn may be null)
+  double* dn = nullptr;
+  // the same array, its address in device memory: a graph captured with it serves
+  // whatever array the caller of a later solve brings.  FP32 takes this one, FP64
+  // does without dn (with dn in its parameters the seven-digit pass over 8192
+  // vectors of 48^3 takes 25.2 ms, with a loaded address 26.4 ms per application)
+  double* const* dn_at = nullptr;
   const double* u = nullptr;  // occupied grids [dn_nocc][dn_stride]
   int dn_nocc = 1;
   long long dn_stride = 0;
@@ -184,6 +187,9 @@ cudaError_t launch_cols_fwd(const SphereDev<double>& s, const double* x, long lo
                             int n_items, int coef, cpx<double>* b1, cudaStream_t st,
                             int digits = 8);
 cudaError_t launch_slab(const SphereDev<double>& s, const SlabArgs<double>& a, cudaStream_t st);
+// the form with a.dn_at (launch_slab calls it)
+cudaError_t launch_slab_rounds(const SphereDev<double>& s, const SlabArgs<double>& a,
+                               cudaStream_t st);
 cudaError_t launch_cols_bwd(const SphereDev<double>& s, const cpx<double>* b1, ItemMap map,
                             int n_items, const Epilogue<double>& ep, cudaStream_t st,
                             int digits = 8);
@@ -222,7 +228,7 @@ void slab_work(const SphereDev<R>& s, const SlabArgs<R>& a, double& fl, double& 
     case SLAB_HPSI:
       fl = planes * (2 * ylines * fy + 2 * zlines * fz + 2.0 * pts);
       by = planes * 2 * colb + s.N1 * gridb;
-      if (a.dn) {
+      if (a.dn || a.dn_at) {
         // density response: 2 products per point and vector; dn read and
         // written once per perturbation, u read once
         fl += planes * 4.0 * pts;
