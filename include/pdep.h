@@ -112,8 +112,8 @@ typedef enum {
                           refinement rounds follow.  The refinement's products
                           are those of the TF32 mode, so solutions still reach
                           cg_tol in the FP64 residual.  On the 48^3 workload it
-                          is 13% slower than PDEP_MIXED_TF32 (5 rounds instead of
-                          2) and matches FP64 eigenvalues to 4e-10. */
+                          is 15% slower than PDEP_MIXED_TF32 (5 rounds instead of
+                          2) and matches FP64 eigenvalues to 1.5e-8. */
 } pdep_precision;
 #define PDEP_MIXED PDEP_MIXED_TF32 /* the default mixed mode */
 

@@ -474,13 +474,6 @@ size_t b1_count(const SysData& s, int n_items) {
   return (size_t)n_items * s.N[0] * s.n_col;
 }
 
-// Y = (H - eps_v) X for the vectors of 'map' (H = -nabla^2/2 + V); vector i
-// uses occupied state i % n_occ; without with_shift Y = H X.  Then, if
-// with_pv, the occupied and deflated states are shifted:
-// Y += Psi_ext diag(sigma) (Psi_ext^T X) on the same columns.
-// dn (may be null): the transform also accumulates the density response
-// dn_j(r) += (4/Omega) u_v(r) x_i(r) of every vector i = j n_occ + v it
-// transforms (Eq. deltani); the array must hold the (i / n_occ) perturbations.
 bool capturing(cudaStream_t st) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
@@ -537,9 +530,6 @@ std::string shape_key(const char* what, const SysData& s) {
   return std::string(what) + ":" + std::to_string(s.n_ext) + ":" + std::to_string(s.n_pw);
 }
 
-// d_count (with d_list): device length of the list; n_list is then the
-// largest length, which sizes the launches (kernels read the count).
-//
 // Items (vector pairs) up to which FP32 H x takes three launches over all planes
 // instead of one with a block per item, whose time is then one item's (11, 17, 37
 // and 54 us on 24^3 .. 48^3).  One chi0 application in us, three launches against
@@ -548,6 +538,15 @@ std::string shape_key(const char* what, const SysData& s) {
 // 3854 against 4145; 48^3, 64 items 6267 against 6961, 128 items 10032 against 7904.
 int few_items(int N) { return N <= 24 ? 0 : N <= 32 ? 38 : 76; }
 
+// Y = (H - eps_v) X for the vectors of 'map' (H = -nabla^2/2 + V); vector i
+// uses occupied state i % n_occ; without with_shift Y = H X.  Then, if
+// with_pv, the occupied and deflated states are shifted:
+// Y += Psi_ext diag(sigma) (Psi_ext^T X) on the same columns.
+// dn (may be null): the transform also accumulates the density response
+// dn_j(r) += (4/Omega) u_v(r) x_i(r) of every vector i = j n_occ + v it
+// transforms (Eq. deltani); the array must hold the (i / n_occ) perturbations.
+// d_count (with d_list): device length of the list; n_list is then the
+// largest length, which sizes the launches (kernels read the count).
 // R: FP32 or FP64.  refine (FP64): the product of a mixed-mode refinement, whose
 // transforms take seven digits (errors below 2e-15 of the product, far below the
 // FP32 inner solve's needs).
@@ -1224,15 +1223,6 @@ CgTail step_tail(const pdep_ctx* c, int* list, int max_iter, cudaGraphConditiona
   return t;
 }
 
-// Captures one CG loop over n RHS into an executable graph:
-//   prologue: active = 0, cg_start (r = b, p = K b, active count), loop_begin
-//   while (go): active list, A p on the listed RHS, PCG step, loop_next
-// Up to CG_TAIL_MAX RHS the step's last cluster builds the next list and takes
-// the loop decision (the first list comes with the prologue), and where the
-// states are read within few_projection's limit the step adds the projection:
-// a step is then the transform's launches and one more.
-// Launches inside are sized for n; the kernels read the list length from
-// the device loop state.  All workspace is allocated beforehand (cg_workspace).
 // captures what fn enqueues on the capture stream as a child graph of g behind
 // 'after' (may be null); launches counts its kernels
 template <typename F>
@@ -1271,7 +1261,17 @@ int add_while(cudaGraph_t g, cudaGraphNode_t after, cudaGraphConditionalHandle h
   return PDEP_OK;
 }
 
-// The CG loop's nodes in graph g, behind 'after' (may be null).
+// The nodes of one CG loop over n RHS in graph g, behind 'after' (may be null):
+//   prologue: active = 0, cg_start (r = b, p = K b, active count), loop_begin
+//   while (go): active list, A p on the listed RHS, PCG step, loop_next
+// Up to CG_TAIL_MAX RHS the step's last cluster builds the next list and takes
+// the loop decision (the first list comes with the prologue), and where the
+// states are read within few_projection's limit the step adds the projection:
+// a step is then the transform's launches and one more.
+// Launches inside are sized for n; the kernels read the list length from
+// the device loop state.  All workspace is allocated beforehand (cg_workspace).
+// prologue counts the kernels before the loop; those of its passes are counted on
+// the device.
 template <typename R>
 int add_cg_loop(pdep_ctx* c, SysData& s, CgArgs<R> a, const R* b, int n, int max_iter, int* list,
                 cudaGraph_t g, cudaGraphNode_t after, cudaGraphNode_t* node, int* prologue) {
@@ -1346,14 +1346,7 @@ int capture_cg_graph(pdep_ctx* c, SysData& s, const CgArgs<R>& a, const R* b, in
   });
 }
 
-// Sternheimer PCG on (H - eps_v + sum_w sigma_w |w><w|) x = b for n RHS
-// (b, x: [n][ld]), each to ||r|| <= tol ||b|| or max_iter steps.  mask
-// (optional, device): RHS i takes part only if mask[i] != 0.  The loop runs on
-// the device: a CUDA graph with a while node whose body is one CG step and a
-// control kernel (no host round trip per step).  While the autotuner is
-// still timing launch shapes (or use_graph is 0) the same steps are launched
-// from a host loop that reads the control flag after each step.
-// H x inside the loop is the inner CG's (restored on every return)
+// H x inside the scope is the inner CG's (restored on every return)
 struct InnerFlag {
   bool& f;
   bool old;
@@ -1384,6 +1377,13 @@ int cg_setup(pdep_ctx* c, SysData& s, R* x, int n, double tol, CgScal* sc, const
   a.tolv = tolv;
   return PDEP_OK;
 }
+// Sternheimer PCG on (H - eps_v + sum_w sigma_w |w><w|) x = b for n RHS
+// (b, x: [n][ld]), each to ||r|| <= tol ||b|| or max_iter steps.  mask
+// (optional, device): RHS i takes part only if mask[i] != 0.  The loop runs on
+// the device: a CUDA graph with a while node whose body is one CG step or
+// four and its control (no host round trip per step).  While the autotuner is
+// still timing launch shapes (or use_graph is 0) the same steps are launched
+// from a host loop that reads the control flag after each step.
 template <typename R>
 int cg_loop(pdep_ctx* c, SysData& s, const R* b, R* x, int n, double tol, int max_iter,
             CgScal* sc, const double* mask, cudaStream_t st, const double* tolv) {

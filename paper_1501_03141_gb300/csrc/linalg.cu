@@ -473,7 +473,7 @@ cudaError_t eigh(int n, const double* M, long long ldm, double* W, double* V, lo
   int tpb = 64;
   const JacobiRound round_k = jacobi_round_for(n, &tpb);
   // column weights and squared norms: the tail of the scratch, unused until the
-  // sweeps are done (n >= 2; a single column needs neither)
+  // sweeps are done
   double *wt = wk.tmp, *norm = wk.tmp + n;
   // One sweep = nn - 1 dependent rounds; they are replayed from a CUDA graph
   // captured once per (size, buffers) to avoid nn - 1 stream launches.
