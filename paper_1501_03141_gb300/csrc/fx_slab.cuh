@@ -1,9 +1,10 @@
 // The FP64 slab pass on the tensor cores (fx_line.cuh): y- and z-lines of one
 // x-plane of one item per block.
 //
-// Bound by the issue of the digit conversions and the integer sums (43% of the
-// issue slots, ALU 47%, tensor pipe 20%, two blocks of six warps per SM on 48^3),
-// no longer by the FP64 pipe.  128 items on 48^3: 0.88 -> 0.27 ms; the mixed
+// Bound by the issue of the digit conversions and the integer sums and their
+// latency (seven digits with the density on 48^3: 43% of the issue slots, ALU 49%,
+// FP64 pipe 39%, tensor pipe 17%, two blocks of six warps per SM), no longer by the
+// FP64 pipe.  128 items on 48^3: 0.88 -> 0.27 ms; the mixed
 // refinement's passes (seven digits, before in double-float) over 4096 items,
 // there and back with the density and from the grid, 35.9 -> 25.3 ms.
 #pragma once
