@@ -21,12 +21,14 @@ def ctx():
         yield c
 
 
-def _check(ctx, val, vec, f):
-    out = ctx.screening_apply("chibar", val, vec, f)
+def _check(ctx, val, vec, f, kind="chibar"):
+    out = ctx.screening_apply(kind, val, vec, f)
     v, p, x = (np.asarray(a, dtype=np.longdouble) for a in (val, vec, f))
     g = v / (1 - v)
     ref = ((x @ p.T) * g) @ p
     size = ((np.abs(x) @ np.abs(p.T)) * np.abs(g)) @ np.abs(p)
+    if kind == "epsinv":
+        ref, size = ref + x, size + np.abs(x)
     # Per product, a kept digit sum errs by K 2^-56.8 A B (A, B: the largest
     # magnitudes) with sum |a b| >= 2^-5 A B, a recomputed one by K 2^-53 sum |a b|:
     # K 2^-51.8 either way; K = dim, then n_pdep
@@ -57,7 +59,8 @@ def test_opposite_along_the_plane_waves(ctx, n_pdep, n, decay):
 
 
 # one vector of each kind in a tile, zeros among them
-def test_mixed_tile(ctx):
+@pytest.mark.parametrize("kind", ["chibar", "epsinv"])
+def test_mixed_tile(ctx, kind):
     dim = ctx.sizes()["n_pdep_dim"]
     rng = np.random.default_rng(22)
     w = np.exp(-50.0 * np.arange(dim) / dim)
@@ -65,7 +68,7 @@ def test_mixed_tile(ctx):
     vec = np.concatenate([vec[0] * w, vec[1], vec[2] * w[::-1]])
     f = np.concatenate([f[0] * w, f[1], f[2] * w[::-1], f[3] * 0.0])
     vec[:, rng.integers(0, dim, dim // 3)] = 0.0
-    _check(ctx, -np.linspace(3.0, 0.01, 60), vec, f)
+    _check(ctx, -np.linspace(3.0, 0.01, 60), vec, f, kind)
 
 
 # the second product: vectors of falling size, eigenvalues that rise
